@@ -46,9 +46,14 @@ template <typename real, int D>
 int launch_permute(const PArrays<real, D>& src, const PArrays<real, D>& dst, const uint32_t* perm,
                    size_t np, cudaStream_t s);
 
-// dst[pid[i]] = src[i] for every particle array (back to the original order).
+// dst[pid[i]] = src[i] for every particle array (back to the original order;
+// dst's pid is not written).  scratch: unpermute_scratch_bytes(np) bytes
+// aligned to 32, or nullptr for the direct scatter.
 template <typename real, int D>
-int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, size_t np, cudaStream_t s);
+int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, size_t np, void* scratch,
+                     cudaStream_t s);
+template <typename real, int D>
+size_t unpermute_scratch_bytes(size_t np);
 
 // counts[key] += 1 for every sorted key (counts zeroed by the caller).
 int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_t s);

@@ -345,10 +345,94 @@ __global__ void __launch_bounds__(256) k_unpermute(PArrays<real, D> src, PArrays
   if (dst.pid) dst.pid[j] = j;
 }
 
+// The same in two passes through an array of records, one per particle in
+// the original order: (u, v, w) padded to whole 32-byte sectors.  The scatter
+// writes every record with full-sector stores, so that L2 evicts complete
+// sectors; the direct form above leaves seven (five in 2D) 4-byte pieces in
+// as many sectors, which DRAM reads and merges once the destination no
+// longer fits L2.  The second pass reads the records in order and writes
+// the arrays.  Bound: HBM (the payload read, the records written in random
+// 32-byte sectors and read back, the payload written).  16,777,216 particles
+// in 3D: 600 us in all against 4180 us direct.
 template <typename real, int D>
-int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, size_t np, cudaStream_t s) {
+struct __align__(32) ParticleRecord {
+  static constexpr int words = ((2 * D + 1) * (int)sizeof(real) + 31) / 32 * (32 / (int)sizeof(real));
+  real x[words];
+};
+
+__device__ __forceinline__ void st_sector(float* p, const float* x) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]),
+               "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7])
+               : "memory");
+}
+__device__ __forceinline__ void st_sector(double* p, const double* x) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(x[0]), "d"(x[1]), "d"(x[2]), "d"(x[3])
+               : "memory");
+}
+__device__ __forceinline__ void ld_sector(const float* p, float* x) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
+               : "l"(p));
+}
+__device__ __forceinline__ void ld_sector(const double* p, double* x) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3]) : "l"(p));
+}
+
+template <typename real, int D>
+__global__ void __launch_bounds__(256) k_unpermute_pack(PArrays<real, D> src, ParticleRecord<real, D>* rec, size_t np) {
+  constexpr int PER = 32 / (int)sizeof(real), W = ParticleRecord<real, D>::words;
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= np) return;
+  real x[W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) x[k] = (real)0;
+#pragma unroll
+  for (int m = 0; m < D; ++m) {
+    x[m] = src.u[m][i];
+    x[D + m] = src.v[m][i];
+  }
+  x[2 * D] = src.w[i];
+  real* d = rec[src.pid[i]].x;
+#pragma unroll
+  for (int k = 0; k < W; k += PER) st_sector(d + k, x + k);
+}
+
+template <typename real, int D>
+__global__ void __launch_bounds__(256) k_unpermute_unpack(const ParticleRecord<real, D>* rec, PArrays<real, D> dst,
+                                                          size_t np) {
+  constexpr int PER = 32 / (int)sizeof(real), W = ParticleRecord<real, D>::words;
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= np) return;
+  real x[W];
+#pragma unroll
+  for (int k = 0; k < W; k += PER) ld_sector(rec[i].x + k, x + k);
+#pragma unroll
+  for (int m = 0; m < D; ++m) {
+    dst.u[m][i] = x[m];
+    dst.v[m][i] = x[D + m];
+  }
+  dst.w[i] = x[2 * D];
+}
+
+template <typename real, int D>
+size_t unpermute_scratch_bytes(size_t np) {
+  return np * sizeof(ParticleRecord<real, D>);
+}
+
+template <typename real, int D>
+int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, size_t np, void* scratch,
+                     cudaStream_t s) {
   if (np == 0) return SG_OK;
-  k_unpermute<real, D><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(src, dst, np);
+  const unsigned blocks = (unsigned)((np + 255) / 256);
+  if (!scratch) {
+    k_unpermute<real, D><<<blocks, 256, 0, s>>>(src, dst, np);
+    SG_CHECK_LAUNCH();
+    return SG_OK;
+  }
+  auto* rec = static_cast<ParticleRecord<real, D>*>(scratch);
+  k_unpermute_pack<real, D><<<blocks, 256, 0, s>>>(src, rec, np);
+  SG_CHECK_LAUNCH();
+  k_unpermute_unpack<real, D><<<blocks, 256, 0, s>>>(rec, dst, np);
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
@@ -666,7 +750,9 @@ int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_
                                         unsigned long long*, unsigned*, cudaStream_t);                  \
   template int launch_permute<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, const uint32_t*, \
                                        size_t, cudaStream_t);                                             \
-  template int launch_unpermute<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, size_t, cudaStream_t); \
+  template int launch_unpermute<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, size_t, void*,        \
+                                         cudaStream_t);                                                          \
+  template size_t unpermute_scratch_bytes<real, D>(size_t);                                              \
   template int launch_tile_keys<real, D>(const PArrays<real, D>&, size_t, int, const SortFuse&, unsigned*,         \
                                          cudaStream_t);                                                            \
   template int launch_tile_scatter<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, const uint32_t*,     \
