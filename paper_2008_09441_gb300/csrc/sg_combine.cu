@@ -1,108 +1,252 @@
 // Signed combination of the component fields on the regular nodes:
 //   E_comb(x_j) = sum_i c_i (P_i E_i)(x_j)
 // (eq. sparse_filter's c_i and P_i of eq. restriction, applied to the
-// fields).  Two kernels share the scheme below: a warp per line for lines of
-// up to 1024 nodes (values in registers), a block per line beyond.  Block
-// per line: one block per regular row (a y line in 2D, a (y, z) line in
-// 3D).  Every (level l, coarse x index k) pair of the row is an independent
-// work item: it interpolates, in the transverse axes, every grid whose x level
-// is l at the row's coordinate and adds c_i times the result (grids in a fixed
-// order).  The x-prolongation is then applied once per level by Horner's
-// scheme (prolong level l to l+1, add level l+1, ...), exact for nested
-// node-centred grids.  Accumulation is float-float (FP32 path) or double
-// (FP64 path); the row is written as hi / lo planes and contributes its share
-// of sum |E_comb|^2 to the field energy.
+// fields).  P_i is a product of one prolongation per axis, so the sum is taken
+// axis by axis, the last axis first:
+//   3D: k_combine_planes prolongs along z.  The grids that share the levels
+//       (l_1, l_2) -- at most three, of coefficients +1, -2, +1 -- collapse
+//       into one "pair" array on 2^l_1 x 2^l_2 x N nodes.
+//   2D, and every z plane of a 3D run: k_combine_line interpolates each array
+//       (2D: the component grids, 3D: the plane's pairs) between the two
+//       coarse lines that bracket a regular line, and prolongs along x by
+//       Horner's scheme (prolong level l to l + 1, add the arrays of x level
+//       l + 1, ...), exact for nested node-centred grids.
+// Arrays per regular line drop from the 64 component grids with four
+// brackets each to 28 pairs with two (3D, n = 7, tau = 1).
+//
+// The fields are stored node-interleaved, from the solve's output to the
+// combined field, so one load brings all components of a node and one thread
+// carries them through the same operations two at a time (f32x2
+// instructions; 3D pads the third component with a zero fourth).
+#include <algorithm>
+#include <atomic>
+#include <type_traits>
+
 #include "sg_kernels.cuh"
 
 namespace sg {
 
-// ---------------------------------------------------------------- warp-per-line combination
+// ---------------------------------------------------------------- accumulators
 //
-// For lines of at most 1024 nodes: one warp per (regular line, field
-// component), the level-l partial sum held in registers (2^l / 32
-// consecutive values per lane once 2^l >= 32, one value on 2^l lanes
-// before).  Each Horner step prolongs in place (even nodes copy, odd nodes
-// average the two neighbours, the right neighbour's first value by shuffle)
-// and adds the transverse interpolation of the grids whose x level is the
-// new level, read with vector loads.  No block barriers.
+// Values of W components at one node, and their sums.
 //
-// FP32 path: the values are float pairs hi + lo carried without
+// FP32 path: the sums are float pairs hi + lo carried without
 // renormalisation: every hi addition is an error-free two_sum whose error
 // goes to lo, so lo collects the exact rounding errors of hi and the pair
 // stays accurate to ~2^-48 of the largest intermediate, whatever the
 // cancellation; one final two_sum renormalises before the hi / lo planes
 // are stored.  FP64 path: plain double.
-template <typename real>
-struct CAcc;
-template <>
-struct CAcc<float> {
-  using term = float;  // type of one grid's interpolated, scaled term
-  float hi, lo;
-  static __device__ __forceinline__ CAcc zero() { return {0.f, 0.f}; }
-  static __device__ __forceinline__ CAcc avg(const CAcc& a, const CAcc& b) {
-    const ff s = two_sum(a.hi, b.hi);
-    return {s.hi * 0.5f, (a.lo + b.lo + s.lo) * 0.5f};
-  }
-  static __device__ __forceinline__ CAcc add(const CAcc& a, const CAcc& b) {
-    const ff s = two_sum(a.hi, b.hi);
-    return {s.hi, a.lo + b.lo + s.lo};
-  }
-  static __device__ __forceinline__ CAcc first(float t) { return {t, 0.f}; }
-  static __device__ __forceinline__ CAcc add_term(const CAcc& a, float t) {
-    const ff s = two_sum(a.hi, t);
-    return {s.hi, a.lo + s.lo};
-  }
-  __device__ __forceinline__ CAcc shfl(int src) const {
-    return {__shfl_sync(0xffffffffu, hi, src), __shfl_sync(0xffffffffu, lo, src)};
-  }
-  __device__ __forceinline__ ff normalised() const { return two_sum(hi, lo); }
-};
-template <>
-struct CAcc<double> {
-  using term = double;
-  double v;
-  static __device__ __forceinline__ CAcc zero() { return {0.0}; }
-  static __device__ __forceinline__ CAcc avg(const CAcc& a, const CAcc& b) { return {(a.v + b.v) * 0.5}; }
-  static __device__ __forceinline__ CAcc add(const CAcc& a, const CAcc& b) { return {a.v + b.v}; }
-  static __device__ __forceinline__ CAcc first(double t) { return {t}; }
-  static __device__ __forceinline__ CAcc add_term(const CAcc& a, double t) { return {a.v + t}; }
-  __device__ __forceinline__ CAcc shfl(int src) const { return {__shfl_sync(0xffffffffu, v, src)}; }
-};
-
+//
 // FP32 fields combined with FP64 accumulation (sg_params.combine =
 // SG_COMBINE_FP64): each grid's term c_i w E_i is formed in double, which
 // is exact (c_i and the transverse weights w are dyadic, E_i a float), and
 // the alternating-sign sum and the Horner prolongation run in double.  The
-// result is split into hi + lo floats for the same output planes as the
-// float-float accumulator.  GB300 issues double arithmetic at a small
-// fraction of the float rate, so this variant is the slower one.
-struct CAccD {
-  using term = double;
-  double v;
-  static __device__ __forceinline__ CAccD zero() { return {0.0}; }
-  static __device__ __forceinline__ CAccD avg(const CAccD& a, const CAccD& b) { return {(a.v + b.v) * 0.5}; }
-  static __device__ __forceinline__ CAccD add(const CAccD& a, const CAccD& b) { return {a.v + b.v}; }
-  static __device__ __forceinline__ CAccD first(double t) { return {t}; }
-  static __device__ __forceinline__ CAccD add_term(const CAccD& a, double t) { return {a.v + t}; }
-  __device__ __forceinline__ CAccD shfl(int src) const { return {__shfl_sync(0xffffffffu, v, src)}; }
-  __device__ __forceinline__ ff normalised() const {
-    const float hi = (float)v;
-    return {hi, (float)(v - (double)hi)};
+// result is split into hi + lo floats for the same output planes.  GB300
+// issues double arithmetic at a small fraction of the float rate, so this
+// variant is the slower one.
+
+// Two floats in one 64-bit register pair, operated on by one instruction.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_pack(float x, float y) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(f2 a, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a)); }
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) { return f2_fma(b, f2_pack(-1.f, -1.f), a); }  // one rounding
+__device__ __forceinline__ f2 f2_two_sum(f2 a, f2 b, f2& err) {
+  const f2 s = f2_add(a, b);
+  const f2 bb = f2_sub(s, a);
+  err = f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb));
+  return s;
+}
+
+// One node's W values: T float in pairs (W even), else plain.
+template <typename T, int W>
+struct Term {
+  static constexpr bool packed = sizeof(T) == 4 && W % 2 == 0;
+  static constexpr int P = packed ? W / 2 : W;
+  using E = typename std::conditional<packed, f2, T>::type;
+  E v[P];
+  static __device__ __forceinline__ E splat(T x) {
+    if constexpr (packed) return f2_pack(x, x);
+    else return x;
+  }
+  // w0 * a + w1 * b, the second product fused (weights are exact)
+  static __device__ __forceinline__ Term lerp(T w0, const Term& a, T w1, const Term& b) {
+    Term r;
+    const E s0 = splat(w0), s1 = splat(w1);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      if constexpr (packed) r.v[p] = f2_fma(s1, b.v[p], f2_mul(s0, a.v[p]));
+      else r.v[p] = fma(s1, b.v[p], s0 * a.v[p]);
+    }
+    return r;
+  }
+  static __device__ __forceinline__ Term mid(const Term& a, const Term& b) {  // (a + b) / 2
+    Term r;
+    const E h = splat((T)0.5);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      if constexpr (packed) r.v[p] = f2_mul(h, f2_add(a.v[p], b.v[p]));
+      else r.v[p] = h * (a.v[p] + b.v[p]);
+    }
+    return r;
+  }
+  static __device__ __forceinline__ Term select(bool c, const Term& a, const Term& b) {
+    Term r;
+#pragma unroll
+    for (int p = 0; p < P; ++p) r.v[p] = c ? a.v[p] : b.v[p];
+    return r;
   }
 };
 
-template <typename AC>
-constexpr bool kFp64Acc = false;
-template <>
-constexpr bool kFp64Acc<CAccD> = true;
+// Loads node i of an array stored with DP values per node.
+template <typename T, int W, int DP, typename GT>
+__device__ __forceinline__ Term<T, W> load_node(const GT* __restrict__ g, int i) {
+  Term<T, W> t;
+  const GT* p = g + (size_t)(unsigned)i * DP;
+  if constexpr (Term<T, W>::packed) {
+    if constexpr (W == 2) {
+      t.v[0] = __ldg(reinterpret_cast<const f2*>(p));
+    } else {
+      const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2*>(p));
+      t.v[0] = q.x;
+      t.v[1] = q.y;
+    }
+  } else {
+#pragma unroll
+    for (int w = 0; w < W; ++w) t.v[w] = (T)__ldg(p + w);
+  }
+  return t;
+}
 
-// Transverse interpolation weights and coarse-row offsets of one grid at
-// regular line (y, z): the 2^(d-1) coarse x-lines that bracket the line,
-// each weight times the grid's coefficient (dyadic products: exact).
-template <typename real, int D>
-struct RowTerm {
-  int off[1 << (D - 1)];
-  real w[1 << (D - 1)];
+template <typename T, int W>
+struct Sum {  // FP64 accumulation
+  using Tm = Term<T, W>;
+  T v[W];
+  static __device__ __forceinline__ Sum zero() {
+    Sum r;
+#pragma unroll
+    for (int p = 0; p < W; ++p) r.v[p] = (T)0;
+    return r;
+  }
+  static __device__ __forceinline__ Sum avg(const Sum& a, const Sum& b) {
+    Sum r;
+#pragma unroll
+    for (int p = 0; p < W; ++p) r.v[p] = (a.v[p] + b.v[p]) * (T)0.5;
+    return r;
+  }
+  static __device__ __forceinline__ Sum add(const Sum& a, const Sum& b) {
+    Sum r;
+#pragma unroll
+    for (int p = 0; p < W; ++p) r.v[p] = a.v[p] + b.v[p];
+    return r;
+  }
+  __device__ __forceinline__ void add_term(const Tm& t) {
+#pragma unroll
+    for (int p = 0; p < W; ++p) v[p] += t.v[p];
+  }
+  __device__ __forceinline__ void value(T* x) const {
+#pragma unroll
+    for (int p = 0; p < W; ++p) x[p] = v[p];
+  }
+};
+template <int W>
+struct __align__(16) Sum<float, W> {  // float pairs
+  using Tm = Term<float, W>;
+  static constexpr int P = Tm::P;
+  using E = typename Tm::E;
+  E hi[P], lo[P];
+  static __device__ __forceinline__ E two_sum_e(E a, E b, E& err) {
+    if constexpr (Tm::packed) {
+      return f2_two_sum(a, b, err);
+    } else {
+      const ff s = two_sum(a, b);
+      err = s.lo;
+      return s.hi;
+    }
+  }
+  static __device__ __forceinline__ E add_e(E a, E b) {
+    if constexpr (Tm::packed) return f2_add(a, b);
+    else return a + b;
+  }
+  static __device__ __forceinline__ Sum zero() {
+    Sum r;
+#pragma unroll
+    for (int p = 0; p < P; ++p) r.hi[p] = r.lo[p] = Tm::splat(0.f);
+    return r;
+  }
+  static __device__ __forceinline__ Sum avg(const Sum& a, const Sum& b) {
+    Sum r;
+    const E h = Tm::splat(0.5f);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      E err;
+      const E s = two_sum_e(a.hi[p], b.hi[p], err);
+      const E l = add_e(add_e(a.lo[p], b.lo[p]), err);
+      if constexpr (Tm::packed) {
+        r.hi[p] = f2_mul(s, h);
+        r.lo[p] = f2_mul(l, h);
+      } else {
+        r.hi[p] = s * h;
+        r.lo[p] = l * h;
+      }
+    }
+    return r;
+  }
+  static __device__ __forceinline__ Sum add(const Sum& a, const Sum& b) {
+    Sum r;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      E err;
+      r.hi[p] = two_sum_e(a.hi[p], b.hi[p], err);
+      r.lo[p] = add_e(add_e(a.lo[p], b.lo[p]), err);
+    }
+    return r;
+  }
+  __device__ __forceinline__ void add_term(const Tm& t) {
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      E err;
+      hi[p] = two_sum_e(hi[p], t.v[p], err);
+      lo[p] = add_e(lo[p], err);
+    }
+  }
+  // the normalised hi and lo parts, by component
+  __device__ __forceinline__ void split(float* h, float* l) const {
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      E err;
+      const E s = two_sum_e(hi[p], lo[p], err);
+      if constexpr (Tm::packed) {
+        f2_unpack(s, h[2 * p], h[2 * p + 1]);
+        f2_unpack(err, l[2 * p], l[2 * p + 1]);
+      } else {
+        h[p] = s;
+        l[p] = err;
+      }
+    }
+  }
+  __device__ __forceinline__ void value(float* x) const {
+    float l[W];
+    split(x, l);
+  }
 };
 
 // The two level-lev nodes that bracket regular node y along one axis and
@@ -125,86 +269,155 @@ __device__ __forceinline__ void bracket(int y, int n, int lev, int& k0, int& k1,
   k1 = (k0 + 1) & (nl - 1);
 }
 
-template <typename real, int D, bool CELL>
-__device__ __forceinline__ RowTerm<real, D> row_term(const GridDesc& g, int n, int y, int z) {
-  RowTerm<real, D> t;
-  const int nx = 1 << g.l[0];
-  const int ny = 1 << g.l[1];
-  int ky0, ky1;
-  real fy;
-  bracket<real, CELL>(y, n, g.l[1], ky0, ky1, fy);
-  const real c = (real)g.coeff;
-  if (D == 2) {
-    t.off[0] = g.offset + ky0 * nx;
-    t.off[(1 << (D - 1)) - 1] = g.offset + ky1 * nx;
-    t.w[0] = c * ((real)1 - fy);
-    t.w[(1 << (D - 1)) - 1] = c * fy;
-  } else {
-    int kz0, kz1;
-    real fz;
-    bracket<real, CELL>(z, n, g.l[D - 1], kz0, kz1, fz);
-    constexpr int R = 1 << (D - 1);
-    t.off[0] = g.offset + (kz0 * ny + ky0) * nx;
-    t.off[1 % R] = g.offset + (kz0 * ny + ky1) * nx;
-    t.off[2 % R] = g.offset + (kz1 * ny + ky0) * nx;
-    t.off[3 % R] = g.offset + (kz1 * ny + ky1) * nx;
-    t.w[0] = c * (((real)1 - fy) * ((real)1 - fz));
-    t.w[1 % R] = c * (fy * ((real)1 - fz));
-    t.w[2 % R] = c * (((real)1 - fy) * fz);
-    t.w[3 % R] = c * (fy * fz);
+// Values per node of an array of NC components: 2D fields 2, 3D fields 4
+// (one pad), a density 1.
+template <int NC>
+constexpr int node_stride() { return NC == 1 ? 1 : NC == 2 ? 2 : 4; }
+// Components a thread of the line kernel carries: floats all of them, in
+// whole pairs; doubles one (their latency is long, more threads hide it).
+template <typename T, int NC>
+constexpr int carried() { return sizeof(T) == 4 ? node_stride<NC>() : 1; }
+
+// ---------------------------------------------------------------- 3D: prolongation along z
+//
+// out[z][off_p + e] = sum over the pair's grids of c_i times the linear
+// interpolation along z of in-plane node e.  The sum runs in the accumulator
+// and is rounded once to the type of the grids' terms, as a grid's own
+// interpolated term is in k_combine_line.  One thread per in-plane node
+// walks PL_Z planes; loads are consecutive in e.  Bound: latency (9400
+// cycles, about 5 us, at n = 7, tau = 1: 394 K nodes from 64 grids).
+constexpr int PL_Z = 4;
+constexpr int PL_LEVELS = 9;  // 3D levels 0..8
+template <typename T>
+struct __align__(16) PlaneBracket {
+  int k0, k1;
+  T w0, w1;
+};
+template <typename real, typename T, int NC, bool CELL>
+__global__ void __launch_bounds__(256) k_combine_planes(const PlanePair* __restrict__ pairs, int npairs,
+                                                        const real* __restrict__ E, int S2, int n, int z0, int nz,
+                                                        T* __restrict__ out) {
+  constexpr int DP = node_stride<NC>(), W = sizeof(T) == 4 ? DP : NC;
+  __shared__ PlanePair sp[CB_MAX_GRIDS];
+  __shared__ PlaneBracket<T> sb[PL_LEVELS][PL_Z];
+  pdl_trigger();
+  const int zb = blockIdx.y * PL_Z;
+  {
+    const int* src = reinterpret_cast<const int*>(pairs);
+    int* dst = reinterpret_cast<int*>(sp);
+    for (int i = threadIdx.x; i < npairs * (int)(sizeof(PlanePair) / 4); i += blockDim.x) dst[i] = src[i];
+    if (threadIdx.x < (n + 1) * PL_Z) {
+      const int l = threadIdx.x / PL_Z, z = threadIdx.x % PL_Z;
+      PlaneBracket<T> t;
+      bracket<T, CELL>(z0 + zb + z, n, l, t.k0, t.k1, t.w1);
+      t.w0 = (T)1 - t.w1;
+      sb[l][z] = t;
+    }
   }
-  return t;
+  __syncthreads();
+  pdl_wait();  // the solve's fields
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= S2) return;
+  int lo = 0, hi = npairs;  // the last pair with off <= e
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (sp[mid].off <= e) lo = mid;
+    else hi = mid;
+  }
+  const PlanePair P = sp[lo];
+  const int le = e - P.off;
+  const int x = le & ((1 << P.lx) - 1);
+  const int at = e - x + line_pos(x, P.lx, n);
+#pragma unroll
+  for (int z = 0; z < PL_Z; ++z) {
+    if (zb + z >= nz) break;
+    Sum<T, W> acc = Sum<T, W>::zero();
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      if (q < P.ng) {
+        const PlaneBracket<T> t = sb[P.lz[q]][z];
+        const T c = (T)P.coeff[q];
+        const int g = P.goff[q] + le;
+        acc.add_term(Term<T, W>::lerp(c * t.w0, load_node<T, W, DP>(E, g + (t.k0 << P.logs)), c * t.w1,
+                                      load_node<T, W, DP>(E, g + (t.k1 << P.logs))));
+      }
+    }
+    T xv[W];
+    acc.value(xv);
+    T* d = out + ((size_t)(zb + z) * S2 + at) * DP;
+    if constexpr (sizeof(T) == 4 && W == 4) {
+      *reinterpret_cast<float4*>(d) = make_float4(xv[0], xv[1], xv[2], xv[3]);
+    } else {
+#pragma unroll
+      for (int w = 0; w < W; ++w) d[w] = xv[w];
+    }
+  }
 }
 
-// Adds, to the K consecutive values T[0..K) at x index x0.. (K and x0
-// multiples of 4), c_i times the transverse interpolation of every grid of
-// x level `level`; the grids' row terms come from this warp's shared-memory
-// table.  Grid by grid, all of a grid's loads first (one latency per grid).
-template <typename real, int D, int K, typename AC>
-__device__ __forceinline__ void add_level_terms(AC* T, const RowTerm<real, D>* rt_tab, const int* lstart,
-                                                int level, const real* __restrict__ Em, int x0) {
-  using TT = typename AC::term;
-  constexpr int R = 1 << (D - 1);
-  for (int gi = lstart[level]; gi < lstart[level + 1]; ++gi) {
-    const RowTerm<real, D> rt = rt_tab[gi];
-    TT t[K];
+// ---------------------------------------------------------------- lines
+//
+// Levels up to n - log2 K: the block's threads hold one node each of every
+// line in shared memory (all arrays that enter at any of these levels are
+// interpolated at once, then the prolongation runs level by level), so no
+// value is computed twice and every load is consecutive.  Above, a thread
+// computes K consecutive nodes: it needs 2 nodes of the shared level, then
+// 3, 5, ..., K + 1, and prolongs that cone by itself, which spares the
+// barriers of the widest levels for a few values computed twice.  Bound:
+// 3D, the L1 data pipe (53% busy) and latency at 31% occupancy; 2D, the
+// latency of the block's phases (36% of issue slots).  With profiling events,
+// before (one warp per line, all grids) -> now, planes included: 3D n = 7
+// 151 -> 59 us, tau = 2 137 -> 69, n = 6 cell-centred 64 -> 25; 2D n = 11
+// 134 -> 51, n = 10 27 -> 20.5, n = 8 14.3 -> 12.3 us.
+
+// Transverse interpolation of one array at regular line y: the two coarse
+// lines that bracket it, each weight times the coefficient (dyadic: exact).
+template <typename T>
+struct __align__(16) RowTerm {
+  int off[2];
+  T w[2];
+};
+
+template <typename T, int W, int DP, typename GT>
+__device__ __forceinline__ Term<T, W> row_node(const GT* __restrict__ G, const RowTerm<T>& rt, int x) {
+  return Term<T, W>::lerp(rt.w[0], load_node<T, W, DP>(G, rt.off[0] + x), rt.w[1],
+                          load_node<T, W, DP>(G, rt.off[1] + x));
+}
+
+// R consecutive nodes of an array of x level l at line y, from node a (a
+// multiple of R), X of them past the run's end, periodically (X = 1).  PERM:
+// the array is stored in line_pos order.
+template <typename T, int W, int DP, int R, int X, bool PERM, typename GT>
+__device__ __forceinline__ void row_run(const GT* __restrict__ G, const RowTerm<T>& rt, int a, int l, Term<T, W>* t) {
+  constexpr int LR = R == 4 ? 2 : R == 2 ? 1 : 0;
+  const int mask = (1 << l) - 1;
+  if constexpr (!PERM && W == 1 && sizeof(GT) == 4 && R > 1) {  // a plain density: vector loads
+    GT x[2][R];
 #pragma unroll
-    for (int k = 0; k < K; k += 4) {
-      const V4<real> a = ld4(Em + rt.off[0] + x0 + k);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) t[k + q] = (TT)rt.w[0] * (TT)a.x[q];
-    }
-#pragma unroll
-    for (int r = 1; r < R; ++r) {
-#pragma unroll
-      for (int k = 0; k < K; k += 4) {
-        const V4<real> a = ld4(Em + rt.off[r] + x0 + k);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) t[k + q] = fma((TT)rt.w[r], (TT)a.x[q], t[k + q]);
+    for (int k = 0; k < 2; ++k) {
+      const GT* p = G + rt.off[k] + a;
+      if constexpr (R == 4) {
+        const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+        x[k][0] = q.x;
+        x[k][1] = q.y;
+        x[k][2] = q.z;
+        x[k][3] = q.w;
+      } else {
+        const float2 q = __ldg(reinterpret_cast<const float2*>(p));
+        x[k][0] = q.x;
+        x[k][1] = q.y;
       }
     }
 #pragma unroll
-    for (int k = 0; k < K; ++k) T[k] = AC::add_term(T[k], t[k]);
-  }
-}
-
-// The same at one x index (lines with fewer than 4 values per lane).
-template <typename real, int D, typename AC>
-__device__ __forceinline__ AC level_term1(const RowTerm<real, D>* rt_tab, const int* lstart, int level,
-                                          const real* __restrict__ Em, int x) {
-  using TT = typename AC::term;
-  constexpr int R = 1 << (D - 1);
-  AC acc = AC::zero();
-  bool first = true;
-  for (int gi = lstart[level]; gi < lstart[level + 1]; ++gi) {
-    const RowTerm<real, D> rt = rt_tab[gi];
-    TT t = (TT)rt.w[0] * (TT)Em[rt.off[0] + x];
+    for (int j = 0; j < R; ++j) t[j].v[0] = fma(rt.w[1], (T)x[1][j], rt.w[0] * (T)x[0][j]);
+  } else {
 #pragma unroll
-    for (int r = 1; r < R; ++r) t = fma((TT)rt.w[r], (TT)Em[rt.off[r] + x], t);
-    acc = first ? AC::first(t) : AC::add_term(acc, t);
-    first = false;
+    for (int j = 0; j < R; ++j)
+      t[j] = row_node<T, W, DP>(G, rt, PERM ? (j << (l - LR)) + (a >> LR) : a + j);
   }
-  return acc;
+  if constexpr (X) {
+    const int b = (a + R) & mask;
+    t[R] = row_node<T, W, DP>(G, rt, PERM ? b >> LR : b);
+  }
 }
 
 // Cell-centred grids.  Linear interpolation through the centres of a
@@ -212,97 +425,78 @@ __device__ __forceinline__ AC level_term1(const RowTerm<real, D>* rt_tab, const 
 // whose odd nodes are the centres (g[2k+1] = E[k]) and whose even nodes are
 // the midpoints (g[2k] = (E[k-1] + E[k]) / 2); the regular centres are the
 // midpoints of the level-n nodes.  So the same Horner scheme runs with each
-// grid entering one level higher as g, and the regular-centre values are
-// (T[j] + T[j+1]) / 2 of its level-n result, plus the grids of x level n
+// array entering one level higher as g, and the regular-centre values are
+// (T[j] + T[j+1]) / 2 of its level-n result, plus the arrays of x level n
 // at their own centres.
 
-// g of the grids of x level `level - 1` at Horner level `level`, index t.
-template <typename real, int D, typename AC>
-__device__ __forceinline__ AC cell_term1(const RowTerm<real, D>* rt_tab, const int* lstart, int level,
-                                         const real* __restrict__ Em, int t) {
-  if (level < 1) return AC::zero();
-  const int lc = level - 1, nc = 1 << lc;
-  if (t & 1) return level_term1<real, D, AC>(rt_tab, lstart, lc, Em, t >> 1);
-  return AC::avg(level_term1<real, D, AC>(rt_tab, lstart, lc, Em, ((t >> 1) - 1) & (nc - 1)),
-                 level_term1<real, D, AC>(rt_tab, lstart, lc, Em, t >> 1));
-}
-
-// Adds g of every grid of x level `level - 1` to the K >= 2 consecutive
-// values T[0..K) at Horner-level index x0.. (x0 a multiple of K): the
-// grid's K/2 centre values from x0/2 on (vector loads once K/2 >= 4) and
-// the one before, periodically.
-template <typename real, int D, int K, typename AC>
-__device__ __forceinline__ void add_level_terms_cell(AC* T, const RowTerm<real, D>* rt_tab,
-                                                     const int* lstart, int level, const real* __restrict__ Em,
-                                                     int x0) {
-  using TT = typename AC::term;
-  constexpr int R = 1 << (D - 1);
-  constexpr int H = K / 2;
-  const int lc = level - 1, nc = 1 << lc;
-  const int c0 = x0 >> 1, cm = (c0 - 1) & (nc - 1);
-  for (int gi = lstart[lc]; gi < lstart[lc + 1]; ++gi) {
-    const RowTerm<real, D> rt = rt_tab[gi];
-    TT t[H + 1];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const real* row = Em + rt.off[r];
-      const TT w = (TT)rt.w[r];
-      const TT prev = (TT)row[cm];
-      t[0] = r == 0 ? w * prev : fma(w, prev, t[0]);
-      if constexpr (H >= 4) {
-#pragma unroll
-        for (int k = 0; k < H; k += 4) {
-          const V4<real> a = ld4(row + c0 + k);
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            t[1 + k + q] = r == 0 ? w * (TT)a.x[q] : fma(w, (TT)a.x[q], t[1 + k + q]);
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < H; ++k)
-          t[1 + k] = r == 0 ? w * (TT)row[c0 + k] : fma(w, (TT)row[c0 + k], t[1 + k]);
-      }
+// Sum, at node x of `level`, of the arrays that enter there.
+template <typename T, int W, int DP, bool CELL, typename GT>
+__device__ __forceinline__ Sum<T, W> entering(const GT* __restrict__ G, const RowTerm<T>* tab, const int* start,
+                                              int level, int x) {
+  Sum<T, W> acc = Sum<T, W>::zero();
+  const int l = CELL ? level - 1 : level;
+  if (CELL && l < 0) return acc;
+  const int mask = (1 << l) - 1;
+  const int i1 = CELL ? x >> 1 : x;
+  const int end = start[l + 1];
+#pragma unroll 2
+  for (int gi = start[l]; gi < end; ++gi) {
+    const RowTerm<T> rt = tab[gi];
+    Term<T, W> t = row_node<T, W, DP>(G, rt, i1);
+    if constexpr (CELL) {  // an even node: the midpoint of two centres
+      const int i0 = (x & 1) ? i1 : (i1 - 1) & mask;
+      const Term<T, W> t0 = row_node<T, W, DP>(G, rt, i0);
+      t = Term<T, W>::select(x & 1, t, Term<T, W>::mid(t0, t));
     }
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-      T[2 * j + 1] = AC::add_term(T[2 * j + 1], t[j + 1]);
-      T[2 * j] = AC::add_term(T[2 * j], (TT)0.5 * (t[j] + t[j + 1]));
-    }
+    acc.add_term(t);
   }
+  return acc;
 }
 
-// One Horner step in the register phase: Vc values per lane -> 2 Vc, then
-// add the new level's terms; recurse up to level n (2 Vc <= VMAX).
-template <typename real, int D, int Vc, int VMAX, bool CELL, typename AC>
-struct CombLevels {
-  static __device__ __forceinline__ void run(AC* T, int& level, int n, int lane,
-                                             const RowTerm<real, D>* rt_tab, const int* lstart,
-                                             const real* __restrict__ Em) {
-    if constexpr (2 * Vc <= VMAX) {
-      const AC right = T[0].shfl((lane + 1) & 31);
+// Nodes a .. a + C of `level` (a a multiple of C) -> a' .. a' + 2C of the next
+// one, with its arrays added; up to CB_RUN nodes of level n.  The node past
+// the thread's last one is dropped at level n, unless the cell-centred
+// midpoints need it.
+template <typename T, int W, int DP, int C, bool CELL, bool PERM, typename GT>
+__device__ __forceinline__ void expand(Sum<T, W>* v, const GT* __restrict__ G, const RowTerm<T>* tab,
+                                       const int* start, int level, int j0, int n) {
+  using S = Sum<T, W>;
+  if constexpr (C < CB_RUN) {
+    constexpr int C2 = 2 * C, X = (C2 < CB_RUN || CELL) ? 1 : 0;
+    v[C2] = v[C];
 #pragma unroll
-      for (int i = Vc - 1; i >= 0; --i) {  // in place, high to low
-        const AC nxt = (i == Vc - 1) ? right : T[i + 1];
-        T[2 * i + 1] = AC::avg(T[i], nxt);
-        T[2 * i] = T[i];
-      }
-      ++level;
-      constexpr int K = 2 * Vc;
+    for (int i = C - 1; i >= 0; --i) {  // in place, high to low
+      v[2 * i + 1] = S::avg(v[i], v[i + 1 < C ? 2 * (i + 1) : C2]);
+      v[2 * i] = v[i];
+    }
+    ++level;
+    const int l = CELL ? level - 1 : level;
+    const int mask = (1 << l) - 1;
+    const int a = (j0 >> (n - level)) >> (CELL ? 1 : 0);
+    const int end = start[l + 1];
+    for (int gi = start[l]; gi < end; ++gi) {
+      const RowTerm<T> rt = tab[gi];
       if constexpr (CELL) {
-        add_level_terms_cell<real, D, K, AC>(T, rt_tab, lstart, level, Em, lane * K);
-      } else if constexpr (K >= 4) {
-        add_level_terms<real, D, K, AC>(T, rt_tab, lstart, level, Em, lane * K);
-      } else {
+        Term<T, W> t[C + 2];
+        const int b = (a - 1) & mask;
+        t[0] = row_node<T, W, DP>(G, rt, PERM && C == 2 ? ((b & 1) << (l - 1)) + (b >> 1) : b);
+        row_run<T, W, DP, C, 1, PERM && C == 2>(G, rt, a, l, t + 1);
 #pragma unroll
-        for (int k = 0; k < K; ++k)
-          T[k] = AC::add(T[k], level_term1<real, D, AC>(rt_tab, lstart, level, Em, lane * K + k));
+        for (int j = 0; j <= C; ++j) v[2 * j].add_term(Term<T, W>::mid(t[j], t[j + 1]));
+#pragma unroll
+        for (int j = 0; j < C; ++j) v[2 * j + 1].add_term(t[j + 1]);
+      } else {
+        Term<T, W> t[C2 + X];
+        row_run<T, W, DP, C2, X, PERM>(G, rt, a, l, t);
+#pragma unroll
+        for (int j = 0; j < C2 + X; ++j) v[j].add_term(t[j]);
       }
-      if (level < n) CombLevels<real, D, 2 * Vc, VMAX, CELL, AC>::run(T, level, n, lane, rt_tab, lstart, Em);
     }
+    expand<T, W, DP, C2, CELL, PERM>(v, G, tab, start, level, j0, n);
   }
-};
+}
 
-// Shared by both combination kernels: the last block to finish reduces the
+// The last block to finish reduces the
 // energy partials (and the push's kinetic-energy partials) in FP64, in a
 // fixed order, so the step needs no separate bookkeeping launch.
 __device__ __forceinline__ void combine_finalize(const double* partials, int n_part, const CombineFinal& fin,
@@ -333,425 +527,258 @@ __device__ __forceinline__ void combine_finalize(const double* partials, int n_p
   }
 }
 
-// Lines per block of the warp-per-line kernel (one warp per line and
-// component) and the bytes of its row-term tables (one per line).
-template <int D>
-constexpr int combine_rows_per_block() { return 4; }  // 3D: 2 rows measured 16% slower
-template <typename real, int D, int NC>
-__host__ __device__ constexpr size_t combine_table_bytes(int ngl) {
-  return ((size_t)combine_rows_per_block<D>() * ngl * sizeof(RowTerm<real, D>) + 15) / 16 * 16;
+// Sum of one value per warp (the same in all its lanes), valid in thread 0.
+__device__ __forceinline__ double block_sum_warps(double w, double* sh) {
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = w;
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x == 0)
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r += sh[k];
+  return r;
 }
-// Stride of the output between nodes: NC = D fields are stored
-// node-interleaved (ec_stride), a single density plainly.
-template <int D, int NC>
-constexpr int combine_out_stride() { return NC == 1 ? 1 : ec_stride<D>(); }
 
-template <typename real, int D, int V, int NC, bool CELL, typename AC>
-__global__ void __launch_bounds__(32 * combine_rows_per_block<D>() * NC) k_combine_warp(const GridDesc* __restrict__ grids, LevelLists ll, int lmin,
-                                                      const real* __restrict__ E, size_t S, int n,
-                                                      real* __restrict__ Ehi, float* __restrict__ Elo,
-                                                      double* __restrict__ partials, const CombineFinal fin) {
+constexpr int CL_THREADS = 256;
+
+// One block: `lpb` consecutive lines, N / CB_RUN threads per line and group of
+// carried components.  zstride: values between the planes of G (2D: one
+// plane).  row0: first line of the launch.
+template <typename real, typename GT, typename T, int NC, bool CELL, bool PERM>
+__global__ void __launch_bounds__(CL_THREADS, sizeof(T) == 8 ? 2 : NC == 3 ? 3 : 4)
+    k_combine_line(const LineGrid* __restrict__ lg, const LevelStarts ls, int lmin, const GT* __restrict__ G,
+                   size_t zstride, int n, int lpb, int row0, size_t nd, real* __restrict__ Ehi,
+                   float* __restrict__ Elo, double* __restrict__ partials, int n_part, const CombineFinal fin) {
+  constexpr int K = CB_RUN, LK = 2;
+  constexpr int DP = node_stride<NC>(), W = carried<T, NC>();
+  constexpr int MG = W >= NC ? 1 : NC;  // groups of components
+  constexpr int WO = W < NC ? W : NC;   // components a thread writes
+  using S = Sum<T, W>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
+  __shared__ int start[18];
   const int N = 1 << n;
-  const int rows = D == 2 ? N : N * N;
-  const size_t ND = (size_t)rows * N;
-  const int wib = threadIdx.x >> 5;
-  const int task = blockIdx.x * (blockDim.x >> 5) + wib;  // (row, component)
-  const int lane = threadIdx.x & 31;
-  const int m = task % NC, row = task / NC;
-  const int y = row & (N - 1);
-  const int z = D == 3 ? (row >> n) : 0;
-  const real* Em = E + (size_t)m * S;
-  __shared__ int s_start[18];
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < 18; ++i) s_start[i] = ll.start[i];  // constant indices: no local copy
-  }
-  const int ngl = ll.start[17];
-  constexpr int RPB = combine_rows_per_block<D>();  // the block's lines: all NC components of each
-  constexpr int DP = combine_out_stride<D, NC>();
-  // one row-term table per line, shared by the line's NC component warps
-  RowTerm<real, D>* rt_all = reinterpret_cast<RowTerm<real, D>*>(smem_raw);
-  RowTerm<real, D>* rt_tab = rt_all + (size_t)(wib / NC) * ngl;
-  // [RPB][N][DP] with one padding word after every V nodes (a lane's run), so
-  // that the lanes' stores of one step fall in distinct banks
-  real* stage = reinterpret_cast<real*>(smem_raw + combine_table_bytes<real, D, NC>(ngl));
-  const int row0 = blockIdx.x * RPB;
+  const int ipl = N >> LK;  // threads per line and group
+  const int ngl = ls.start[17];
+  RowTerm<T>* tab = reinterpret_cast<RowTerm<T>*>(smem_raw);  // [lpb][ngl]
+  // node x of level l of line and group q at lat[q * 2 ipl + 2^l + x], q = line * MG + group
+  S* lat = reinterpret_cast<S*>(tab + (size_t)lpb * ngl);
+  const int brow = row0 + blockIdx.x * lpb;  // first line of the block
   pdl_trigger();
-  for (int e = threadIdx.x; e < RPB * ngl; e += blockDim.x) {
-    const int r = e / ngl, gi = e - r * ngl;
-    const int rr = row0 + r;  // the block's line r
-    rt_all[e] = row_term<real, D, CELL>(grids[ll.grid[gi]], n, rr & (N - 1), D == 3 ? (rr >> n) : 0);
-  }
-  __syncthreads();
-  pdl_wait();  // the solve's fields
-  real energy = (real)0;
-  double energy_d = 0.0;  // FP64 accumulation: the squares of the double results
-  if (row < rows) {
-    AC T[V];
-    // coarse phase: one value on 2^level lanes, up to 32 values.  The terms
-    // of every coarse level, pairs (l, x) with l in [level, ltop] and
-    // x < 2^l, numbered p = 2^l - 2^level + x (at most 62), are computed
-    // first, two pairs per lane (p = lane and lane + 32) so that every lane
-    // works, and are handed to lane x of level l by shuffles.  Each term sums
-    // its level's grids in the same order as before.  Cell-centred grids
-    // enter one level higher.
-    int level = min(CELL ? lmin + 1 : lmin, min(n, 5));
-    const int ltop = min(n, 5);
-    const int p0 = 1 << level;
-    const int npairs = (2 << ltop) - p0;
-    AC pv[2];
-#pragma unroll
-    for (int sl = 0; sl < 2; ++sl) {
-      const int p = lane + 32 * sl;
-      if (p < npairs) {
-        const int l = 31 - __clz(p + p0);
-        const int x = p + p0 - (1 << l);
-        pv[sl] = CELL ? cell_term1<real, D, AC>(rt_tab, s_start, l, Em, x)
-                      : level_term1<real, D, AC>(rt_tab, s_start, l, Em, x);
-      } else {
-        pv[sl] = AC::zero();
-      }
-    }
-    // the level-l term of this lane's x (zero beyond 2^l); every lane shuffles
-    auto coarse = [&](int l) {
-      const int p = (1 << l) - p0 + lane;
-      const AC a = pv[0].shfl(p & 31), b = pv[1].shfl(p & 31);
-      return lane < (1 << l) ? ((p >> 5) ? b : a) : AC::zero();
-    };
-    T[0] = coarse(level);
-#pragma unroll
-    for (int j = 1; j < 6; ++j) {
-      if (level < ltop) {
-        const int h = 1 << level;
-        const int k = lane >> 1;
-        const AC a = T[0].shfl(k & (h - 1));
-        const AC b = T[0].shfl((k + 1) & (h - 1));
-        T[0] = (lane & 1) ? AC::avg(a, b) : a;
-        ++level;
-        const AC c = coarse(level);
-        if (lane < (1 << level)) T[0] = AC::add(T[0], c);
-      }
-    }
-    // register phase: 2^level / 32 consecutive values per lane
-    if (level < n) CombLevels<real, D, 1, V, CELL, AC>::run(T, level, n, lane, rt_tab, s_start, Em);
-    if constexpr (CELL) {  // to the regular centres, then the grids of x level n
-      if (N >= 32) {
-        const AC right = T[0].shfl((lane + 1) & 31);
-#pragma unroll
-        for (int k = 0; k < V; ++k) T[k] = AC::avg(T[k], k == V - 1 ? right : T[k + 1]);
-        if constexpr (V >= 4) {
-          add_level_terms<real, D, V, AC>(T, rt_tab, s_start, n, Em, lane * V);
-        } else {
-#pragma unroll
-          for (int k = 0; k < V; ++k)
-            T[k] = AC::add(T[k], level_term1<real, D, AC>(rt_tab, s_start, n, Em, lane * V + k));
-        }
-      } else {
-        const AC right = T[0].shfl((lane + 1) & (N - 1));
-        T[0] = AC::avg(T[0], right);
-        if (lane < N) T[0] = AC::add(T[0], level_term1<real, D, AC>(rt_tab, s_start, n, Em, lane));
-      }
-    }
-    // hi parts to the block's node-interleaved stage, lo planes straight out
-    const size_t o0 = (size_t)m * ND + (size_t)row * N;
-    const int nb = (row - row0) * N;  // first node of this line in the block
-    real* srow = stage + (size_t)nb * DP + nb / V + m;  // node x at srow[x * DP + x / V]
-    const int per = N >= 32 ? V : 1;
-    if (N >= 32 || lane < N) {
-      if constexpr (sizeof(real) == 4) {
-        if constexpr (V >= 4) {
-#pragma unroll
-          for (int k = 0; k < V; k += 4) {
-            ff v[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              v[q] = T[k + q].normalised();
-              if constexpr (kFp64Acc<AC>) energy_d = fma(T[k + q].v, T[k + q].v, energy_d);
-              else energy = fmaf(v[q].hi, v[q].hi, energy);
-              srow[(size_t)(lane * V + k + q) * DP + lane] = v[q].hi;
-            }
-            if (Elo)
-              *reinterpret_cast<float4*>(Elo + o0 + (size_t)lane * V + k) =
-                  make_float4(v[0].lo, v[1].lo, v[2].lo, v[3].lo);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < V; ++k)
-            if (k < per) {
-              const ff v = T[k].normalised();
-              srow[(size_t)(lane * per + k) * DP + (lane * per + k) / V] = v.hi;
-              if (Elo) Elo[o0 + (size_t)lane * per + k] = v.lo;
-              if constexpr (kFp64Acc<AC>) energy_d = fma(T[k].v, T[k].v, energy_d);
-              else energy = fmaf(v.hi, v.hi, energy);
-            }
-        }
-      } else {
-#pragma unroll
-        for (int k = 0; k < V; ++k)
-          if (k < per) {
-            srow[(size_t)(lane * per + k) * DP + (lane * per + k) / V] = T[k].v;
-            energy = fma(T[k].v, T[k].v, energy);
-          }
-      }
-    }
-  }
-  __syncthreads();
-  {  // the block's RPB lines are contiguous nodes: coalesced stores of the stage
-    const int nreal = RPB * N * DP;
-    real* dst = Ehi + (size_t)row0 * N * DP;
-    for (int i = threadIdx.x; i < nreal; i += blockDim.x) dst[i] = stage[i + (i / DP) / V];
-  }
-  const double tot = warp_sum((double)energy + energy_d);
-  if (lane == 0 && row < rows) partials[task] = tot;
-  if (!fin.active) return;
-  combine_finalize(partials, rows * NC, fin, red);
-}
-
-// ---------------------------------------------------------------- block-per-line combination (lines > 1024)
-
-// Block-kernel accumulator of FP32 fields with FP64 accumulation (the
-// counterpart of CAccD): double sum, split into hi + lo floats on output.
-struct AccF64 {
-  using term = double;
-  double v = 0.0;
-  __device__ __forceinline__ void add(double a) { v += a; }
-  __device__ __forceinline__ void add_acc(const AccF64& o) { v += o.v; }
-  __device__ __forceinline__ void scale(double s) { v *= s; }
-  __device__ __forceinline__ float hi() const { return (float)v; }
-  __device__ __forceinline__ float lo() const { return (float)(v - (double)(float)v); }
-};
-template <typename A>
-constexpr bool kFp64BlockAcc = false;
-template <>
-constexpr bool kFp64BlockAcc<AccF64> = true;
-
-template <typename real, int D, int NC, bool CELL, typename AccT>
-__global__ void __launch_bounds__(256) k_combine(const GridDesc* __restrict__ grids, LevelLists ll, int lmin,
-                                                 const real* __restrict__ E, size_t S, int n, real* __restrict__ Ehi,
-                                                 float* __restrict__ Elo, double* __restrict__ partials,
-                                                 const CombineFinal fin) {
-  using TT = typename AccT::term;
-  extern __shared__ unsigned char smem_raw[];
-  AccT* A = reinterpret_cast<AccT*>(smem_raw);  // [NC][2N], level l of comp m at m*2N + [2^l, 2^(l+1))
-  __shared__ double red[32];
-  const int N = 1 << n;
-  const size_t ND = (size_t)N * (D == 2 ? N : (size_t)N * N);
-  const int row = blockIdx.x;
-  const int y = row & (N - 1);
-  const int z = (D == 3) ? (row >> n) : 0;
-  // Per-grid row parameters of this block's (y, z), computed once: the
-  // 2^(d-1) coarse x-lines that bracket the row and their interpolation
-  // weights (dyadic, exact), the grid's coefficient, in level-list order.
-  constexpr int R = 1 << (D - 1);
-  __shared__ int s_start[18];
-  __shared__ int s_off[CB_MAX_GRIDS][R];
-  __shared__ real s_w[CB_MAX_GRIDS][R];
-  __shared__ real s_c[CB_MAX_GRIDS];
   if (threadIdx.x == 0) {
 #pragma unroll
-    for (int i = 0; i < 18; ++i) s_start[i] = ll.start[i];  // constant indices: no local copy
+    for (int i = 0; i < 18; ++i) start[i] = ls.start[i];  // constant indices: no local copy
   }
-  const int ngl = ll.start[17];
-  for (int gi = threadIdx.x; gi < ngl; gi += blockDim.x) {
-    const GridDesc g = grids[ll.grid[gi]];
-    const int nx = 1 << g.l[0];
-    const int ny = 1 << g.l[1];
-    int ky0, ky1;
-    real fy;
-    bracket<real, CELL>(y, n, g.l[1], ky0, ky1, fy);
-    if (D == 2) {
-      s_off[gi][0] = g.offset + ky0 * nx;
-      s_off[gi][R - 1] = g.offset + ky1 * nx;
-      s_w[gi][0] = (real)1 - fy;
-      s_w[gi][R - 1] = fy;
-    } else {
-      int kz0, kz1;
-      real fz;
-      bracket<real, CELL>(z, n, g.l[D - 1], kz0, kz1, fz);
-      s_off[gi][0] = g.offset + (kz0 * ny + ky0) * nx;
-      s_off[gi][1 % R] = g.offset + (kz0 * ny + ky1) * nx;
-      s_off[gi][2 % R] = g.offset + (kz1 * ny + ky0) * nx;
-      s_off[gi][3 % R] = g.offset + (kz1 * ny + ky1) * nx;
-      s_w[gi][0] = ((real)1 - fy) * ((real)1 - fz);
-      s_w[gi][1 % R] = fy * ((real)1 - fz);
-      s_w[gi][2 % R] = ((real)1 - fy) * fz;
-      s_w[gi][3 % R] = fy * fz;
-    }
-    s_c[gi] = (real)g.coeff;
+  for (int e = threadIdx.x; e < lpb * ngl; e += blockDim.x) {
+    const int r = e / ngl;
+    const LineGrid g = lg[e - r * ngl];
+    int k0, k1;
+    T f;
+    bracket<T, CELL>((brow + r) & (N - 1), n, g.ly, k0, k1, f);
+    const T c = (T)g.coeff;
+    RowTerm<T> rt;
+    rt.off[0] = g.off + (k0 << g.lx);
+    rt.off[1] = g.off + (k1 << g.lx);
+    rt.w[0] = c * ((T)1 - f);
+    rt.w[1] = c * f;
+    tab[e] = rt;
   }
   __syncthreads();
-
-  // the transverse interpolation of grid gi, component m, at x index kx
-  auto tval = [&](int gi, int m, int kx) {
-    const real* base = E + (size_t)m * S + kx;
-    TT val = (TT)s_w[gi][0] * (TT)base[s_off[gi][0]];
-#pragma unroll
-    for (int r = 1; r < R; ++r) val = fma((TT)s_w[gi][r], (TT)base[s_off[gi][r]], val);
-    return val;
-  };
-  // every (level, x index) of the levels Horner reads: each grid's term in
-  // the run's precision (one rounding per product, like the component field
-  // itself), then an error-free addition into the accumulator, so the
-  // alternating-sign sum loses nothing to cancellation.  Cell-centred grids
-  // of x level l enter at level l+1 as centre values (odd) and midpoints
-  // (even), as in the warp kernel.
-  const int l0 = CELL ? min(lmin + 1, n) : lmin;
-  for (int e = threadIdx.x + (1 << l0); e < 2 * N; e += blockDim.x) {
+  pdl_wait();  // the fields (3D: their pairs)
+  const int ntask = lpb * MG * ipl;
+  const GT* Gz = G + (size_t)((brow - row0) >> n) * zstride;  // lpb <= N: the block's lines lie in one plane
+  int level = min(CELL ? lmin + 1 : lmin, n - LK);
+  for (int t = threadIdx.x; t < 2 * ntask; t += blockDim.x) {
+    const int e = t & (2 * ipl - 1), q = t >> (n - LK + 1);
     const int l = 31 - __clz(e);
-    const int kx = e - (1 << l);
-    AccT acc[NC];
-    const int lg = CELL ? l - 1 : l;
-    for (int gi = s_start[lg]; gi < s_start[lg + 1]; ++gi) {
-      const TT c = (TT)s_c[gi];
-#pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        if (!CELL) {
-          acc[m].add(c * tval(gi, m, kx));  // |c| is 1 or 2 (a power of two): exact
-        } else if (kx & 1) {
-          acc[m].add(c * tval(gi, m, kx >> 1));
-        } else {
-          const int nc = 1 << lg;
-          acc[m].add((TT)0.5 * c * tval(gi, m, ((kx >> 1) - 1) & (nc - 1)));
-          acc[m].add((TT)0.5 * c * tval(gi, m, kx >> 1));
-        }
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < NC; ++m) A[m * 2 * N + e] = acc[m];
+    if (l >= level) lat[t] = entering<T, W, DP, CELL>(Gz + q % MG, tab + q / MG * ngl, start, l, e - (1 << l));
   }
   __syncthreads();
-  for (int l = l0; l < n; ++l) {
-    const int cnt = 2 << l;  // size of level l+1
-    const int half = 1 << l;
-    for (int e2 = threadIdx.x; e2 < NC * cnt; e2 += blockDim.x) {
-      const int m = e2 >> (l + 1), e = e2 & (cnt - 1);
-      AccT* Am = A + m * 2 * N;
-      const int k = e >> 1;
-      AccT v = Am[half + k];
-      if (e & 1) {
-        v.add_acc(Am[half + ((k + 1) & (half - 1))]);
-        v.scale((TT)0.5);
-      }
-      Am[cnt + e].add_acc(v);
+  while (level < n - LK) {  // prolong level by level
+    ++level;
+    for (int t = threadIdx.x; t < (lpb * MG << level); t += blockDim.x) {
+      const int x = t & ((1 << level) - 1);
+      S* base = lat + (size_t)(t >> level) * 2 * ipl;
+      const S* pl = base + (1 << (level - 1));
+      S v = pl[x >> 1];
+      if (x & 1) v = S::avg(v, pl[((x >> 1) + 1) & ((1 << (level - 1)) - 1)]);
+      base[(1 << level) + x] = S::add(v, base[(1 << level) + x]);
     }
     __syncthreads();
   }
-  // field energy: each thread sums the squares of its few nodes in the run's
-  // precision; the block and the step reduce the partials in FP64
   real energy = (real)0;
   double energy_d = 0.0;  // FP64 accumulation: the squares of the double results
-  for (int e2 = threadIdx.x; e2 < NC * N; e2 += blockDim.x) {
-    const int m = e2 >> n, x = e2 & (N - 1);
-    AccT v = A[m * 2 * N + N + x];
-    if (CELL) {  // to the regular centres, then the grids of x level n
-      v.add_acc(A[m * 2 * N + N + ((x + 1) & (N - 1))]);
-      v.scale((TT)0.5);
-      for (int gi = s_start[n]; gi < s_start[n + 1]; ++gi) v.add((TT)s_c[gi] * tval(gi, m, x));
+  for (int task = threadIdx.x; task < ntask; task += blockDim.x) {
+    const int item = task & (ipl - 1);
+    const int q = task >> (n - LK), r = q / MG, m0 = q % MG;
+    const int j0 = item << LK;
+    const RowTerm<T>* rtab = tab + r * ngl;
+    const GT* Gm = Gz + m0;
+    const S* top = lat + (size_t)q * 2 * ipl + ipl;
+    S v[K + 1];
+    v[0] = top[item];
+    v[1] = top[(item + 1) & (ipl - 1)];
+    expand<T, W, DP, 1, CELL, PERM>(v, Gm, rtab, start, level, j0, n);
+    if constexpr (CELL) {  // to the regular centres, then the arrays of x level n
+#pragma unroll
+      for (int k = 0; k < K; ++k) v[k] = S::avg(v[k], v[k + 1]);
+      const int end = start[n + 1];
+      for (int gi = start[n]; gi < end; ++gi) {
+        const RowTerm<T> rt = rtab[gi];
+        Term<T, W> t[K];
+        row_run<T, W, DP, K, 0, PERM>(Gm, rt, j0, n, t);
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k].add_term(t[k]);
+      }
     }
-    const size_t o = (size_t)m * ND + (size_t)row * N + x;
-    Ehi[((size_t)row * N + x) * combine_out_stride<D, NC>() + m] = (real)v.hi();
-    if (Elo) Elo[o] = (float)v.lo();
-    if constexpr (kFp64BlockAcc<AccT>) energy_d = fma(v.v, v.v, energy_d);
-    else energy = fma((real)v.hi(), (real)v.hi(), energy);
+    const size_t node = (size_t)(brow + r) * N + j0;
+    real* dst = Ehi + node * DP + m0;
+    if constexpr (sizeof(real) == 4) {
+      float lo[WO][K];
+      float hi[K][W];
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        float l[W];
+        if constexpr (sizeof(T) == 4) {
+          v[k].split(hi[k], l);
+#pragma unroll
+          for (int m = 0; m < WO; ++m) energy = fmaf(hi[k][m], hi[k][m], energy);
+        } else {
+          hi[k][0] = (float)v[k].v[0];
+          l[0] = (float)(v[k].v[0] - (double)hi[k][0]);
+          energy_d = fma(v[k].v[0], v[k].v[0], energy_d);
+        }
+#pragma unroll
+        for (int m = 0; m < WO; ++m) lo[m][k] = l[m];
+      }
+      if constexpr (W == DP) {
+        const float* h = &hi[0][0];
+#pragma unroll
+        for (int i = 0; i < K * DP; i += 4)
+          *reinterpret_cast<float4*>(dst + i) = make_float4(h[i], h[i + 1], h[i + 2], h[i + 3]);
+      } else {
+#pragma unroll
+        for (int k = 0; k < K; ++k) dst[k * DP] = hi[k][0];
+      }
+      if (Elo) {
+#pragma unroll
+        for (int m = 0; m < WO; ++m)
+          *reinterpret_cast<float4*>(Elo + (size_t)(m0 + m) * nd + node) =
+              make_float4(lo[m][0], lo[m][1], lo[m][2], lo[m][3]);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        dst[k * DP] = v[k].v[0];
+        energy = fma(v[k].v[0], v[k].v[0], energy);
+      }
+    }
   }
-  double tot = block_sum_double((double)energy + energy_d, red);
-  if (threadIdx.x == 0) partials[row] = tot;
+  double tot;
+  if constexpr (sizeof(T) == 4) {  // float pairs within the warp, double across warps
+    const ff w = warp_sum_ff(ff{energy, 0.f});
+    tot = block_sum_warps(ff_to_double(w), red);
+  } else {
+    tot = block_sum_double((double)energy + energy_d, red);
+  }
+  if (threadIdx.x == 0) partials[blockIdx.x] = tot;
   if (!fin.active) return;
-  combine_finalize(partials, (int)gridDim.x, fin, red);
+  combine_finalize(partials - (n_part - (int)gridDim.x), n_part, fin, red);
 }
 
-template <typename real, int D, int V, int NC, bool CELL, typename AC>
-static int launch_combine_warp(const GridDesc* grids, const LevelLists& ll, int lmin, const real* E, size_t S, int n,
-                               real* Ehi, float* Elo, double* energy_partials, const CombineFinal& fin,
-                               cudaStream_t s) {
-  const int N = 1 << n;
-  const long long rows = D == 2 ? N : (long long)N * N;
-  constexpr int RPB = combine_rows_per_block<D>();
-  const unsigned blocks = (unsigned)(rows / RPB);  // N >= 4: RPB divides the line count
-  const size_t smem = combine_table_bytes<real, D, NC>(ll.start[17]) +
-                      ((size_t)RPB * N * combine_out_stride<D, NC>() + (size_t)RPB * N / V) * sizeof(real);
-  static bool attr_set = false;
-  if (!attr_set && smem > 48 * 1024) {
-    SG_CUDA(cudaFuncSetAttribute(k_combine_warp<real, D, V, NC, CELL, AC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+template <typename real, typename GT, typename T, int NC, bool CELL, bool PERM>
+static int launch_lines(const CombineTables& ct, const GT* G, size_t zstride, int n, int row0, int rows, size_t nd,
+                        real* Ehi, float* Elo, double* partials, int* part0, const CombineFinal& fin,
+                        cudaStream_t s) {
+  const int N = 1 << n, ipl = N / CB_RUN;
+  constexpr int W = carried<T, NC>(), MG = W >= NC ? 1 : NC;
+  // Threads per block and tasks to share among them.  From 2^18 tasks on
+  // (2D n = 10, 3D n = 7) a block takes 384 or more, two per thread, which
+  // spreads its tables and barriers: 3D n = 7 59 us against 71 us with 128
+  // and 128, 2D n = 10 20.5 against 21.2.  Below, small blocks reach more SMs:
+  // 3D n = 6 25 against 43 us, 2D n = 8 12.3 against 14.5.  Doubles on tiny
+  // grids go smaller still (2D n = 6: 13.5 against 14.3 us).
+  const size_t tasks = nd * MG / CB_RUN;
+  const bool large = sizeof(T) == 4 && tasks >= ((size_t)1 << 18);
+  const int ft = large ? 384 : sizeof(T) == 8 && tasks < ((size_t)1 << 14) ? 64 : 128;
+  const int fthr = large ? 192 : ft;
+  int lpb = 1;
+  while (2 * lpb <= std::min(rows, N) && lpb * MG * ipl < ft) lpb *= 2;
+  const int ngl = ct.ls.start[17];
+  const unsigned blocks = (unsigned)(rows / lpb);  // both powers of two
+  const unsigned threads = (unsigned)std::min(fthr, (lpb * MG * ipl + 31) / 32 * 32);
+  const size_t smem = (size_t)lpb * ngl * sizeof(RowTerm<T>) + (size_t)2 * lpb * MG * ipl * sizeof(Sum<T, W>);
+  static std::atomic<bool> attr_set{false};
+  if (smem > 40 * 1024 && !attr_set) {  // with the static part the total may pass 48 KB
+    SG_CUDA(cudaFuncSetAttribute(k_combine_line<real, GT, T, NC, CELL, PERM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  200 * 1024));
     attr_set = true;
   }
-  SG_CUDA(launch_pdl(k_combine_warp<real, D, V, NC, CELL, AC>, dim3(blocks), dim3(32 * RPB * NC), smem, s, grids, ll, lmin, E,
-                     S, n, Ehi, Elo, energy_partials, fin));
+  SG_CUDA(launch_pdl(k_combine_line<real, GT, T, NC, CELL, PERM>, dim3(blocks), dim3(threads), smem, s, ct.lines, ct.ls,
+                     ct.lmin, G, zstride, n, lpb, row0, nd, Ehi, Elo, partials + *part0, *part0 + (int)blocks, fin));
+  *part0 += (int)blocks;
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
 
-template <typename real, int D, int NC, bool CELL, typename AC, typename AccT>
-static int launch_combine_nc(const GridDesc* grids, const LevelLists& ll, int lmin, const real* E, size_t S, int n,
-                             real* Ehi, float* Elo, double* energy_partials, const CombineFinal& fin,
-                             cudaStream_t s) {
+template <typename real, int D, int NC, bool CELL, typename T>
+static int launch_combine_nc(const CombineTables& ct, const real* E, int n, real* Ehi, float* Elo, double* partials,
+                             const CombineFinal& fin, cudaStream_t s) {
   const int N = 1 << n;
-  switch (N) {  // lines of up to 1024 nodes: warp per line, values in registers
-    case 4:
-    case 8:
-    case 16:
-    case 32:
-      return launch_combine_warp<real, D, 1, NC, CELL, AC>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-    case 64:
-      return launch_combine_warp<real, D, 2, NC, CELL, AC>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-    case 128:
-      return launch_combine_warp<real, D, 4, NC, CELL, AC>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-    case 256:
-      return launch_combine_warp<real, D, 8, NC, CELL, AC>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-    case 512:
-      return launch_combine_warp<real, D, 16, NC, CELL, AC>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-    case 1024:
-      return launch_combine_warp<real, D, 32, NC, CELL, AC>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-    default:
-      break;
+  const size_t nd = (size_t)1 << (D * n);
+  int part0 = 0;
+  if constexpr (D == 2) {
+    return launch_lines<real, real, T, NC, CELL, (NC > 1)>(ct, E, 0, n, 0, N, nd, Ehi, Elo, partials, &part0, fin, s);
+  } else {
+    // as many planes at a time as the pair scratch holds (a power of two, so
+    // that every launch has whole blocks); the last launch closes the step
+    constexpr int DP = node_stride<NC>();
+    const size_t plane = (size_t)DP * ct.S2;
+    int nz = N;
+    while (nz > 1 && (size_t)nz * plane * sizeof(T) > ct.scratch_bytes) nz >>= 1;
+    if ((size_t)nz * plane * sizeof(T) > ct.scratch_bytes) {
+      set_error("combination: pair scratch smaller than one plane");
+      return SG_ERR_SIZE;
+    }
+    T* G = static_cast<T*>(ct.scratch);
+    for (int z0 = 0; z0 < N; z0 += nz) {
+      SG_CUDA(launch_pdl(k_combine_planes<real, T, NC, CELL>,
+                         dim3((unsigned)((ct.S2 + 255) / 256), (unsigned)((nz + PL_Z - 1) / PL_Z)), dim3(256), 0, s,
+                         ct.pairs, ct.npairs, E, ct.S2, n, z0, nz, G));
+      SG_CHECK_LAUNCH();
+      CombineFinal f = fin;
+      if (z0 + nz < N) f.active = 0;
+      SG_TRY(launch_lines<real, T, T, NC, CELL, true>(ct, G, plane, n, z0 * N, nz * N, nd, Ehi, Elo, partials, &part0, f,
+                                                      s));
+    }
+    return SG_OK;
   }
-  unsigned rows = (unsigned)(D == 2 ? N : N * N);
-  size_t smem = (size_t)NC * 2 * N * sizeof(AccT);
-  static bool attr_set = false;
-  if (!attr_set) {
-    SG_CUDA(cudaFuncSetAttribute(k_combine<real, D, NC, CELL, AccT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set = true;
-  }
-  k_combine<real, D, NC, CELL, AccT><<<rows, 256, smem, s>>>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin);
-  SG_CHECK_LAUNCH();
-  return SG_OK;
 }
 
-template <typename real, int D, typename AC, typename AccT>
-static int launch_combine_acc(const GridDesc* grids, const LevelLists& ll, int lmin, const real* E, size_t S, int n,
-                              real* Ehi, float* Elo, double* energy_partials, const CombineFinal& fin, cudaStream_t s,
-                              int ncomp, bool cell) {
+template <typename real, int D, typename T>
+static int launch_combine_acc(const CombineTables& ct, const real* E, int n, real* Ehi, float* Elo, double* partials,
+                              const CombineFinal& fin, cudaStream_t s, int ncomp, bool cell) {
   if (cell) {
-    if (ncomp == 1)
-      return launch_combine_nc<real, D, 1, true, AC, AccT>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-    return launch_combine_nc<real, D, D, true, AC, AccT>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
+    if (ncomp == 1) return launch_combine_nc<real, D, 1, true, T>(ct, E, n, Ehi, Elo, partials, fin, s);
+    return launch_combine_nc<real, D, D, true, T>(ct, E, n, Ehi, Elo, partials, fin, s);
   }
-  if (ncomp == 1)
-    return launch_combine_nc<real, D, 1, false, AC, AccT>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
-  return launch_combine_nc<real, D, D, false, AC, AccT>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s);
+  if (ncomp == 1) return launch_combine_nc<real, D, 1, false, T>(ct, E, n, Ehi, Elo, partials, fin, s);
+  return launch_combine_nc<real, D, D, false, T>(ct, E, n, Ehi, Elo, partials, fin, s);
 }
 
-// fp64_acc selects FP64 accumulation of FP32 fields (CAccD / AccF64); the
-// FP64 path always accumulates in double.
+// fp64_acc selects FP64 accumulation of FP32 fields; the FP64 path always
+// accumulates in double.
 template <typename real, int D>
-int launch_combine(const GridDesc* grids, const LevelLists& ll, int lmin, const real* E, size_t S, int n, real* Ehi,
-                   float* Elo, double* energy_partials, const CombineFinal& fin, cudaStream_t s, int ncomp,
-                   bool cell, bool fp64_acc) {
+int launch_combine(const CombineTables& ct, const real* E, int n, real* Ehi, float* Elo, double* energy_partials,
+                   const CombineFinal& fin, cudaStream_t s, int ncomp, bool cell, bool fp64_acc) {
   if constexpr (sizeof(real) == 4) {
-    if (fp64_acc)
-      return launch_combine_acc<real, D, CAccD, AccF64>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin, s,
-                                                        ncomp, cell);
+    if (fp64_acc) return launch_combine_acc<real, D, double>(ct, E, n, Ehi, Elo, energy_partials, fin, s, ncomp, cell);
   }
-  return launch_combine_acc<real, D, CAcc<real>, Acc<real>>(grids, ll, lmin, E, S, n, Ehi, Elo, energy_partials, fin,
-                                                            s, ncomp, cell);
+  return launch_combine_acc<real, D, real>(ct, E, n, Ehi, Elo, energy_partials, fin, s, ncomp, cell);
 }
 
-#define SG_INST_COMB(real, D)                                                                                   \
-  template int launch_combine<real, D>(const GridDesc*, const LevelLists&, int, const real*, size_t, int, real*, \
-                                       float*, double*, const CombineFinal&, cudaStream_t, int, bool, bool);
+#define SG_INST_COMB(real, D)                                                                                     \
+  template int launch_combine<real, D>(const CombineTables&, const real*, int, real*, float*, double*,            \
+                                       const CombineFinal&, cudaStream_t, int, bool, bool);
 SG_INST_COMB(float, 2)
 SG_INST_COMB(float, 3)
 SG_INST_COMB(double, 2)

@@ -689,13 +689,21 @@ class Engine final : public EngineBase {
       return SG_ERR_STATE;
     }
     if (cap < (size_t)D * S_) return size_error("sg_pic_get_grid_field");
-    std::vector<double> all((size_t)D * S_);
-    SG_TRY(copy_to_host_double(E_arena_, all.data(), (size_t)D * S_));
+    constexpr size_t st = ec_stride<D>();
+    std::vector<double> all(st * S_);
+    SG_TRY(copy_to_host_double(E_arena_, all.data(), st * S_));
     size_t o = 0;
     for (int g = 0; g < ngrids_; ++g) {
       size_t sz = (size_t)gdesc_[g].size, off = (size_t)gdesc_[g].offset;
       for (int m = 0; m < D; ++m) {
-        std::memcpy(E + o, all.data() + (size_t)m * S_ + off, sz * sizeof(double));
+        for (size_t k = 0; k < sz; ++k) {
+          size_t at = k;
+          if (D == 2) {  // stored in the line kernel's order
+            const int l = gdesc_[g].l[0], x = (int)(k & (((size_t)1 << l) - 1));
+            at = k - x + line_pos(x, l, n_);
+          }
+          E[o + k] = all[(off + at) * st + m];
+        }
         o += sz;
       }
     }
@@ -720,7 +728,7 @@ class Engine final : public EngineBase {
     SG_TRY(alloc((void**)&tmp, ND_ * sizeof(real)));
     CombineFinal off;
     std::memset(&off, 0, sizeof(off));
-    int st = launch_combine<real, D>(grids_dev_, levels_, lmin_, rho_arena_, S_, n_, tmp, nullptr, fe_partials_, off,
+    int st = launch_combine<real, D>(comb_, rho_arena_, n_, tmp, nullptr, fe_partials_, off,
                                      stream_, 1, cfg_.cell, cfg_.combine_fp64);
     if (st == SG_OK) st = copy_to_host_double(tmp, rho, ND_);
     free_one(tmp);
@@ -1046,7 +1054,6 @@ class Engine final : public EngineBase {
     ngrids_ = (int)grids_.size();
     gdesc_.assign(ngrids_, GridDesc{});
     size_t off = 0;
-    lmin_ = n_;
     for (int g = 0; g < ngrids_; ++g) {
       GridDesc& d = gdesc_[g];
       std::memset(&d, 0, sizeof(d));
@@ -1063,44 +1070,100 @@ class Engine final : public EngineBase {
       d.size = sz;
       d.vol = vol;
       off += (size_t)sz;
-      lmin_ = std::min(lmin_, d.l[0]);
     }
     S_ = off;
     // (re)allocate arenas
     for (void* p : grid_bufs_) free_one(p);
     grid_bufs_.clear();
     SG_TRY(galloc((void**)&grids_dev_, ngrids_ * sizeof(GridDesc)));
-    {  // grids grouped by x level for the combination
-      std::vector<int> order;
-      std::memset(&levels_, 0, sizeof(levels_));
-      for (int l = 0; l <= n_; ++l) {
-        levels_.start[l] = (int)order.size();
-        for (int g = 0; g < ngrids_; ++g)
-          if (gdesc_[g].l[0] == l) order.push_back(g);
-      }
-      for (int l = n_ + 1; l < 18; ++l) levels_.start[l] = (int)order.size();
-      if ((int)order.size() > CB_MAX_GRIDS) {
-        set_error("too many component grids for the combination kernel");
-        return SG_ERR_UNSUPPORTED;
-      }
-      int* dev = nullptr;
-      SG_TRY(galloc((void**)&dev, order.size() * sizeof(int)));
-      SG_CUDA(cudaMemcpyAsync(dev, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice, stream_));
-      levels_.grid = dev;
-    }
+    SG_TRY(build_combine_tables());
     SG_TRY(galloc((void**)&rho_arena_, S_ * sizeof(real)));
     SG_TRY(galloc((void**)&A_, S_ * sizeof(cplx<real>)));
-    SG_TRY(galloc((void**)&B_, (size_t)D * S_ * sizeof(cplx<real>)));
-    SG_TRY(galloc((void**)&E_arena_, (size_t)D * S_ * sizeof(real)));
+    SG_TRY(galloc((void**)&B_, (size_t)((D + 1) / 2) * S_ * sizeof(cplx<real>)));  // component pairs
+    SG_TRY(galloc((void**)&E_arena_, (size_t)ec_stride<D>() * S_ * sizeof(real)));  // node-interleaved
     SG_CUDA(cudaMemcpyAsync(grids_dev_, gdesc_.data(), ngrids_ * sizeof(GridDesc), cudaMemcpyHostToDevice, stream_));
     SG_TRY(build_restrict_jobs());
     SG_TRY(build_fft_jobs());
+    if (D == 3) {
+      // The combination's pair scratch takes what the run's estimated
+      // footprint leaves (all planes at tau = 1: 6.3 MB at n = 7); larger tau,
+      // whose pairs grow towards the regular grid, go in several runs of
+      // planes instead of past the estimate that serving admits by (which
+      // leaves out the estimator's and the filter mode's arrays), in eight
+      // runs at most.
+      const size_t plane = (size_t)ec_stride<D>() * comb_.S2 * ((sizeof(real) == 8 || cfg_.combine_fp64) ? 8 : 4);
+      const size_t est = estimate_footprint(sizeof(real) == 8 ? SG_FP64 : SG_FP32, D, n_, tau_, np_);
+      const size_t used = bytes_ - est_bytes_;
+      const size_t left = std::max(est > used ? est - used : 0, plane * N_ / 8);
+      comb_.scratch_bytes = std::max(plane, std::min(plane * (size_t)N_, left));
+      SG_TRY(galloc(&comb_.scratch, comb_.scratch_bytes));
+    }
     SG_CUDA(cudaStreamSynchronize(stream_));
     return SG_OK;
   }
   int galloc(void** p, size_t bytes) {
     SG_TRY(alloc(p, bytes));
     grid_bufs_.push_back(*p);
+    return SG_OK;
+  }
+
+  // The combination's arrays grouped by x level: 2D, the component grids;
+  // 3D, the pairs (l_1, l_2) whose grids the z prolongation collapses.
+  int build_combine_tables() {
+    std::vector<LineGrid> lines;
+    std::vector<PlanePair> pairs;
+    comb_ = CombineTables();
+    comb_.lmin = n_;
+    int S2 = 0;
+    for (int l = 0; l <= n_; ++l) {
+      comb_.ls.start[l] = (int)lines.size();
+      for (int g = 0; g < ngrids_; ++g) {
+        const GridDesc& d = gdesc_[g];
+        if (d.l[0] != l) continue;
+        comb_.lmin = std::min(comb_.lmin, l);
+        if (D == 2) {
+          lines.push_back({d.l[0], d.l[1], d.offset, d.coeff});
+          continue;
+        }
+        size_t p = (size_t)comb_.ls.start[l];
+        while (p < lines.size() && lines[p].ly != d.l[1]) ++p;
+        if (p == lines.size()) {
+          lines.push_back({d.l[0], d.l[1], S2, 1});
+          PlanePair q;
+          std::memset(&q, 0, sizeof(q));
+          q.off = S2;
+          q.logs = d.l[0] + d.l[1];
+          q.lx = l;
+          pairs.push_back(q);
+          S2 += 1 << q.logs;
+        }
+        PlanePair& q = pairs[p];
+        if (q.ng == 3) {
+          set_error("combination: more than three grids share two levels");
+          return SG_ERR_UNSUPPORTED;
+        }
+        q.goff[q.ng] = d.offset;
+        q.lz[q.ng] = d.l[D - 1];
+        q.coeff[q.ng++] = d.coeff;
+      }
+    }
+    for (int l = n_ + 1; l < 18; ++l) comb_.ls.start[l] = (int)lines.size();
+    if ((int)lines.size() > CB_MAX_GRIDS) {
+      set_error("too many component grids for the combination kernel");
+      return SG_ERR_UNSUPPORTED;
+    }
+    LineGrid* ld = nullptr;
+    SG_TRY(galloc((void**)&ld, lines.size() * sizeof(LineGrid)));
+    SG_CUDA(cudaMemcpyAsync(ld, lines.data(), lines.size() * sizeof(LineGrid), cudaMemcpyHostToDevice, stream_));
+    comb_.lines = ld;
+    if (D == 3) {
+      PlanePair* pd = nullptr;
+      SG_TRY(galloc((void**)&pd, pairs.size() * sizeof(PlanePair)));
+      SG_CUDA(cudaMemcpyAsync(pd, pairs.data(), pairs.size() * sizeof(PlanePair), cudaMemcpyHostToDevice, stream_));
+      comb_.pairs = pd;
+      comb_.npairs = (int)pairs.size();
+      comb_.S2 = S2;
+    }
     return SG_OK;
   }
 
@@ -1271,6 +1334,7 @@ class Engine final : public EngineBase {
 
   int ensure_estimator_buffers() {
     if (est_z_) return SG_OK;
+    const size_t before = bytes_;
     SG_TRY(alloc((void**)&est_rho_, ND_ * sizeof(double)));
     SG_TRY(alloc((void**)&est_z_, ND_ * sizeof(cplx<double>)));
     SG_TRY(alloc((void**)&est_w_, ND_ * sizeof(cplx<double>)));
@@ -1278,6 +1342,7 @@ class Engine final : public EngineBase {
     const std::vector<cplx<double>> tw = make_twiddles<double>(n_);
     SG_TRY(alloc((void**)&tw64_, tw.size() * sizeof(cplx<double>)));
     SG_CUDA(cudaMemcpyAsync(tw64_, tw.data(), tw.size() * sizeof(cplx<double>), cudaMemcpyHostToDevice, stream_));
+    est_bytes_ = bytes_ - before;
     return SG_OK;
   }
 
@@ -1632,7 +1697,7 @@ class Engine final : public EngineBase {
     fin.fe_scale = fe_scale();
     fin.dd = dd_;
     fin.counter = comb_counter_;
-    return launch_combine<real, D>(grids_dev_, levels_, lmin_, E_arena_, S_, n_, Ehi_, Elo_, fe_partials_, fin,
+    return launch_combine<real, D>(comb_, E_arena_, n_, Ehi_, Elo_, fe_partials_, fin,
                                    stream_, D, cfg_.cell, cfg_.combine_fp64);
   }
 
@@ -1642,7 +1707,7 @@ class Engine final : public EngineBase {
   int enqueue_filter_density() {
     CombineFinal off;
     std::memset(&off, 0, sizeof(off));
-    return launch_combine<real, D>(grids_dev_, levels_, lmin_, rho_arena_, S_, n_, rho_f_, nullptr, fe_partials_, off,
+    return launch_combine<real, D>(comb_, rho_arena_, n_, rho_f_, nullptr, fe_partials_, off,
                                    stream_, 1, cfg_.cell, cfg_.combine_fp64);
   }
   int enqueue_regular_solve(const double* ke) {
@@ -1884,7 +1949,7 @@ class Engine final : public EngineBase {
 
   std::vector<DevBuf> bufs_;
   std::vector<void*> grid_bufs_;
-  size_t bytes_ = 0;
+  size_t bytes_ = 0, est_bytes_ = 0;  // device memory, and the estimator's share of it
 
   PArrays<real, D> P_[2];
   int cur_ = 0;
@@ -1928,8 +1993,8 @@ class Engine final : public EngineBase {
 
   std::vector<GridSpec> grids_;
   std::vector<GridDesc> gdesc_;
-  int ngrids_ = 0, lmin_ = 0;
-  LevelLists levels_{};
+  int ngrids_ = 0;
+  CombineTables comb_;
   bool per_grid_ = false;
   int solve_mode_ = -1;  // -1 untuned, 0 per-axis passes, 1 one block per grid
   int force_mode_ = -1;  // solve variant fixed by the caller, -1 autotuned

@@ -167,8 +167,8 @@ struct SolveArena {
   const GridDesc* grids;
   const real* rho;     // S
   cplx<real>* A;       // S
-  cplx<real>* B;       // D * S
-  real* E;             // D * S
+  cplx<real>* B;       // (D + 1) / 2 * S
+  real* E;             // ec_stride * S: node-interleaved components (3D: a zero fourth)
   size_t S;
   const cplx<real>* tw;  // make_twiddles(log_nmax)
   int log_nmax;
@@ -220,15 +220,41 @@ int launch_fft_array_axis(cplx<real>* data, int D, int logn, int axis, bool inve
                           const cplx<real>* tw, int log_nmax, cudaStream_t s);
 
 // ---------------------------------------------------------------- combine
-// Grids grouped by their x level: grid[start[l] .. start[l+1]) have l_1 = l;
-// start[l] for l > n holds the total count.
+// Place of node x of a level-l line in the arrays the line kernel reads (2D:
+// the component fields, 3D: the planes of pairs).  A thread of that kernel
+// takes CB_RUN consecutive nodes of a level-n line and half as many one
+// level below; node j of every thread's run is stored next to the other
+// threads' node j, so that a warp's loads are consecutive.
+constexpr int CB_RUN = 4;
+__host__ __device__ __forceinline__ int line_pos(int x, int l, int n) {
+  return l == n ? ((x & 3) << (l - 2)) + (x >> 2) : l == n - 1 ? ((x & 1) << (l - 1)) + (x >> 1) : x;
+}
+// The arrays the line kernel combines: 2D, the component grids; 3D, the pairs
+// (l_1, l_2) with the z axis already prolonged.  Grouped by x level:
+// start[l] .. start[l+1] have l_1 = l; start[l] for l > n holds the count.
 constexpr int CB_MAX_GRIDS = 128;
-struct LevelLists {
-  int start[18];
-  const int* grid;
+struct LineGrid {
+  int lx, ly, off, coeff;
 };
-
-
+struct LevelStarts {
+  int start[18];
+};
+// 3D: the grids of one pair, and the pair's place in a plane of pairs.
+struct PlanePair {
+  int off, logs, ng, lx;  // offset in the plane, l_1 + l_2, number of grids, l_1
+  int goff[3], lz[3], coeff[3];
+  int pad2[3];
+};
+struct CombineTables {
+  const LineGrid* lines = nullptr;
+  LevelStarts ls{};
+  int lmin = 0;  // smallest x level
+  // 3D only
+  const PlanePair* pairs = nullptr;
+  int npairs = 0, S2 = 0;  // S2: values of one plane and component
+  void* scratch = nullptr;
+  size_t scratch_bytes = 0;
+};
 
 // ---------------------------------------------------------------- push
 // The combined field the push gathers from is stored node-interleaved:
@@ -316,12 +342,13 @@ struct CombineFinal {
   unsigned* counter;  // zero between launches; the last block resets it
 };
 
+// E: the component fields, node-interleaved (ncomp = D, ec_stride values per
+// node), or a density (ncomp = 1); Ehi likewise.
 template <typename real, int D>
-int launch_combine(const GridDesc* grids, const LevelLists& ll, int lmin, const real* E, size_t S, int n,
-                   real* Ehi, float* Elo, double* energy_partials, const CombineFinal& fin,
-                   cudaStream_t s, int ncomp,  // ncomp = D: the fields, interleaved; 1: a density, plain
-                   bool cell,                  // cell-centred grids
-                   bool fp64_acc);             // FP32 path: accumulate in double instead of float-float
+int launch_combine(const CombineTables& ct, const real* E, int n, real* Ehi, float* Elo, double* energy_partials,
+                   const CombineFinal& fin, cudaStream_t s, int ncomp,
+                   bool cell,       // cell-centred grids
+                   bool fp64_acc);  // FP32 path: accumulate in double instead of float pairs
 
 template <typename real>
 int launch_to_double(const real* src, double* dst, size_t n, cudaStream_t s);

@@ -221,9 +221,10 @@ __global__ void __launch_bounds__(FFT_BLOCK_VALUES / 2) k_fft_pass(int kind, Sol
       a.A[g.offset + off] = v;
     } else if (kind == FFT_INV_MID) {
       a.B[(size_t)J.comp * S + g.offset + off] = v;
-    } else {  // FFT_INV_LAST: real part -> component 2p, imaginary -> 2p + 1
-      a.E[(size_t)(2 * J.comp) * S + g.offset + off] = v.x;
-      if (2 * J.comp + 1 < a.dim) a.E[(size_t)(2 * J.comp + 1) * S + g.offset + off] = v.y;
+    } else {  // FFT_INV_LAST: real part -> component 2p, imaginary -> 2p + 1 (none: zero)
+      const bool two = 2 * J.comp + 1 < a.dim;
+      const long long at = a.dim == 2 ? off - t + line_pos(t, logn, a.log_nmax) : off;  // the axis is x
+      reinterpret_cast<cplx<real>*>(a.E)[(g.offset + at) * ((a.dim + 1) / 2) + J.comp] = {v.x, two ? v.y : (real)0};
     }
   }
 }
@@ -361,8 +362,9 @@ __device__ __forceinline__ void solve_grid_block(const SolveArena<real>& a, int 
     __syncthreads();
     for (int ax = 0; ax < D; ++ax) fft_axis_inplace<real>(B, logs, S, ax, true, tws);
     for (int e = threadIdx.x; e < S; e += blockDim.x) {
-      a.E[(size_t)ma * a.S + g.offset + e] = B[e].x;
-      if (mb < D) a.E[(size_t)mb * a.S + g.offset + e] = B[e].y;
+      const int x = e & (n0 - 1);
+      const int at = D == 2 ? e - x + line_pos(x, logs[0], a.log_nmax) : e;
+      reinterpret_cast<cplx<real>*>(a.E)[(size_t)(g.offset + at) * ((D + 1) / 2) + pr] = {B[e].x, mb < D ? B[e].y : (real)0};
     }
     __syncthreads();
   }
