@@ -496,37 +496,6 @@ __device__ __forceinline__ void expand(Sum<T, W>* v, const GT* __restrict__ G, c
   }
 }
 
-// The last block to finish reduces the
-// energy partials (and the push's kinetic-energy partials) in FP64, in a
-// fixed order, so the step needs no separate bookkeeping launch.
-__device__ __forceinline__ void combine_finalize(const double* partials, int n_part, const CombineFinal& fin,
-                                                 double* red) {
-  __shared__ int s_last;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned t = atomicAdd(fin.counter, 1u);
-    s_last = (t == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  double a = 0.0;
-  for (int i = threadIdx.x; i < n_part; i += blockDim.x) a += __ldcg(partials + i);
-  const double fe = block_sum_double(a, red);
-  double b = 0.0;
-  if (fin.ke_partials)
-    for (int i = threadIdx.x; i < fin.n_ke; i += blockDim.x) b += __ldcg(fin.ke_partials + i);
-  const double ke = block_sum_double(b, red);
-  if (threadIdx.x == 0) {
-    DevDiag* dd = fin.dd;
-    dd->field_energy_prev = dd->field_energy;
-    dd->field_energy = fe * fin.fe_scale;
-    if (fin.ke_partials) dd->kinetic_energy = ke;
-    *fin.counter = 0u;
-  }
-}
-
 // Sum of one value per warp (the same in all its lanes), valid in thread 0.
 __device__ __forceinline__ double block_sum_warps(double w, double* sh) {
   __syncthreads();

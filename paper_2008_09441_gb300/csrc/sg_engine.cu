@@ -178,17 +178,18 @@ class Engine final : public EngineBase {
     }
     filter_ = cfg.mode == SG_MODE_FILTER;
     if (filter_) {
+      // the regular-grid solve has no low parts: the planes stay zero
+      if (Elo_) SG_CUDA(cudaMemsetAsync(Elo_, 0, (size_t)D * ND_ * sizeof(float), stream_));
       SG_TRY(alloc((void**)&rho_f_, ND_ * sizeof(real)));
-      SG_TRY(alloc((void**)&regA_, ND_ * sizeof(cplx<real>)));
-      SG_TRY(alloc((void**)&regB_, ND_ * sizeof(cplx<real>)));
+      SG_TRY(alloc((void**)&regA_, half_spectrum(D, n_) * sizeof(cplx<real>)));
+      SG_TRY(alloc((void**)&regB_, D * half_spectrum(D, n_) * sizeof(cplx<real>)));
       std::vector<real> kt((size_t)D * N_);
       for (int m = 0; m < D; ++m)
         for (int i = 0; i < N_; ++i)
           kt[(size_t)m * N_ + i] = (real)(2.0 * M_PI / cfg_.L[m] * (double)(i < N_ / 2 ? i : i - N_));
       SG_TRY(alloc((void**)&ktab_, kt.size() * sizeof(real)));
       SG_CUDA(cudaMemcpyAsync(ktab_, kt.data(), kt.size() * sizeof(real), cudaMemcpyHostToDevice, stream_));
-      reg_blocks_ = (int)std::min<size_t>(152 * 8, (ND_ + 255) / 256);
-      SG_TRY(alloc((void**)&reg_partials_, (size_t)2 * reg_blocks_ * sizeof(double)));
+      SG_TRY(alloc((void**)&reg_partials_, (ND_ / N_ * 3 / 2) * sizeof(double)));
     }
 
     SG_TRY(particle_stats());
@@ -492,64 +493,43 @@ class Engine final : public EngineBase {
       }
     SG_TRY(ensure_estimator_buffers());
     const double L = cfg_.L[0];
-    // rho~ of the current positions (the deposit of the last step).
-    SG_TRY(launch_to_double<real>(rho_reg_, est_rho_, ND_, stream_));
-    SG_TRY(launch_real_to_cplx(est_rho_, est_z_, ND_, 1.0 / (double)ND_, stream_));
-    for (int ax = 0; ax < D; ++ax) SG_TRY(launch_fft_array_axis<double>(est_z_, D, n_, ax, false, tw64_, n_, stream_));
-    SG_TRY(launch_maxabs_cplx(est_z_, ND_, est_scalar_ + 0, stream_));
     const double Pc = (double)np_ / (double)ND_;
     const double frac = cfg_.alpha * std::sqrt(cfg_.pc_ref / Pc);
-    SG_TRY(launch_threshold(est_z_, ND_, est_scalar_ + 0, frac, stream_));
     double kfac[3] = {0, 0, 0};
     for (int m = 0; m < D; ++m) kfac[m] = 2.0 * M_PI / cfg_.L[m];
     // masks: kappa_m (single axis), beta (pairs), gamma (all three)
-    std::vector<int> masks;
-    for (int m = 0; m < D; ++m) masks.push_back(1 << m);
-    if (D == 2) {
-      masks.push_back(3);
-    } else {
-      masks.push_back(3);  // xy
-      masks.push_back(6);  // yz
-      masks.push_back(5);  // zx
-      masks.push_back(7);  // xyz
-    }
+    constexpr int nmask = D == 2 ? 3 : 7;
+    constexpr int masks2[3] = {1, 2, 3}, masks3[7] = {1, 2, 4, 3 /* xy */, 6 /* yz */, 5 /* zx */, 7};
     const bool paper = cfg_.tau_constants == SG_TAU_CONST_PAPER;
-    for (size_t i = 0; i < masks.size(); ++i) {
-      if (paper) {
-        SG_TRY(launch_kmult(est_z_, est_w_, D, n_, kfac, masks[i], stream_));
-        for (int ax = 0; ax < D; ++ax)
-          SG_TRY(launch_fft_array_axis<double>(est_w_, D, n_, ax, true, tw64_, n_, stream_));
-        SG_TRY(launch_maxabs_real_part(est_w_, ND_, est_scalar_ + 1 + i, stream_));
-      } else {
-        SG_TRY(launch_maxabs_kmult(est_z_, D, n_, kfac, masks[i], est_scalar_ + 1 + i, stream_));
-      }
-    }
-    SG_TRY(launch_maxabs_real(est_rho_, ND_, est_scalar_ + 8, stream_));
-    double sc[9];
-    SG_CUDA(cudaMemcpyAsync(sc, est_scalar_, sizeof(sc), cudaMemcpyDeviceToHost, stream_));
+    // rho~ of the current positions (the deposit of the last step)
+    SG_TRY(launch_estimator<real>(rho_reg_, est_z_, est_w_, est_wcount_, D, n_, kfac, frac, D == 2 ? masks2 : masks3,
+                                  nmask, paper, tw64_, est_scalar_, stream_));
+    SG_TRY(ensure_pinned(&est_host_, &est_host_bytes_, 9 * sizeof(double)));
+    const double* sc = static_cast<const double*>(est_host_);
+    SG_CUDA(cudaMemcpyAsync(est_host_, est_scalar_, 9 * sizeof(double), cudaMemcpyDeviceToHost, stream_));
     SG_CUDA(cudaStreamSynchronize(stream_));
     double kappa[3] = {0, 0, 0}, beta[3] = {0, 0, 0}, gamma = 0, sigma;
     const double Q = std::fabs(charge_total_);
     if (paper) {
-      for (int m = 0; m < D; ++m) kappa[m] = 0.25 * sc[1 + m];
+      for (int m = 0; m < D; ++m) kappa[m] = 0.25 * sc[m];
       if (D == 2) {
-        beta[0] = sc[1 + 2] / 72.0;
+        beta[0] = sc[2] / 72.0;
       } else {
-        beta[0] = sc[1 + 3] / 72.0;
-        beta[1] = sc[1 + 4] / 72.0;
-        beta[2] = sc[1 + 5] / 72.0;
-        gamma = sc[1 + 6] / 864.0;
+        beta[0] = sc[3] / 72.0;
+        beta[1] = sc[4] / 72.0;
+        beta[2] = sc[5] / 72.0;
+        gamma = sc[6] / 864.0;
       }
       sigma = std::sqrt(std::pow(2.0 / 3.0, D) * Q * sc[8]);
     } else {
-      for (int m = 0; m < D; ++m) kappa[m] = sc[1 + m];
+      for (int m = 0; m < D; ++m) kappa[m] = sc[m];
       if (D == 2) {
-        beta[0] = sc[1 + 2];
+        beta[0] = sc[2];
       } else {
-        beta[0] = sc[1 + 3];
-        beta[1] = sc[1 + 4];
-        beta[2] = sc[1 + 5];
-        gamma = sc[1 + 6];
+        beta[0] = sc[3];
+        beta[1] = sc[4];
+        beta[2] = sc[5];
+        gamma = sc[6];
       }
       sigma = std::sqrt(Q * sc[8]);
     }
@@ -964,6 +944,9 @@ class Engine final : public EngineBase {
     if (diag_host_) cudaFreeHost(diag_host_);
     diag_host_ = nullptr;
     diag_host_bytes_ = 0;
+    if (est_host_) cudaFreeHost(est_host_);
+    est_host_ = nullptr;
+    est_host_bytes_ = 0;
     if (stats_host_) cudaFreeHost(stats_host_);
     stats_host_ = nullptr;
     stats_host_bytes_ = 0;
@@ -1335,9 +1318,12 @@ class Engine final : public EngineBase {
   int ensure_estimator_buffers() {
     if (est_z_) return SG_OK;
     const size_t before = bytes_;
-    SG_TRY(alloc((void**)&est_rho_, ND_ * sizeof(double)));
-    SG_TRY(alloc((void**)&est_z_, ND_ * sizeof(cplx<double>)));
-    SG_TRY(alloc((void**)&est_w_, ND_ * sizeof(cplx<double>)));
+    // half spectra: the density's, and as many derivatives' as 256 MB hold
+    // (all of them up to 3D n = 7), at least two
+    const size_t hs = half_spectrum(D, n_) * sizeof(cplx<double>);
+    est_wcount_ = (int)std::max<size_t>(2, std::min<size_t>(D == 2 ? 3 : 7, ((size_t)256 << 20) / hs));
+    SG_TRY(alloc((void**)&est_z_, hs));
+    SG_TRY(alloc((void**)&est_w_, est_wcount_ * hs));
     SG_TRY(alloc((void**)&est_scalar_, 16 * sizeof(double)));
     const std::vector<cplx<double>> tw = make_twiddles<double>(n_);
     SG_TRY(alloc((void**)&tw64_, tw.size() * sizeof(cplx<double>)));
@@ -1686,17 +1672,22 @@ class Engine final : public EngineBase {
     return SG_OK;
   }
 
-  // The combination's last block also closes the step's FP64 bookkeeping
-  // (field energy, previous field energy, kinetic energy of the push when
-  // ke is given) unless finalize is false.
-  int enqueue_combine(bool finalize = true, const double* ke = nullptr) {
+  CombineFinal field_final(const double* ke) const {
     CombineFinal fin;
-    fin.active = finalize ? 1 : 0;
+    fin.active = 1;
     fin.ke_partials = ke;
     fin.n_ke = nke_;
     fin.fe_scale = fe_scale();
     fin.dd = dd_;
     fin.counter = comb_counter_;
+    return fin;
+  }
+  // The combination's last block also closes the step's FP64 bookkeeping
+  // (field energy, previous field energy, kinetic energy of the push when
+  // ke is given) unless finalize is false.
+  int enqueue_combine(bool finalize = true, const double* ke = nullptr) {
+    CombineFinal fin = field_final(ke);
+    if (!finalize) fin.active = 0;
     return launch_combine<real, D>(comb_, E_arena_, n_, Ehi_, Elo_, fe_partials_, fin,
                                    stream_, D, cfg_.cell, cfg_.combine_fp64);
   }
@@ -1711,10 +1702,8 @@ class Engine final : public EngineBase {
                                    stream_, 1, cfg_.cell, cfg_.combine_fp64);
   }
   int enqueue_regular_solve(const double* ke) {
-    SG_TRY(launch_regular_solve<real>(rho_f_, regA_, regB_, ktab_, tw_, D, n_, Ehi_, Elo_,
-                                      ec_stride<D>(), reg_partials_, reg_blocks_, stream_));
-    return launch_finalize_step(reg_partials_, reg_blocks_ * ((D + 1) / 2), ke, ke ? nke_ : 0, fe_scale(), dd_,
-                                stream_);
+    return launch_regular_solve<real>(rho_f_, regA_, regB_, ktab_, tw_, D, n_, Ehi_, ec_stride<D>(),
+                                      reg_partials_, field_final(ke), stream_);
   }
   int enqueue_filter_field(const double* ke) {
     SG_TRY(enqueue_filter_density());
@@ -1971,7 +1960,6 @@ class Engine final : public EngineBase {
   cplx<real>* regB_ = nullptr;
   real* ktab_ = nullptr;
   double* reg_partials_ = nullptr;
-  int reg_blocks_ = 0;
   int nke_ = 0, nrows_ = 0;
   // particle-pass tuner: the push grid (one resident wave, and the count in
   // use), the deposit window capacity in use, the compared timings (ms)
@@ -2021,7 +2009,9 @@ class Engine final : public EngineBase {
   std::vector<Pass> rpasses_;
   std::vector<FPass> fpasses_;
 
-  double* est_rho_ = nullptr;
+  int est_wcount_ = 0;
+  void* est_host_ = nullptr;  // pinned: the estimator's reductions
+  size_t est_host_bytes_ = 0;
   cplx<double>* est_z_ = nullptr;
   cplx<double>* est_w_ = nullptr;
   double* est_scalar_ = nullptr;

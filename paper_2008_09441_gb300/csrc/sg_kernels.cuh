@@ -203,21 +203,47 @@ struct SolveJob {
 template <typename real>
 int launch_solve_batch(const SolveJob<real>* jobs, int njobs, int max_size, int max_log, cudaStream_t s);
 
-// The filter mode's regular-grid solve: rho_f -> E on the regular nodes
-// (E_hi node-interleaved with `stride`, FP32 low planes zeroed), per-block
-// field-energy partials at partials[pair * blocks + block] (ceil(dim/2) pairs).
-// rho_f is the combination of the component densities, a deviation from the
-// mean like them.
-template <typename real>
-int launch_regular_solve(const real* rho_f, cplx<real>* A, cplx<real>* B, const real* ktab,
-                         const cplx<real>* tw, int dim, int n, real* Ehi, float* Elo, int stride, double* partials,
-                         int blocks, cudaStream_t s);
+// Device diagnostics record updated at the end of each step.
+struct DevDiag {
+  double field_energy;
+  double field_energy_prev;
+  double kinetic_energy;
+  unsigned long long checksum;
+  unsigned status;
+  unsigned pad;
+};
 
-// Generic in-place complex FFT of a whole N^D array (regular grid) along one
-// axis, forward or inverse (unnormalised), in the given precision.
+// Step bookkeeping closed by the last block of the kernel that writes the field:
+// field energy from the per-row partials (scaled by fe_scale), the previous
+// field energy, and the kinetic energy from the push partials when given.
+struct CombineFinal {
+  int active;
+  int n_ke;
+  const double* ke_partials;
+  double fe_scale;
+  DevDiag* dd;
+  unsigned* counter;  // zero between launches; the last block resets it
+};
+
+// ---------------------------------------------------------------- regular-grid spectral work
+// Complex values of a half spectrum (k_x = 0 .. N/2) of the regular grid.
+size_t half_spectrum(int dim, int n);
+// The filter mode's regular-grid solve: rho_f -> E on the regular nodes
+// (E_hi node-interleaved with `stride`), closing the step's FP64 bookkeeping as `fin` says.  rho_f is the combination of the
+// component densities, a deviation from the mean like them.  Z and W hold
+// one and `dim` half spectra, partials 3/2 2^(n (dim - 1)) values.
 template <typename real>
-int launch_fft_array_axis(cplx<real>* data, int D, int logn, int axis, bool inverse,
-                          const cplx<real>* tw, int log_nmax, cudaStream_t s);
+int launch_regular_solve(const real* rho_f, cplx<real>* Z, cplx<real>* W, const real* ktab, const cplx<real>* tw,
+                         int dim, int n, real* Ehi, int stride, double* partials, const CombineFinal& fin,
+                         cudaStream_t s);
+// Algorithm 1's reductions (FP64) of the density rho: out[q] of each mask q (bit m:
+// the factor k_m^2), with the spectrum thresholded at frac max|rho^|: the
+// largest |value| of the inverse transform (paper) or of the modes; out[8] =
+// max|rho|.  out holds 10 values; Z one half spectrum, W wcount of them.
+template <typename real>
+int launch_estimator(const real* rho, cplx<double>* Z, cplx<double>* W, int wcount, int dim, int n,
+                     const double* kfac, double frac, const int* masks, int nmask, bool paper,
+                     const cplx<double>* tw, double* out, cudaStream_t s);
 
 // ---------------------------------------------------------------- combine
 // Place of node x of a level-l line in the arrays the line kernel reads (2D:
@@ -309,19 +335,6 @@ template <typename real, int D>
 int launch_wrap_check(const PArrays<real, D>& p, size_t np, unsigned* status, cudaStream_t s);
 
 
-// Device diagnostics record updated at the end of each step.
-struct DevDiag {
-  double field_energy;
-  double field_energy_prev;
-  double kinetic_energy;
-  unsigned long long checksum;
-  unsigned status;
-  unsigned pad;
-};
-
-int launch_finalize_step(const double* fe_partials, int n_fe, const double* ke_partials, int n_ke,
-                         double fe_scale, DevDiag* dd, cudaStream_t s);
-
 // The diagnostics record in one buffer, for one device-to-host copy: *dd at
 // 0, *cks at o_cks, *st at o_cks + 8, and V_i sum_k rho_i(x_k) of every grid
 // (FP64) from o_ch on (one block per grid).
@@ -330,17 +343,35 @@ int launch_diag_record(const GridDesc* grids, int ngrids, const real* rho, const
                        const unsigned long long* cks, const unsigned* st, void* out, size_t o_cks, size_t o_ch,
                        cudaStream_t s);
 
-// Step bookkeeping closed by the last block of the combination kernel:
-// field energy from the per-row partials (scaled by fe_scale), the previous
-// field energy, and the kinetic energy from the push partials when given.
-struct CombineFinal {
-  int active;
-  int n_ke;
-  const double* ke_partials;
-  double fe_scale;
-  DevDiag* dd;
-  unsigned* counter;  // zero between launches; the last block resets it
-};
+// The last block of a field kernel to finish reduces the energy partials (and the push's kinetic-energy partials) in FP64, in a
+// fixed order, so the step needs no separate bookkeeping launch.
+__device__ __forceinline__ void combine_finalize(const double* partials, int n_part, const CombineFinal& fin,
+                                                 double* red) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(fin.counter, 1u);
+    s_last = (t == gridDim.x - 1);
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double a = 0.0;
+  for (int i = threadIdx.x; i < n_part; i += blockDim.x) a += __ldcg(partials + i);
+  const double fe = block_sum_double(a, red);
+  double b = 0.0;
+  if (fin.ke_partials)
+    for (int i = threadIdx.x; i < fin.n_ke; i += blockDim.x) b += __ldcg(fin.ke_partials + i);
+  const double ke = block_sum_double(b, red);
+  if (threadIdx.x == 0) {
+    DevDiag* dd = fin.dd;
+    dd->field_energy_prev = dd->field_energy;
+    dd->field_energy = fe * fin.fe_scale;
+    if (fin.ke_partials) dd->kinetic_energy = ke;
+    *fin.counter = 0u;
+  }
+}
 
 // E: the component fields, node-interleaved (ncomp = D, ec_stride values per
 // node), or a density (ncomp = 1); Ehi likewise.
@@ -356,16 +387,5 @@ int launch_to_double(const real* src, double* dst, size_t n, cudaStream_t s);
 template <typename real>
 int launch_field_to_double(const real* hi, const float* lo, double* dst, size_t nd, int dim, int stride,
                            cudaStream_t s);
-
-// ---------------------------------------------------------------- tau estimator
-int launch_real_to_cplx(const double* src, cplx<double>* dst, size_t n, double scale, cudaStream_t s);
-int launch_maxabs_cplx(const cplx<double>* z, size_t n, double* out_max, cudaStream_t s);
-int launch_maxabs_real_part(const cplx<double>* z, size_t n, double* out_max, cudaStream_t s);
-int launch_maxabs_real(const double* x, size_t n, double* out_max, cudaStream_t s);
-int launch_threshold(cplx<double>* z, size_t n, const double* maxabs, double frac, cudaStream_t s);
-int launch_kmult(const cplx<double>* src, cplx<double>* dst, int D, int logn, const double* kfac,
-                 int mask, cudaStream_t s);
-int launch_maxabs_kmult(const cplx<double>* src, int D, int logn, const double* kfac, int mask,
-                        double* out_max, cudaStream_t s);
 
 }  // namespace sg
