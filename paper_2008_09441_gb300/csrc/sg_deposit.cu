@@ -68,7 +68,7 @@ __device__ __forceinline__ void cell_frac(double s, int mask, int& c, double& f)
 
 // ---------------------------------------------------------------- deposit
 //
-// Persistent blocks walk chunks of DEP_CHUNK consecutive particles
+// Persistent blocks walk chunks of 4 THREADS (DEP_CHUNK, or a quarter) consecutive particles
 // (consecutive in tile-key order after a sort, so a chunk covers a compact
 // group of cells).  Per chunk every thread reads the chunk's middle particle
 // and takes its cell as the anchor of a fixed window of side^d regular nodes
@@ -86,11 +86,12 @@ __device__ __forceinline__ void cell_frac(double s, int mask, int& c, double& f)
 // FP32: WinAcc fixed point with the run's scale 2^(20 - E), max_p |q_p|/V <=
 // 2^E (1 - 2^-11) (set at upload; charges do not change), so a window of at
 // most 2^11 particles cannot overflow.  FP64: plain double, scale 1.
-template <typename real, int D>
-__global__ void __launch_bounds__(DEP_THREADS) k_deposit(PArrays<real, D> p, size_t np, int n,
+template <typename real, int D, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_deposit(PArrays<real, D> p, size_t np, int n,
                                                          real inv_cell_vol, real* __restrict__ rho, int side,
                                                          real scale, real inv_scale, real shift) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int CHUNK = THREADS * DEP_ITEMS;
   using W = WinAcc<real>;
   using T = typename W::T;
   T* win = reinterpret_cast<T*>(smem_raw);
@@ -106,21 +107,28 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(PArrays<real, D> p, siz
   {
     uint4* w4 = reinterpret_cast<uint4*>(smem_raw);
     const int n4 = (int)((nwin * sizeof(T) + 15) / 16);
-    for (int i = threadIdx.x; i < n4; i += DEP_THREADS) w4[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < n4; i += THREADS) w4[i] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x < 2 * D) {
       s_box[0][threadIdx.x] = threadIdx.x < D ? INT_MAX : INT_MIN;
       s_box[1][threadIdx.x] = threadIdx.x < D ? INT_MAX : INT_MIN;
     }
   }
-  const size_t nchunks = (np + DEP_CHUNK - 1) / DEP_CHUNK;
+  const size_t nchunks = (np + CHUNK - 1) / CHUNK;
   int par = 0;
   for (size_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x, par ^= 1) {
-    const size_t chunk = ch * DEP_CHUNK;
+    const size_t chunk = ch * CHUNK;
     // ---- this thread's particles: DEP_ITEMS / 4 vectors of four
     real ub[DEP_ITEMS][D], qb[DEP_ITEMS];
 #pragma unroll
     for (int j = 0; j < DEP_ITEMS / 4; ++j) {
-      const size_t i0 = chunk + ((size_t)j * DEP_THREADS + threadIdx.x) * 4;
+      // Which four particles.  FP32: consecutive threads, consecutive vectors
+      // (equal addresses of a warp's integer adds are merged; spreading them
+      // cost 40%).  FP64: the shared double add is a compare-and-swap loop
+      // that repeats once per lane on the same node, so the lanes of a warp
+      // take particles THREADS / 8 apart, in other cells (2D n = 6, 16
+      // particles per cell: 20.4 -> 18.5 us).
+      const int vec = sizeof(real) == 8 ? lane * (THREADS / 32) + (int)(threadIdx.x >> 5) : (int)threadIdx.x;
+      const size_t i0 = chunk + ((size_t)j * THREADS + vec) * 4;
       if (i0 + 4 <= np) {
 #pragma unroll
         for (int m = 0; m < D; ++m) {
@@ -144,7 +152,7 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(PArrays<real, D> p, siz
     // ---- anchor: the cell of the chunk's middle (or last) particle, read by every thread
     int anchor[D];
     {
-      size_t mid = chunk + DEP_CHUNK / 2;
+      size_t mid = chunk + CHUNK / 2;
       if (mid >= np) mid = np - 1;
 #pragma unroll
       for (int m = 0; m < D; ++m) anchor[m] = cell_of(__ldg(p.u[m] + mid), n, N);
@@ -254,7 +262,7 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(PArrays<real, D> p, siz
       const int x0 = W::fixed ? (blo[0] & ~3) : blo[0];
       const int nx = (bhi[0] - x0) / PER + 1;
       const int total = nrows * nx;
-      for (int f = threadIdx.x; f < total; f += DEP_THREADS) {
+      for (int f = threadIdx.x; f < total; f += THREADS) {
         const int r = f / nx;
         const int x = x0 + (f - r * nx) * PER;
         const int ly = blo[1 % D] + (D == 2 ? r : r % ny);
@@ -284,6 +292,40 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(PArrays<real, D> p, siz
   }
 }
 
+template <typename real, int D, int THREADS>
+static int launch_deposit_threads(const PArrays<real, D>& p, size_t np, int n, real inv_cell_vol, real* rho, int side,
+                                  size_t smem, int sms, real scale, real inv_scale, real shift, cudaStream_t s) {
+  // resident blocks per SM for each window size met so far (the autotuner
+  // tries several capacities; the answer depends on the window's bytes)
+  static bool attr_set = false;
+  static size_t known_smem[8];
+  static int known_per_sm[8];
+  static int nknown = 0;
+  if (!attr_set) {
+    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    attr_set = true;
+  }
+  int per_sm = 0;
+  for (int i = 0; i < nknown; ++i)
+    if (known_smem[i] == smem) per_sm = known_per_sm[i];
+  if (!per_sm) {
+    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_deposit<real, D, THREADS>, THREADS, smem));
+    if (per_sm < 1) per_sm = 1;
+    if (nknown < 8) {
+      known_smem[nknown] = smem;
+      known_per_sm[nknown] = per_sm;
+      ++nknown;
+    }
+  }
+  constexpr int CHUNK = THREADS * DEP_ITEMS;
+  const size_t nchunks = (np + CHUNK - 1) / CHUNK;
+  const unsigned blocks = (unsigned)std::min<size_t>(nchunks, (size_t)sms * per_sm);
+  k_deposit<real, D, THREADS><<<blocks, THREADS, smem, s>>>(p, np, n, inv_cell_vol, rho, side, scale, inv_scale, shift);
+  SG_CHECK_LAUNCH();
+  return SG_OK;
+}
+
 template <typename real, int D>
 int launch_deposit(const PArrays<real, D>& p, size_t np, int n, real inv_cell_vol, real* rho, int win_cap_nodes,
                    real scale, real inv_scale, real shift, cudaStream_t s) {
@@ -308,40 +350,21 @@ int launch_deposit(const PArrays<real, D>& p, size_t np, int n, real inv_cell_vo
     set_error("deposit: window capacity above 200 KB of shared memory");
     return SG_ERR_UNSUPPORTED;
   }
-  // resident blocks per SM for each window size met so far (the autotuner
-  // tries several capacities; the answer depends on the window's bytes)
-  static bool attr_set = false;
-  static size_t known_smem[8];
-  static int known_per_sm[8];
-  static int nknown = 0;
-  if (!attr_set) {
-    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    attr_set = true;
-  }
-  int per_sm = 0;
-  for (int i = 0; i < nknown; ++i)
-    if (known_smem[i] == smem) per_sm = known_per_sm[i];
-  if (!per_sm) {
-    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_deposit<real, D>, DEP_THREADS, smem));
-    if (per_sm < 1) per_sm = 1;
-    if (nknown < 8) {
-      known_smem[nknown] = smem;
-      known_per_sm[nknown] = per_sm;
-      ++nknown;
-    }
-  }
   static int sms = 0;
   if (!sms) {
     int dev = 0;
     SG_CUDA(cudaGetDevice(&dev));
     SG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   }
-  const size_t nchunks = (np + DEP_CHUNK - 1) / DEP_CHUNK;
-  const unsigned blocks = (unsigned)std::min<size_t>(nchunks, (size_t)sms * per_sm);
-  k_deposit<real, D><<<blocks, DEP_THREADS, smem, s>>>(p, np, n, inv_cell_vol, rho, side, scale, inv_scale, shift);
-  SG_CHECK_LAUNCH();
-  return SG_OK;
+  // Fewer than two chunks per SM: blocks and chunks a quarter the size, so
+  // that every SM gets some (us, FP64 2D n = 6, 65,536 particles 36.6 -> 20.4,
+  // 3D n = 5 56.5 -> 28.3; FP32 3D n = 5, 100,003 particles 13.2 -> 11.6, 2D
+  // n = 6 10.6 -> 8.8; no change from 500,000 particles on).
+  if ((np + DEP_CHUNK - 1) / DEP_CHUNK < (size_t)2 * sms)
+    return launch_deposit_threads<real, D, DEP_THREADS / 4>(p, np, n, inv_cell_vol, rho, side, smem, sms, scale,
+                                                            inv_scale, shift, s);
+  return launch_deposit_threads<real, D, DEP_THREADS>(p, np, n, inv_cell_vol, rho, side, smem, sms, scale, inv_scale,
+                                                      shift, s);
 }
 
 // ---------------------------------------------------------------- restriction

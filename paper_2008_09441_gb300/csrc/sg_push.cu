@@ -13,7 +13,8 @@
 namespace sg {
 
 static __device__ __forceinline__ bool finite_r(float x) { return isfinite(x); }
-static __device__ __forceinline__ bool finite_r(double x) { return isfinite(x); }
+// by the exponent bits: a comparison would take the slow double pipe
+static __device__ __forceinline__ bool finite_r(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
 
 
 // Kinetic-energy accumulator of one thread: FP32 path a float pair whose
@@ -58,8 +59,12 @@ __device__ __forceinline__ void gather_cell(double s, int mask, int& c, double& 
 // Periodic wrap of a drifted position: u - floor(u), a rounded-up 1 mapped
 // to 0.  A drift of less than one box per step needs only a compare and an
 // add of +-1 (the same operation floor would select); larger ones take floor.
+// Doubles inside [0, 1) are recognised by their high word (integer compare).
 template <typename real>
 __device__ __forceinline__ real wrap_drifted(real u) {
+  if constexpr (sizeof(real) == 8) {
+    if ((unsigned)__double2hiint(u) < 0x3FF00000u) return u;
+  }
   real w = u < (real)0 ? u + (real)1 : (u >= (real)1 ? u - (real)1 : u);
   if (w < (real)0 || w >= (real)1) w = u - sg_floor(u);
   return w >= (real)1 ? (real)0 : w;
@@ -262,17 +267,27 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? (D == 2 ? 4 : 2) : 0)
   if (threadIdx.x == 0 && ke_partials) ke_partials[blockIdx.x] = tot;
 }
 
+// Threads per block.  The double pipe is the FP64 push's bound, so a small
+// FP64 run takes small blocks to reach every SM's (65,536 particles: 23.8 ->
+// 17.5 us in 2D, 35.3 -> 24.0 in 3D).  FP32 keeps 256: its push gains nothing
+// and the larger number of partial sums costs the step 2 us.
+template <typename real>
+static int push_threads(size_t np) {
+  return sizeof(real) == 8 && np / 4 / 256 < (size_t)4 * 152 ? 64 : 256;
+}
 // Blocks of the push: one resident wave (SMs x blocks per SM at the kernel's
 // register budget), each block walking its particles grid-stride; fewer for
 // small runs.  A second wave of blocks measured 7% slower on the 2D step.
 template <typename real, int D>
 int push_blocks(size_t np) {
-  static int cap = 0;
+  static int caps[2] = {0, 0};
+  const int threads = push_threads<real>(np);
+  int& cap = caps[threads == 256];
   if (!cap) {
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push<real, D>, 256, 0) == cudaSuccess &&
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_push<real, D>, threads, 0) == cudaSuccess &&
         sms > 0 && per_sm > 0) {
       cap = sms * per_sm;
     } else {
@@ -280,7 +295,7 @@ int push_blocks(size_t np) {
       cap = 152 * 4;
     }
   }
-  size_t b = (np / 4 + 255) / 256;
+  size_t b = (np / 4 + threads - 1) / threads;
   if (b > (size_t)cap) b = (size_t)cap;
   if (b == 0) b = 1;
   return (int)b;
@@ -290,10 +305,11 @@ template <typename real, int D>
 int launch_push(const PArrays<real, D>& p, size_t np, int n, const real* Ecomb, PushParams<real> pp,
                 double* ke_partials, unsigned* status, const SortFuse& sf, cudaStream_t s, int blocks) {
   if (blocks <= 0) blocks = push_blocks<real, D>(np);
+  const int threads = push_threads<real>(np);
   if (sf.keys)  // sort steps: memsets precede the push
-    k_push<real, D><<<blocks, 256, 0, s>>>(p, np, n, Ecomb, pp, ke_partials, status, sf);
+    k_push<real, D><<<blocks, threads, 0, s>>>(p, np, n, Ecomb, pp, ke_partials, status, sf);
   else
-    SG_CUDA(launch_pdl(k_push<real, D>, dim3(blocks), dim3(256), 0, s, p, np, n, Ecomb, pp, ke_partials, status, sf));
+    SG_CUDA(launch_pdl(k_push<real, D>, dim3(blocks), dim3(threads), 0, s, p, np, n, Ecomb, pp, ke_partials, status, sf));
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
