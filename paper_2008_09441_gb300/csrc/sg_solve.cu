@@ -169,55 +169,71 @@ int launch_fft_pass(int kind, const SolveArena<real>& a, const FftJob* jobs_dev,
 
 // ---------------------------------------------------------------- one block per grid
 //
-// When every component grid fits in shared memory (twice: spectrum and one
-// field component), one launch solves all of them: a block loads its grid,
-// transforms it along every axis in place (bit-reversal swap, then the
-// butterfly stages), forms each E^_m and transforms it back.
-template <typename real>
-__device__ void fft_axis_inplace(cplx<real>* buf, const int* logs, int S, int ax, bool inverse,
-                                 const cplx<real>* __restrict__ tw) {
-  const int logn = logs[ax];
-  const int len = 1 << logn;
-  int ls = 0;
-  for (int m = 0; m < ax; ++m) ls += logs[m];
+// When every component grid fits in shared memory (twice in 3D: spectrum and
+// one pair of field components), one launch solves all of them: a block loads
+// its grid, transforms it along every axis in place, forms the E^_m and
+// transforms them back.  Forward transforms decimate in frequency (natural
+// order in, bit-reversed out) and inverse ones in time (bit-reversed in,
+// natural out), so no pass reorders anything: the spectral step reads the
+// frequency of a position by reversing its bits.  Both take their stages in
+// pairs (radix 2^2), half the passes over shared memory and barriers.
+// Bound: latency (one block per grid, one barrier per pass).  With
+// profiling events, with single stages and bit-reversal passes -> now: 2D
+// n = 10 18.4 -> 12.3 us, n = 8 10.2 -> 8.2, 3D n = 7 14.3 -> 10.3.  Half a
+// grid of threads: a quarter took 12.3 us in 3D, the same in 2D.
+//
+// Element (o, t, i) of axis ax at ((o << logn) + t) << ls | i; consecutive
+// work items take consecutive inner indices i (the axes below ax, contiguous
+// in the buffer), then the butterflies of one line, then the outer lines, so
+// that a warp's accesses are contiguous along every axis.
+template <typename real, bool INV>
+__device__ __forceinline__ void fft_axis(cplx<real>* buf, int S, int logn, int ls, const cplx<real>* __restrict__ tw) {
   const int smask = (1 << ls) - 1;
-  for (int e = threadIdx.x; e < S; e += blockDim.x) {
-    const int t = (e >> ls) & (len - 1);
-    const int r = bitrev(t, logn);
-    if (r > t) {
-      const int e2 = e + ((r - t) << ls);
-      cplx<real> x = buf[e];
-      buf[e] = buf[e2];
-      buf[e2] = x;
-    }
-  }
-  __syncthreads();
-  const int halfN = len >> 1;
-  // Butterfly j of a stage: consecutive j take consecutive inner indices
-  // (the axes below ax, contiguous in the buffer), then the butterflies of
-  // one line, then the outer lines, so that a warp's accesses are
-  // contiguous along every axis (the line itself strides by 2^ls).
-  for (int s = 1; s <= logn; ++s) {
-    const int half = 1 << (s - 1);
+  auto radix2 = [&]() {  // span 2, no twiddle
     for (int j = threadIdx.x; j < (S >> 1); j += blockDim.x) {
-      const int i = j & smask;
-      const int p = (j >> ls) & (halfN - 1);
-      const int o = j >> (ls + logn - 1);
-      const int pos = p & (half - 1);
-      const int grp = p >> (s - 1);
-      const int t0 = grp * 2 * half + pos;
-      const int i0 = (((o << logn) + t0) << ls) + i;
-      const int i1 = i0 + (half << ls);
-      cplx<real> w = tw[twiddle_index(half, pos)];
-      if (inverse) w.y = -w.y;
-      const cplx<real> x0 = buf[i0], x1 = buf[i1];
-      const real bx = x1.x * w.x - x1.y * w.y;
-      const real by = x1.x * w.y + x1.y * w.x;
-      buf[i0] = {x0.x + bx, x0.y + by};
-      buf[i1] = {x0.x - bx, x0.y - by};
+      const int i0 = ((j >> ls) << (ls + 1)) + (j & smask), i1 = i0 + (1 << ls);
+      const cplx<real> a = buf[i0], b = buf[i1];
+      buf[i0] = {a.x + b.x, a.y + b.y};
+      buf[i1] = {a.x - b.x, a.y - b.y};
+    }
+    __syncthreads();
+  };
+  if (INV && (logn & 1)) radix2();
+  for (int k = INV ? (logn & 1) : logn - 2; INV ? k + 1 < logn : k >= 0; k += INV ? 2 : -2) {
+    const int q = 1 << k, st = q << ls;  // elements t, t + q, t + 2q, t + 3q
+    for (int j = threadIdx.x; j < (S >> 2); j += blockDim.x) {
+      const int p = j >> ls;  // butterfly: (outer, group, position)
+      const int pos = p & (q - 1);
+      const int i0 = ((((p >> k) << (k + 2)) + pos) << ls) + (j & smask);
+      cplx<real> w1 = tw[twiddle_index(q, pos)], w2 = tw[twiddle_index(2 * q, pos)];  // W_{2q}^pos, W_{4q}^pos
+      const cplx<real> a0 = buf[i0], a1 = buf[i0 + st], a2 = buf[i0 + 2 * st], a3 = buf[i0 + 3 * st];
+      cplx<real> x0, x1, x2, x3;
+      if constexpr (INV) {
+        w1.y = -w1.y;
+        w2.y = -w2.y;
+        const cplx<real> w3 = {-w2.y, w2.x};  // W_{4q}^(pos + q), conjugated
+        cplx<real> b0, b1, b2, b3;
+        butterfly(a0, a1, w1, b0, b1);
+        butterfly(a2, a3, w1, b2, b3);
+        butterfly(b0, b2, w2, x0, x2);
+        butterfly(b1, b3, w3, x1, x3);
+      } else {
+        const cplx<real> w3 = {w2.y, -w2.x};  // W_{4q}^(pos + q)
+        const cplx<real> b0 = {a0.x + a2.x, a0.y + a2.y}, b1 = {a1.x + a3.x, a1.y + a3.y};
+        const cplx<real> b2 = cmul<real>({a0.x - a2.x, a0.y - a2.y}, w2), b3 = cmul<real>({a1.x - a3.x, a1.y - a3.y}, w3);
+        x0 = {b0.x + b1.x, b0.y + b1.y};
+        x1 = cmul<real>({b0.x - b1.x, b0.y - b1.y}, w1);
+        x2 = {b2.x + b3.x, b2.y + b3.y};
+        x3 = cmul<real>({b2.x - b3.x, b2.y - b3.y}, w1);
+      }
+      buf[i0] = x0;
+      buf[i0 + st] = x1;
+      buf[i0 + 2 * st] = x2;
+      buf[i0 + 3 * st] = x3;
     }
     __syncthreads();
   }
+  if (!INV && (logn & 1)) radix2();
 }
 
 // One block solves grid gi of arena a: load, forward transforms, E^_m,
@@ -227,32 +243,37 @@ __device__ __forceinline__ void solve_grid_block(const SolveArena<real>& a, int 
   extern __shared__ unsigned char smem_raw[];
   const GridDesc g = a.grids[gi];
   const int D = a.dim;
-  int logs[3] = {0, 0, 0};
-  for (int m = 0; m < D; ++m) logs[m] = g.l[m];
+  const int l0 = g.l[0], l1 = g.l[1], l2 = D == 3 ? g.l[2] : 0;
   const int S = g.size;
   cplx<real>* A = reinterpret_cast<cplx<real>*>(smem_raw);
-  cplx<real>* B = A + max_size;
-  cplx<real>* tws = B + max_size;  // twiddle table staged in shared memory
-  const int ntw = twiddle_count(a.log_nmax);
+  cplx<real>* tws = A + (size_t)(D == 3 ? 2 : 1) * max_size;  // twiddles of the grid's longest axis
+  const int ntw = twiddle_count(max(l0, max(l1, l2)));
   for (int e = threadIdx.x; e < ntw; e += blockDim.x) tws[e] = a.tw[e];
+  pdl_wait();  // the component densities
   for (int e = threadIdx.x; e < S; e += blockDim.x) A[e] = {a.rho[g.offset + e], (real)0};
   __syncthreads();
-  for (int ax = 0; ax < D; ++ax) fft_axis_inplace<real>(A, logs, S, ax, false, tws);
+  fft_axis<real, false>(A, S, l0, 0, tws);
+  fft_axis<real, false>(A, S, l1, l0, tws);
+  if (D == 3) fft_axis<real, false>(A, S, l2, l0 + l1, tws);
   const real norm = (real)1 / (real)S;
-  const int n0 = 1 << logs[0], n1 = 1 << logs[1];
+  const int n0 = 1 << l0, n1 = 1 << l1;
   // Field components in pairs: B = E^_a + i E^_b, one inverse transform,
   // E_a its real part and E_b its imaginary part (both fields are real).
-  for (int pr = 0; 2 * pr < D; ++pr) {
+  // The last pair takes the spectrum's place.
+  const int np = (D + 1) / 2;
+  for (int pr = 0; pr < np; ++pr) {
     const int ma = 2 * pr, mb = 2 * pr + 1;
+    cplx<real>* B = pr == np - 1 ? A : A + max_size;
     for (int e = threadIdx.x; e < S; e += blockDim.x) {
-      int idx[3];
-      idx[0] = e & (n0 - 1);
-      idx[1] = (e >> logs[0]) & (n1 - 1);
-      idx[2] = D == 3 ? (e >> (logs[0] + logs[1])) : 0;
+      const int idx[3] = {bitrev(e & (n0 - 1), l0), bitrev((e >> l0) & (n1 - 1), l1),
+                          D == 3 ? bitrev(e >> (l0 + l1), l2) : 0};
+      const int sizes[3] = {n0, n1, 1 << l2};
       real k2 = 0, ka = 0, kb = 0;
       bool nyq_a = false, nyq_b = false;
-      for (int q = 0; q < D; ++q) {
-        const int Nq = 1 << logs[q];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (q >= D) break;
+        const int Nq = sizes[q];
         const real kq = (real)g.kfac[q] * (real)sfreq(idx[q], Nq);
         k2 += kq * kq;
         if (q == ma) {
@@ -282,18 +303,31 @@ __device__ __forceinline__ void solve_grid_block(const SolveArena<real>& a, int 
       B[e] = out;
     }
     __syncthreads();
-    for (int ax = 0; ax < D; ++ax) fft_axis_inplace<real>(B, logs, S, ax, true, tws);
+    if (D == 3) fft_axis<real, true>(B, S, l2, l0 + l1, tws);
+    fft_axis<real, true>(B, S, l1, l0, tws);
+    fft_axis<real, true>(B, S, l0, 0, tws);
     for (int e = threadIdx.x; e < S; e += blockDim.x) {
       const int x = e & (n0 - 1);
-      const int at = D == 2 ? e - x + line_pos(x, logs[0], a.log_nmax) : e;
-      reinterpret_cast<cplx<real>*>(a.E)[(size_t)(g.offset + at) * ((D + 1) / 2) + pr] = {B[e].x, mb < D ? B[e].y : (real)0};
+      const int at = D == 2 ? e - x + line_pos(x, l0, a.log_nmax) : e;
+      reinterpret_cast<cplx<real>*>(a.E)[(size_t)(g.offset + at) * np + pr] = {B[e].x, mb < D ? B[e].y : (real)0};
     }
     __syncthreads();
   }
 }
 
+// Shared memory and threads of the one-block solve.
+template <typename real>
+static size_t solve_block_smem(int dim, int max_size, int max_log) {
+  return ((size_t)(dim == 3 ? 2 : 1) * max_size + (size_t)twiddle_count(max_log)) * sizeof(cplx<real>);
+}
+static int solve_block_threads(int max_size) {
+  const int t = max_size / 2;
+  return t < 64 ? 64 : (t > 1024 ? 1024 : t);
+}
+
 template <typename real>
 __global__ void __launch_bounds__(1024) k_solve_small(SolveArena<real> a, int max_size, int grid0) {
+  pdl_trigger();
   solve_grid_block<real>(a, grid0 + blockIdx.x, max_size);
 }
 
@@ -308,15 +342,14 @@ __global__ void __launch_bounds__(1024) k_solve_batch(const SolveJob<real>* __re
 template <typename real>
 int launch_solve_small(const SolveArena<real>& a, int ngrids, int max_size, cudaStream_t s, int grid0) {
   if (ngrids == 0) return SG_OK;
-  int threads = max_size / 2;
-  threads = threads < 64 ? 64 : (threads > 1024 ? 1024 : threads);
-  size_t smem = ((size_t)2 * max_size + (size_t)twiddle_count(a.log_nmax)) * sizeof(cplx<real>);
+  const int threads = solve_block_threads(max_size);
+  const size_t smem = solve_block_smem<real>(a.dim, max_size, a.log_nmax);
   static bool attr_set = false;
   if (!attr_set) {
     SG_CUDA(cudaFuncSetAttribute(k_solve_small<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     attr_set = true;
   }
-  k_solve_small<real><<<ngrids, threads, smem, s>>>(a, max_size, grid0);
+  SG_CUDA(launch_pdl(k_solve_small<real>, dim3(ngrids), dim3(threads), smem, s, a, max_size, grid0));
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
@@ -331,9 +364,8 @@ int launch_solve_batch(const SolveJob<real>* jobs, int njobs, int max_size, int 
     set_error("cross-run solve: a component grid is larger than one block's shared memory takes");
     return SG_ERR_UNSUPPORTED;
   }
-  int threads = max_size / 2;
-  threads = threads < 64 ? 64 : (threads > 1024 ? 1024 : threads);
-  const size_t smem = ((size_t)2 * max_size + (size_t)twiddle_count(max_log)) * sizeof(cplx<real>);
+  const int threads = solve_block_threads(max_size);
+  const size_t smem = solve_block_smem<real>(3, max_size, max_log);  // runs of either dimension
   static bool attr_set = false;
   if (!attr_set) {
     SG_CUDA(cudaFuncSetAttribute(k_solve_batch<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
