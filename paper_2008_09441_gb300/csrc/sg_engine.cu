@@ -1172,7 +1172,9 @@ class Engine final : public EngineBase {
     int S = N_ + ((N_ >> 5) << 2);  // tile row: 4 padding words per 32, = 4 (mod 32)
     S = (S + 3) & ~3;
     while ((S & 31) != 4) S += 4;
-    for (int a = 0; a < D; ++a) {
+    int first = 0;
+    SG_TRY(build_restrict_planes(&prev, &first));
+    for (int a = first; a < D; ++a) {
       std::map<std::vector<int>, std::set<int>> targets;  // prefix -> levels along axis a
       for (auto& g : grids_) {
         std::vector<int> pre(g.l, g.l + a);
@@ -1256,6 +1258,42 @@ class Engine final : public EngineBase {
       rpasses_.push_back(P);
       prev.swap(next);
     }
+    return SG_OK;
+  }
+  // 3D runs whose plane (with its x levels and carries) fits shared memory --
+  // FP32 node-centred up to n = 7, cell-centred and FP64 n = 6 -- restrict x
+  // and y in one launch; *first is then the z axis and *prev its sources.
+  // With profiling events, all passes: see k_restrict_planes.
+  int build_restrict_planes(std::map<std::vector<int>, real*>* prev, int* first) {
+    restrict_planes_ = nullptr;
+    if (D != 3) return SG_OK;
+    PlaneTargets t;
+    std::memset(&t, 0, sizeof(t));
+    t.lx_min = t.ly_min = n_;
+    for (auto& g : grids_) {
+      t.lx_min = std::min(t.lx_min, g.l[0]);
+      t.ly_min = std::min(t.ly_min, g.l[1]);
+    }
+    if (t.lx_min == n_ && t.ly_min == n_) return SG_OK;  // tau = n: nothing to restrict in the plane
+    if (restrict_planes_smem<real>(n_, t.lx_min, cfg_.cell) > (size_t)RJ_PLANE_SMEM) return SG_OK;
+    std::map<std::vector<int>, real*> next;
+    for (auto& g : grids_) {
+      const std::vector<int> key{g.l[0], g.l[1]};
+      if (next.count(key)) continue;
+      if (g.l[0] == n_ && g.l[1] == n_) {  // unrestricted: the density itself
+        next[key] = rho_reg_;
+        continue;
+      }
+      real* dst = nullptr;
+      SG_TRY(galloc((void**)&dst, ((size_t)N_ << (g.l[0] + g.l[1])) * sizeof(real)));
+      next[key] = dst;
+      t.dst[g.l[0]][g.l[1]] = dst;
+    }
+    SG_TRY(galloc((void**)&restrict_planes_, sizeof(t)));
+    SG_CUDA(cudaMemcpyAsync(restrict_planes_, &t, sizeof(t), cudaMemcpyHostToDevice, stream_));
+    restrict_lx_min_ = t.lx_min;
+    prev->swap(next);
+    *first = 2;
     return SG_OK;
   }
   int find_grid(const std::vector<int>& l) {
@@ -1424,6 +1462,9 @@ class Engine final : public EngineBase {
   }
 
   int enqueue_restrict() {
+    if (restrict_planes_)
+      SG_TRY(launch_restrict_planes<real>(rho_reg_, restrict_planes_, n_, restrict_lx_min_, cfg_.cell, rho_mean(),
+                                          stream_));
     for (auto& P : rpasses_)
       SG_TRY(launch_restrict_pass<real>(P.dev, P.njobs, P.nblocks, P.lpb, P.vpl, P.smem, cfg_.cell, rho_mean(),
                                         stream_));
@@ -2006,6 +2047,8 @@ class Engine final : public EngineBase {
   cplx<real>* A_ = nullptr;
   cplx<real>* B_ = nullptr;
   real* E_arena_ = nullptr;
+  PlaneTargets* restrict_planes_ = nullptr;  // 3D: x and y in one launch
+  int restrict_lx_min_ = 0;
   std::vector<Pass> rpasses_;
   std::vector<FPass> fpasses_;
 

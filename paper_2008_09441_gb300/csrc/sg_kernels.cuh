@@ -130,6 +130,21 @@ template <typename real>
 int launch_restrict_pass(const LineJob* jobs_dev, int njobs, int nblocks, int lines_per_block, int vpl,
                          int smem_bytes, bool cell, real mean, cudaStream_t s);
 
+// 3D: x and y restricted plane by plane in one launch.  dst[l_1][l_2]: the
+// array [z][2^l_2][2^l_1] of a level pair, or nullptr; lx_min / ly_min: the
+// lowest levels needed.
+constexpr int RJ_PLANE_LEVELS = 9;  // 3D levels 0..8
+constexpr int RJ_PLANE_SMEM = 220 * 1024;
+struct PlaneTargets {
+  int lx_min, ly_min;
+  void* dst[RJ_PLANE_LEVELS][RJ_PLANE_LEVELS];
+};
+template <typename real>
+size_t restrict_planes_smem(int n, int lx_min, bool cell);
+template <typename real>
+int launch_restrict_planes(const real* rho, const PlaneTargets* tgt, int n, int lx_min, bool cell, real mean,
+                           cudaStream_t s);
+
 // FFT passes over the component grids.
 enum FftKind { FFT_FWD_FIRST = 0, FFT_FWD_MID = 1, FFT_LAST = 2, FFT_INV_MID = 3, FFT_INV_LAST = 4 };
 
