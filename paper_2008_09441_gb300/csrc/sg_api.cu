@@ -339,50 +339,10 @@ int sg_cell_sort(int precision, int dim, int level, size_t n, const void* const*
   for (int m = 0; n > 0 && m < dim; ++m)
     if (!u[m]) return invalid("sg_cell_sort: NULL position array");
   cudaStream_t s = (cudaStream_t)stream;
-  size_t cells = (size_t)1 << (dim * level);
-  if (n == 0) {
-    if (counts) SG_CUDA(cudaMemsetAsync(counts, 0, cells * 4, s));
-    return SG_OK;
-  }
-  size_t scr_words = sort_scratch_words(n);
-  size_t words = 3 * n + scr_words + 4;
+  if (n == 0) return cell_sort(precision, dim, level, 0, u, keys_sorted, perm, counts, nullptr, s);
   uint32_t* buf = nullptr;
-  SG_CUDA(cudaMallocAsync((void**)&buf, words * 4, s));
-  uint32_t* keys = buf;
-  uint32_t* vals = buf + n;
-  uint32_t* keys_alt = buf + 2 * n;
-  uint32_t* scr = buf + 3 * n;
-  unsigned* status = (unsigned*)(scr + scr_words);
-  SortScratch sc;
-  sort_scratch_bind(sc, scr, n);
-  int st = SG_OK;
-  if (precision == SG_FP32) {
-    st = dim == 2 ? launch_keys_raw<float, 2>((const float* const*)u, n, level, keys, nullptr, nullptr, status, s)
-                  : launch_keys_raw<float, 3>((const float* const*)u, n, level, keys, nullptr, nullptr, status, s);
-  } else {
-    st = dim == 2 ? launch_keys_raw<double, 2>((const double* const*)u, n, level, keys, nullptr, nullptr, status, s)
-                  : launch_keys_raw<double, 3>((const double* const*)u, n, level, keys, nullptr, nullptr, status, s);
-  }
-  bool in_alt = false;
-  // the sorted result lands in (keys, vals) or (keys_alt, perm) depending on the pass count
-  if (st == SG_OK) st = radix_sort_pairs(keys, vals, keys_alt, perm, n, dim * level, true, sc, s, &in_alt);
-  if (st == SG_OK) {
-    const uint32_t* ks = in_alt ? keys_alt : keys;
-    const uint32_t* ps = in_alt ? perm : vals;
-    if (ks != keys_sorted) {
-      cudaError_t e = cudaMemcpyAsync(keys_sorted, ks, n * 4, cudaMemcpyDeviceToDevice, s);
-      if (e != cudaSuccess) st = SG_ERR_CUDA;
-    }
-    if (st == SG_OK && ps != perm) {
-      cudaError_t e = cudaMemcpyAsync(perm, ps, n * 4, cudaMemcpyDeviceToDevice, s);
-      if (e != cudaSuccess) st = SG_ERR_CUDA;
-    }
-    if (st == SG_OK && counts) {
-      cudaError_t e = cudaMemsetAsync(counts, 0, cells * 4, s);
-      if (e != cudaSuccess) st = SG_ERR_CUDA;
-      if (st == SG_OK) st = launch_counts(keys_sorted, n, counts, s);
-    }
-  }
+  SG_CUDA(cudaMallocAsync((void**)&buf, cell_sort_words(n) * 4, s));
+  const int st = cell_sort(precision, dim, level, n, u, keys_sorted, perm, counts, buf, s);
   cudaFreeAsync(buf, s);
   return st;
 }

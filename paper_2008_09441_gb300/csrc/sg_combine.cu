@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(256) k_combine_planes(const PlanePair* __restr
     }
   }
   __syncthreads();
-  pdl_wait();  // the solve's fields
+  pdl_wait(E);  // the solve's fields
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= S2) return;
   int lo = 0, hi = npairs;  // the last pair with off <= e
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(CL_THREADS, sizeof(T) == 8 ? 2 : NC == 3 ? 3 :
     tab[e] = rt;
   }
   __syncthreads();
-  pdl_wait();  // the fields (3D: their pairs)
+  pdl_wait(G);  // the fields (3D: their pairs)
   const int ntask = lpb * MG * ipl;
   const GT* Gz = G + (size_t)((brow - row0) >> n) * zstride;  // lpb <= N: the block's lines lie in one plane
   int level = min(CELL ? lmin + 1 : lmin, n - LK);

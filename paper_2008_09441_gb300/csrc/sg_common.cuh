@@ -57,7 +57,18 @@ unsigned long long launches_so_far();
 // call pdl_wait() before touching anything the predecessor writes (the wait
 // returns once the predecessor has completed and its writes are visible).
 // pdl_trigger() lets the successor start launching early.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The same for loads through the given pointers: each is re-defined after the
+// wait.  A load the compiler takes for invariant (const __restrict__, __ldg)
+// may otherwise move up past it, whatever the wait's memory clobber says.
+template <typename P>
+__device__ __forceinline__ void pdl_renew(P& p) {
+  asm volatile("" : "+l"(p)::"memory");
+}
+template <typename... P>
+__device__ __forceinline__ void pdl_wait(P&... p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (pdl_renew(p), ...);
+}
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>

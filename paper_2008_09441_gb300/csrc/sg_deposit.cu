@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(1024) k_restrict_planes(const real* __restrict
   pdl_trigger();
   for (int i = tid; i < RJ_PLANE_LEVELS * RJ_PLANE_LEVELS; i += nt)
     (&dst[0][0])[i] = static_cast<real*>((&tgt->dst[0][0])[i]);
-  pdl_wait();
+  pdl_wait(rho);
   const real* src = rho + ((size_t)z << (2 * n));
   for (int e = 4 * tid; e < N * N; e += 4 * nt) {  // N >= 4: whole vectors of a row
     const V4<real> t = ld4(src + e);

@@ -637,7 +637,7 @@ class Engine final : public EngineBase {
       uint32_t* dcounts = nullptr;
       SG_TRY(alloc((void**)&dcounts, ND_ * 4));
       SG_CUDA(cudaMemsetAsync(dcounts, 0, ND_ * 4, stream_));
-      SG_TRY(launch_counts(keys_alt_, np_, dcounts, stream_));
+      SG_TRY(launch_counts(keys_alt_, np_, dcounts, stream_, false));
       SG_CUDA(cudaMemcpyAsync(counts, dcounts, ND_ * 4, cudaMemcpyDeviceToHost, stream_));
       SG_CUDA(cudaStreamSynchronize(stream_));
       free_one(dcounts);

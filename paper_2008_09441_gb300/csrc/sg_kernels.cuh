@@ -10,18 +10,9 @@
 namespace sg {
 
 // ---------------------------------------------------------------- sort
-constexpr int RS_THREADS = 256;
-constexpr int RS_ITEMS = 16;
+constexpr int RS_THREADS = 512;
+constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;  // keys per tile
-
-struct SortScratch {
-  uint32_t* tile_hist = nullptr;   // 256 * ntiles
-  uint32_t* block_sums = nullptr;  // scan block totals
-  size_t ntiles = 0;
-};
-
-size_t sort_scratch_words(size_t np);  // u32 words needed for SortScratch
-void sort_scratch_bind(SortScratch& s, uint32_t* base, size_t np);
 
 // keys[i] = Morton key of particle i's level-n cell, idx[i] = i,
 // *checksum += sum_i (keys[i] + 1).
@@ -29,22 +20,12 @@ template <typename real, int D>
 int launch_keys(const PArrays<real, D>& p, size_t np, int n, uint32_t* keys, uint32_t* idx,
                 unsigned long long* checksum, unsigned* status, cudaStream_t s);
 
-// Same for positions given as plain arrays (stand-alone sort entry point).
-template <typename real, int D>
-int launch_keys_raw(const real* const* u, size_t np, int n, uint32_t* keys, uint32_t* idx,
-                    unsigned long long* checksum, unsigned* status, cudaStream_t s);
-
-// Stable LSD radix sort of (key, value) pairs on the low `bits` key bits.
-// Ping-pongs between (keys, vals) and (keys_alt, vals_alt); *in_alt tells
-// where the sorted result ended.  If vals_identity, the first pass uses the
-// input index as value instead of reading vals.
-int radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt,
-                     size_t np, int bits, bool vals_identity, SortScratch& scr, cudaStream_t s,
-                     bool* in_alt);
-
-template <typename real, int D>
-int launch_permute(const PArrays<real, D>& src, const PArrays<real, D>& dst, const uint32_t* perm,
-                   size_t np, cudaStream_t s);
+// The stand-alone cell sort of positions u (dim device arrays in the given
+// precision): sorted keys, stable permutation, counts per cell (may be NULL).
+// scratch: cell_sort_words(n) u32 words.
+size_t cell_sort_words(size_t n);
+int cell_sort(int precision, int dim, int level, size_t n, const void* const* u, uint32_t* keys_sorted, uint32_t* perm,
+              uint32_t* counts, uint32_t* scratch, cudaStream_t s);
 
 // dst[pid[i]] = src[i] for every particle array (back to the original order;
 // dst's pid is not written).  scratch: unpermute_scratch_bytes(np) bytes
@@ -55,8 +36,9 @@ int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, s
 template <typename real, int D>
 size_t unpermute_scratch_bytes(size_t np);
 
-// counts[key] += 1 for every sorted key (counts zeroed by the caller).
-int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_t s);
+// counts[key] += 1 for every key (counts zeroed by the caller); sorted: the
+// keys are in order.
+int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_t s, bool sorted);
 
 // Exclusive scan of m u32 values (out may equal in).
 int exclusive_scan_u32(const uint32_t* in, uint32_t* out, size_t m, uint32_t* block_sums,

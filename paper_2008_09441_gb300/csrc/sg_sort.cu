@@ -1,6 +1,9 @@
-// Cell-key sort of the particles: Morton keys of the level-n cells, a stable
-// LSD radix sort of (key, index) pairs with 8-bit digits, the permutation of
-// the particle arrays and per-cell counts.  Integer work, bit-exact.
+// Cell-key sorts: the stand-alone stable sort of positions (Morton keys of the
+// level-n cells, permutation, per-cell counts; integer work, bit-exact), the
+// step's tile counting sort, and the particles' way back to their original
+// order.
+#include <atomic>
+
 #include "sg_kernels.cuh"
 
 namespace sg {
@@ -34,53 +37,10 @@ __global__ void __launch_bounds__(256) k_keys(PArrays<real, D> p, size_t np, int
 }
 
 template <typename real, int D>
-struct RawU {
-  const real* u[D];
-};
-
-template <typename real, int D>
-__global__ void __launch_bounds__(256) k_keys_raw(RawU<real, D> r, size_t np, int n, uint32_t* keys,
-                                                  uint32_t* idx, unsigned long long* checksum,
-                                                  unsigned* status) {
-  const int N = 1 << n;
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long part = 0;
-  if (i < np) {
-    int c[D];
-    bool bad = false;
-#pragma unroll
-    for (int m = 0; m < D; ++m) {
-      real u = r.u[m][i];
-      bad |= !(u >= (real)0 && u < (real)1);
-      // positions outside [0,1) are wrapped first (periodic box)
-      if (bad) u = wrap_unit(u);
-      c[m] = cell_of(u, n, N);
-    }
-    uint32_t k = morton_key<D>(c, n);
-    keys[i] = k;
-    if (idx) idx[i] = (uint32_t)i;
-    part = (unsigned long long)k + 1ull;
-  }
-  part = warp_sum(part);
-  if ((threadIdx.x & 31) == 0 && checksum && part) atomicAdd(checksum, part);
-}
-
-template <typename real, int D>
 int launch_keys(const PArrays<real, D>& p, size_t np, int n, uint32_t* keys, uint32_t* idx,
                 unsigned long long* checksum, unsigned* status, cudaStream_t s) {
   if (np == 0) return SG_OK;
   k_keys<real, D><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(p, np, n, keys, idx, checksum, status);
-  SG_CHECK_LAUNCH();
-  return SG_OK;
-}
-
-template <typename real, int D>
-int launch_keys_raw(const real* const* u, size_t np, int n, uint32_t* keys, uint32_t* idx,
-                    unsigned long long* checksum, unsigned* status, cudaStream_t s) {
-  if (np == 0) return SG_OK;
-  RawU<real, D> r;
-  for (int m = 0; m < D; ++m) r.u[m] = u[m];
-  k_keys_raw<real, D><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(r, np, n, keys, idx, checksum, status);
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
@@ -183,154 +143,319 @@ int exclusive_scan_u32(const uint32_t* in, uint32_t* out, size_t m, uint32_t* bl
   return SG_OK;
 }
 
-// ---------------------------------------------------------------- radix sort
+// ---------------------------------------------------------------- cell sort
+//
+// Stable LSD radix sort of (key, input index), the digits of equal width: 20
+// key bits take three passes of 7, 7 and 6 bits (the fewest passes of at most
+// 8, then the fewest digit values, which makes the runs a tile writes longer).
+// Per pass: digit counts of every tile, their scan (one block per digit), and
+// the scatter, which orders its tile by digit in shared memory first, so that
+// it writes runs of consecutive keys instead of one sector per key.  The first
+// count makes the keys from the positions; the last scatter writes the
+// caller's arrays.  Bound: L2 (the keys and indices of 4 M positions stay
+// there) and the warps' chains of ranking steps.  4,194,304 positions, 2D
+// level 10, with the counts: 397 us before (8-bit digits, unordered scatter
+// of 89 us a pass, scans of three launches, copies into the result), 132 us
+// now (65,537 positions, level 5: 93 -> 58; 3D level 7, 8 M in double: 1017 ->
+// 521).
 constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_WARP_KEYS = RS_TILE / RS_WARPS;
 static_assert(RS_WARP_KEYS == 32 * RS_ITEMS, "one key per lane per chunk");
 
-size_t sort_scratch_words(size_t np) {
-  size_t ntiles = (np + RS_TILE - 1) / RS_TILE;
-  if (ntiles == 0) ntiles = 1;
-  return 256 * ntiles + scan_block_sums_words(256 * ntiles) + 64;
+static size_t cell_sort_tiles(size_t n) { return (n + RS_TILE - 1) / RS_TILE; }
+size_t cell_sort_words(size_t n) { return 2 * n + 256 * cell_sort_tiles(n) + 256; }
+
+template <typename real, int D>
+struct RawU {
+  const real* u[D];
+};
+
+// Adds the tile's digits to h and writes them out: hist[digit * ntiles + tile].
+__device__ __forceinline__ void store_digits(const uint32_t* h, int bins, uint32_t* hist, size_t ntiles) {
+  __syncthreads();
+  for (int i = threadIdx.x; i < bins; i += RS_THREADS) hist[(size_t)i * ntiles + blockIdx.x] = h[i];
 }
 
-void sort_scratch_bind(SortScratch& s, uint32_t* base, size_t np) {
-  size_t ntiles = (np + RS_TILE - 1) / RS_TILE;
-  if (ntiles == 0) ntiles = 1;
-  s.ntiles = ntiles;
-  s.tile_hist = base;
-  s.block_sums = base + 256 * ntiles;
-}
-
-// Digit histogram of one tile; keys with equal digits in a warp are counted
-// by their leader (match_any aggregation) to avoid shared atomic pile-ups on
-// nearly sorted input.
-__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint32_t* keys, size_t n, int shift,
-                                                           uint32_t* hist, int ntiles) {
+template <typename real, int D>
+__global__ void __launch_bounds__(RS_THREADS) k_cell_keys(RawU<real, D> r, size_t n, int level, uint32_t* __restrict__ keys,
+                                                          int bins, uint32_t* __restrict__ hist, size_t ntiles) {
   __shared__ uint32_t h[256];
-  for (int i = threadIdx.x; i < 256; i += RS_THREADS) h[i] = 0;
+  for (int i = threadIdx.x; i < bins; i += RS_THREADS) h[i] = 0;
   __syncthreads();
-  size_t base = (size_t)blockIdx.x * RS_TILE;
-  int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < RS_TILE; i += RS_THREADS) {
-    size_t idx = base + i;
-    bool valid = idx < n;
-    uint32_t dg = valid ? ((keys[idx] >> shift) & 255u) : 256u;
-    unsigned peers = __match_any_sync(0xffffffffu, dg);
-    if (valid && lane == __ffs(peers) - 1) atomicAdd(&h[dg], (uint32_t)__popc(peers));
+  const size_t base = (size_t)blockIdx.x * RS_TILE;
+  const int N = 1 << level;
+#pragma unroll 4
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const size_t i = base + (size_t)k * RS_THREADS + threadIdx.x;
+    if (i < n) {
+      int c[D];
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        real u = __ldg(r.u[m] + i);
+        // positions outside [0,1) are wrapped first (periodic box)
+        if (!(u >= (real)0 && u < (real)1)) u = wrap_unit(u);
+        c[m] = cell_of(u, level, N);
+      }
+      const uint32_t key = morton_key<D>(c, level);
+      keys[i] = key;
+      atomicAdd(&h[key & (uint32_t)(bins - 1)], 1u);
+    }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += RS_THREADS) hist[(size_t)i * ntiles + blockIdx.x] = h[i];
+  store_digits(h, bins, hist, ntiles);
 }
 
-// Stable scatter of one tile: warp w owns keys [w*512, (w+1)*512) of the
-// tile, taken in 16 chunks of 32 in order; the rank of a key is the count
-// of earlier equal digits in its warp segment, then the warp-ordered prefix,
-// then the tile's global offset for the digit.
-__global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(const uint32_t* keys_in, const uint32_t* vals_in,
-                                                              size_t n, int shift, const uint32_t* offsets,
-                                                              int ntiles, uint32_t* keys_out,
-                                                              uint32_t* vals_out, int vals_identity) {
-  __shared__ uint32_t wh[RS_WARPS][256];
-  __shared__ uint32_t tile_off[256];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < RS_WARPS * 256; i += RS_THREADS) (&wh[0][0])[i] = 0;
-  for (int i = threadIdx.x; i < 256; i += RS_THREADS) tile_off[i] = offsets[(size_t)i * ntiles + blockIdx.x];
+__global__ void __launch_bounds__(RS_THREADS) k_radix_hist(const uint32_t* __restrict__ keys, size_t n, int shift,
+                                                           int bins, uint32_t* __restrict__ hist, size_t ntiles) {
+  __shared__ uint32_t h[256];
+  pdl_trigger();
+  for (int i = threadIdx.x; i < bins; i += RS_THREADS) h[i] = 0;
   __syncthreads();
-  size_t base = (size_t)blockIdx.x * RS_TILE + (size_t)w * RS_WARP_KEYS;
-  uint32_t kk[RS_ITEMS], rank[RS_ITEMS];
+  pdl_wait(keys);
+  const size_t base = (size_t)blockIdx.x * RS_TILE;
+#pragma unroll
+  for (int k = 0; k < RS_ITEMS; ++k) {
+    const size_t i = base + (size_t)k * RS_THREADS + threadIdx.x;
+    if (i < n) atomicAdd(&h[(keys[i] >> shift) & (uint32_t)(bins - 1)], 1u);
+  }
+  store_digits(h, bins, hist, ntiles);
+}
+
+// Block b: exclusive scan of digit b's counts over the tiles, in place, and
+// their sum at total[b].
+__global__ void __launch_bounds__(RS_THREADS) k_radix_scan(uint32_t* __restrict__ hist, size_t ntiles,
+                                                           uint32_t* __restrict__ total) {
+  __shared__ uint32_t ws[RS_WARPS];
+  pdl_trigger();
+  pdl_wait(hist);
+  uint32_t* row = hist + (size_t)blockIdx.x * ntiles;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t carry = 0;
+  for (size_t base = 0; base < ntiles; base += 4 * RS_THREADS) {
+    uint32_t v[4], sum = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const size_t i = base + (size_t)4 * threadIdx.x + j;
+      v[j] = i < ntiles ? row[i] : 0u;
+      sum += v[j];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) ws[w] = incl;
+    __syncthreads();
+    uint32_t before = carry + incl - sum, all = 0;
+#pragma unroll
+    for (int k = 0; k < RS_WARPS; ++k) {
+      if (k < w) before += ws[k];
+      all += ws[k];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const size_t i = base + (size_t)4 * threadIdx.x + j;
+      if (i < ntiles) row[i] = before;
+      before += v[j];
+    }
+    carry += all;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) total[blockIdx.x] = carry;
+}
+
+// Lanes of the warp with the same digit (BITS bits; invalid lanes form a
+// group of their own).
+template <int BITS>
+__device__ __forceinline__ unsigned same_digit(uint32_t dg, bool valid) {
+  unsigned m = __ballot_sync(0xffffffffu, valid);
+  if (!valid) m = ~m;
+#pragma unroll
+  for (int b = 0; b < BITS; ++b) {
+    const bool set = (dg >> b) & 1u;
+    const unsigned s = __ballot_sync(0xffffffffu, set);
+    m &= set ? s : ~s;
+  }
+  return m;
+}
+
+// Stable scatter of one tile.  Warp w owns keys [256 w, 256 (w + 1)) of the
+// tile, in 8 chunks of 32 in order; a key's rank is the count of earlier
+// equal digits of its warp, then of the warps before, then of the tile's
+// smaller digits.
+template <int BITS>
+__global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(const uint32_t* __restrict__ keys_in,
+                                                              const uint32_t* __restrict__ vals_in, size_t n,
+                                                              int shift, const uint32_t* __restrict__ hist,
+                                                              const uint32_t* __restrict__ total, size_t ntiles,
+                                                              uint32_t* __restrict__ keys_out,
+                                                              uint32_t* __restrict__ vals_out) {
+  constexpr int BINS = 1 << BITS;
+  extern __shared__ uint32_t stage[];     // keys, then indices, in the tile's digit order
+  __shared__ uint32_t wh[RS_WARPS][BINS];  // per warp: count, then the offset within the digit's run
+  __shared__ uint32_t lstart[BINS];        // digit's start in the tile
+  __shared__ uint32_t gstart[BINS];        // its run's place in the output, minus lstart
+  __shared__ uint32_t ws[2][RS_WARPS];
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
+  for (int i = tid; i < RS_WARPS * BINS; i += RS_THREADS) (&wh[0][0])[i] = 0;
+  __syncthreads();
+  pdl_wait(keys_in, vals_in, hist, total);
+  const size_t tile0 = (size_t)blockIdx.x * RS_TILE;
+  const size_t base = tile0 + (size_t)w * RS_WARP_KEYS + lane;
+  uint32_t kk[RS_ITEMS], vv[RS_ITEMS], rank[RS_ITEMS];
+#pragma unroll
+  for (int c = 0; c < RS_ITEMS; ++c) {
+    const size_t i = base + c * 32;
+    kk[c] = i < n ? keys_in[i] : 0u;
+    vv[c] = !vals_in ? (uint32_t)i : i < n ? vals_in[i] : 0u;
+  }
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int c = 0; c < RS_ITEMS; ++c) {
-    size_t idx = base + (size_t)c * 32 + lane;
-    bool valid = idx < n;
-    uint32_t key = valid ? keys_in[idx] : 0u;
-    uint32_t dg = valid ? ((key >> shift) & 255u) : 256u;
-    unsigned peers = __match_any_sync(0xffffffffu, dg);
-    uint32_t before = valid ? wh[w][dg] : 0u;
+    const bool valid = base + c * 32 < n;
+    const uint32_t dg = (kk[c] >> shift) & (uint32_t)(BINS - 1);
+    const unsigned peers = same_digit<BITS>(dg, valid);
+    const uint32_t before = wh[w][dg];
     __syncwarp();
-    if (valid && lane == __ffs(peers) - 1) wh[w][dg] = before + (uint32_t)__popc(peers);
+    if (valid && (peers & lt) == 0) wh[w][dg] = before + (uint32_t)__popc(peers);
     __syncwarp();
     rank[c] = before + (uint32_t)__popc(peers & lt);
-    kk[c] = key;
   }
   __syncthreads();
-  for (int d = threadIdx.x; d < 256; d += RS_THREADS) {
-    uint32_t run = 0;
+  {  // thread d: digit d's offsets by warp, its start in the tile and in the output
+    const int d = tid;
+    uint32_t cnt = 0, tot = 0;
+    if (d < BINS) {
 #pragma unroll
-    for (int ww = 0; ww < RS_WARPS; ++ww) {
-      uint32_t t = wh[ww][d];
-      wh[ww][d] = run;
-      run += t;
+      for (int ww = 0; ww < RS_WARPS; ++ww) {
+        const uint32_t t = wh[ww][d];
+        wh[ww][d] = cnt;
+        cnt += t;
+      }
+      tot = total[d];
+    }
+    uint32_t a = cnt, b = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, a, o), y = __shfl_up_sync(0xffffffffu, b, o);
+      if (lane >= o) {
+        a += x;
+        b += y;
+      }
+    }
+    if (lane == 31) {
+      ws[0][w] = a;
+      ws[1][w] = b;
+    }
+    __syncthreads();
+    if (d < BINS) {
+      uint32_t ls = a - cnt, gs = b - tot;
+      for (int k = 0; k < w; ++k) {
+        ls += ws[0][k];
+        gs += ws[1][k];
+      }
+      lstart[d] = ls;
+      gstart[d] = gs + hist[(size_t)d * ntiles + blockIdx.x] - ls;
     }
   }
   __syncthreads();
 #pragma unroll
-  for (int c = 0; c < RS_ITEMS; ++c) {
-    size_t idx = base + (size_t)c * 32 + lane;
-    if (idx < n) {
-      uint32_t dg = (kk[c] >> shift) & 255u;
-      uint32_t pos = tile_off[dg] + wh[w][dg] + rank[c];
-      keys_out[pos] = kk[c];
-      vals_out[pos] = vals_identity ? (uint32_t)idx : vals_in[idx];
+  for (int c = 0; c < RS_ITEMS; ++c)
+    if (base + c * 32 < n) {
+      const uint32_t dg = (kk[c] >> shift) & (uint32_t)(BINS - 1);
+      const uint32_t at = lstart[dg] + wh[w][dg] + rank[c];
+      stage[at] = kk[c];
+      stage[RS_TILE + at] = vv[c];
     }
+  __syncthreads();
+  const int nvalid = (int)min((size_t)RS_TILE, n - tile0);
+  for (int j = tid; j < nvalid; j += RS_THREADS) {
+    const uint32_t key = stage[j];
+    const uint32_t pos = gstart[(key >> shift) & (uint32_t)(BINS - 1)] + (uint32_t)j;
+    keys_out[pos] = key;
+    vals_out[pos] = stage[RS_TILE + j];
   }
-}
-
-int radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, size_t np,
-                     int bits, bool vals_identity, SortScratch& scr, cudaStream_t s, bool* in_alt) {
-  *in_alt = false;
-  if (np == 0) return SG_OK;
-  if (np > 0xFFFFFFFFull) {
-    set_error("radix sort: more than 2^32-1 particles");
-    return SG_ERR_SIZE;
-  }
-  int ntiles = (int)((np + RS_TILE - 1) / RS_TILE);
-  uint32_t *ki = keys, *vi = vals, *ko = keys_alt, *vo = vals_alt;
-  int passes = (bits + 7) / 8;
-  if (passes == 0) passes = 1;
-  bool ident = vals_identity;
-  for (int pass = 0; pass < passes; ++pass) {
-    int shift = pass * 8;
-    k_radix_hist<<<ntiles, RS_THREADS, 0, s>>>(ki, np, shift, scr.tile_hist, ntiles);
-    SG_CHECK_LAUNCH();
-    SG_TRY(exclusive_scan_u32(scr.tile_hist, scr.tile_hist, (size_t)256 * ntiles, scr.block_sums, s));
-    k_radix_scatter<<<ntiles, RS_THREADS, 0, s>>>(ki, vi, np, shift, scr.tile_hist, ntiles, ko, vo, ident ? 1 : 0);
-    SG_CHECK_LAUNCH();
-    ident = false;
-    uint32_t* t;
-    t = ki; ki = ko; ko = t;
-    t = vi; vi = vo; vo = t;
-    *in_alt = !*in_alt;
-  }
-  return SG_OK;
-}
-
-// ---------------------------------------------------------------- permute / counts
-template <typename real, int D>
-__global__ void __launch_bounds__(256) k_permute(PArrays<real, D> src, PArrays<real, D> dst, const uint32_t* perm,
-                                                 size_t np) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= np) return;
-  uint32_t j = perm[i];
-#pragma unroll
-  for (int m = 0; m < D; ++m) {
-    dst.u[m][i] = src.u[m][j];
-    dst.v[m][i] = src.v[m][j];
-  }
-  dst.w[i] = src.w[j];
-  dst.pid[i] = src.pid[j];
 }
 
 template <typename real, int D>
-int launch_permute(const PArrays<real, D>& src, const PArrays<real, D>& dst, const uint32_t* perm, size_t np,
-                   cudaStream_t s) {
-  if (np == 0) return SG_OK;
-  k_permute<real, D><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(src, dst, perm, np);
+static int cell_keys(const void* const* u, size_t n, int level, uint32_t* keys, int bins, uint32_t* hist,
+                     size_t ntiles, cudaStream_t s) {
+  RawU<real, D> r;
+  for (int m = 0; m < D; ++m) r.u[m] = static_cast<const real*>(u[m]);
+  k_cell_keys<real, D><<<(unsigned)ntiles, RS_THREADS, 0, s>>>(r, n, level, keys, bins, hist, ntiles);
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
 
+template <int BITS>
+static int radix_scatter(const uint32_t* ki, const uint32_t* vi, size_t n, int shift, const uint32_t* hist,
+                         const uint32_t* total, size_t ntiles, uint32_t* ko, uint32_t* vo, cudaStream_t s) {
+  static std::atomic<bool> attr_set{false};
+  if (!attr_set) {  // with the static part the total may pass 48 KB
+    SG_CUDA(cudaFuncSetAttribute(k_radix_scatter<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 2 * RS_TILE * (int)sizeof(uint32_t)));
+    attr_set = true;
+  }
+  SG_CUDA(launch_pdl(k_radix_scatter<BITS>, dim3((unsigned)ntiles), dim3(RS_THREADS), 2 * RS_TILE * sizeof(uint32_t), s,
+                     ki, vi, n, shift, hist, total, ntiles, ko, vo));
+  SG_CHECK_LAUNCH();
+  return SG_OK;
+}
+
+int cell_sort(int precision, int dim, int level, size_t n, const void* const* u, uint32_t* keys_sorted, uint32_t* perm,
+              uint32_t* counts, uint32_t* scratch, cudaStream_t s) {
+  if (counts) SG_CUDA(cudaMemsetAsync(counts, 0, ((size_t)1 << (dim * level)) * 4, s));
+  if (n == 0) return SG_OK;
+  const size_t ntiles = cell_sort_tiles(n);
+  uint32_t *tk = scratch, *tv = scratch + n, *hist = scratch + 2 * n, *total = hist + 256 * ntiles;
+  const int bits = dim * level, passes = (bits + 7) / 8;
+  // passes alternate between the scratch and the result, which the last one
+  // writes; the unsorted keys start where the first pass does not write
+  uint32_t* ki = passes & 1 ? tk : keys_sorted;
+  const uint32_t* vi = nullptr;  // the first pass's values are the input indices
+  int shift = 0;
+  for (int p = 0; p < passes; ++p) {
+    const int b = (bits - shift + passes - p - 1) / (passes - p), bins = 1 << b;
+    if (p == 0) {
+      if (precision == SG_FP32)
+        SG_TRY(dim == 2 ? cell_keys<float, 2>(u, n, level, ki, bins, hist, ntiles, s)
+                        : cell_keys<float, 3>(u, n, level, ki, bins, hist, ntiles, s));
+      else
+        SG_TRY(dim == 2 ? cell_keys<double, 2>(u, n, level, ki, bins, hist, ntiles, s)
+                        : cell_keys<double, 3>(u, n, level, ki, bins, hist, ntiles, s));
+    } else {
+      SG_CUDA(launch_pdl(k_radix_hist, dim3((unsigned)ntiles), dim3(RS_THREADS), 0, s, ki, n, shift, bins, hist, ntiles));
+      SG_CHECK_LAUNCH();
+    }
+    SG_CUDA(launch_pdl(k_radix_scan, dim3((unsigned)bins), dim3(RS_THREADS), 0, s, hist, ntiles, total));
+    SG_CHECK_LAUNCH();
+    const bool last_parity = ((passes - 1 - p) & 1) == 0;
+    uint32_t *ko = last_parity ? keys_sorted : tk, *vo = last_parity ? perm : tv;
+    switch (b) {
+#define SG_RS_CASE(B) \
+  case B: SG_TRY(radix_scatter<B>(ki, vi, n, shift, hist, total, ntiles, ko, vo, s)); break;
+      SG_RS_CASE(2)
+      SG_RS_CASE(3)
+      SG_RS_CASE(4)
+      SG_RS_CASE(5)
+      SG_RS_CASE(6)
+      SG_RS_CASE(7)
+      SG_RS_CASE(8)
+#undef SG_RS_CASE
+      default:
+        set_error("cell sort: unsupported digit width");
+        return SG_ERR_UNSUPPORTED;
+    }
+    ki = ko;
+    vi = vo;
+    shift += b;
+  }
+  if (counts) SG_TRY(launch_counts(keys_sorted, n, counts, s, true));
+  return SG_OK;
+}
+
+// ---------------------------------------------------------------- original order / counts
 template <typename real, int D>
 __global__ void __launch_bounds__(256) k_unpermute(PArrays<real, D> src, PArrays<real, D> dst, size_t np) {
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -728,17 +853,28 @@ int launch_tile_scatter(const PArrays<real, D>& src, const PArrays<real, D>& dst
   return SG_OK;
 }
 
-__global__ void __launch_bounds__(256) k_counts(const uint32_t* keys, size_t np, uint32_t* counts) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool valid = i < np;
-  uint32_t k = valid ? keys[i] : 0xFFFFFFFFu;
-  unsigned peers = __match_any_sync(0xffffffffu, k);
-  if (valid && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&counts[k], (uint32_t)__popc(peers));
+// counts[key] of runs of equal keys (any order of the keys; runs make it
+// fast).  A run inside one warp stores its length when `sorted` (it is then
+// the key's only run), others add theirs.
+__global__ void __launch_bounds__(256) k_counts(const uint32_t* __restrict__ keys, size_t np, uint32_t* counts,
+                                                int sorted) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  pdl_wait(keys);
+  const bool valid = i < np;
+  const uint32_t k = valid ? keys[i] : 0xFFFFFFFFu;
+  const uint32_t up = __shfl_up_sync(0xffffffffu, k, 1), dn = __shfl_down_sync(0xffffffffu, k, 1);
+  const unsigned starts = __ballot_sync(0xffffffffu, lane == 0 || up != k);
+  if (!valid || (lane < 31 && dn == k)) return;  // the run's last lane writes
+  const int first = 31 - __clz(starts & (0xFFFFFFFFu >> (31 - lane)));
+  const uint32_t len = (uint32_t)(lane - first + 1);
+  if (sorted && first > 0 && lane < 31) counts[k] = len;
+  else atomicAdd(&counts[k], len);
 }
 
-int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_t s) {
+int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_t s, bool sorted) {
   if (np == 0) return SG_OK;
-  k_counts<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(keys, np, counts);
+  SG_CUDA(launch_pdl(k_counts, dim3((unsigned)((np + 255) / 256)), dim3(256), 0, s, keys, np, counts, sorted ? 1 : 0));
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
@@ -746,10 +882,6 @@ int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_
 #define SG_INST_SORT(real, D)                                                                           \
   template int launch_keys<real, D>(const PArrays<real, D>&, size_t, int, uint32_t*, uint32_t*,        \
                                     unsigned long long*, unsigned*, cudaStream_t);                      \
-  template int launch_keys_raw<real, D>(const real* const*, size_t, int, uint32_t*, uint32_t*,         \
-                                        unsigned long long*, unsigned*, cudaStream_t);                  \
-  template int launch_permute<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, const uint32_t*, \
-                                       size_t, cudaStream_t);                                             \
   template int launch_unpermute<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, size_t, void*,        \
                                          cudaStream_t);                                                          \
   template size_t unpermute_scratch_bytes<real, D>(size_t);                                              \

@@ -1,7 +1,7 @@
 // Cell-key sort without device allocation.
 //
 // sg_cell_sort obtains its scratch (key/index ping-pong buffers, digit
-// histograms, scan totals, a status word) from the stream-ordered allocator
+// histograms and totals) from the stream-ordered allocator
 // on every call.  Some callers cannot do that: code that runs under a device
 // memory budget owned by another allocator (a framework's caching allocator
 // that holds all device memory), or latency-critical loops in which an
@@ -15,8 +15,7 @@
 // host-side stand-in), so the first call on each device looks the address up
 // with cudaGetSymbolAddress while that device is current and caches it.
 // Every call shares the array and it keeps the previous call's contents:
-// the only word that must start at zero (the status word) is cleared on the
-// call's stream, everything else is fully rewritten before it is read.  Two
+// everything is fully rewritten before it is read.  Two
 // calls whose work overlaps on the GPU (different streams, no ordering) race
 // on the array.
 #include <mutex>
@@ -25,11 +24,10 @@
 
 namespace sg {
 
-// keys, index, key ping-pong (3 x max), digit histograms and scan totals of
-// the radix sort, one status word, padding.
+// Keys and indices of the radix sort's alternate passes (2 x max), digit
+// histograms and totals.
 constexpr size_t kStaticMax = SG_CELL_SORT_STATIC_MAX;
-constexpr size_t kStaticTiles = (kStaticMax + RS_TILE - 1) / RS_TILE;
-constexpr size_t kStaticWords = 3 * kStaticMax + 256 * kStaticTiles + (256 * kStaticTiles) / 4096 + 1 + 64 + 16;
+constexpr size_t kStaticWords = 2 * kStaticMax + 256 * ((kStaticMax + RS_TILE - 1) / RS_TILE) + 256;  // cell_sort_words
 static_assert(kStaticWords <= SG_CELL_SORT_STATIC_WORDS, "scratch layout exceeds the declared size");
 
 static __device__ __align__(256) uint32_t g_cell_sort_scratch[SG_CELL_SORT_STATIC_WORDS];
@@ -93,44 +91,8 @@ extern "C" int sg_cell_sort_static(int precision, int dim, int level, size_t n, 
       return SG_ERR_INVALID;
     }
   cudaStream_t s = (cudaStream_t)stream;
-  const size_t cells = (size_t)1 << (dim * level);
-  if (n == 0) {
-    if (counts) SG_CUDA(cudaMemsetAsync(counts, 0, cells * 4, s));
-    return SG_OK;
-  }
+  if (n == 0) return cell_sort(precision, dim, level, 0, u, keys_sorted, perm, counts, nullptr, s);
   uint32_t* buf = nullptr;
   SG_TRY(static_scratch(&buf));
-  uint32_t* keys = buf;
-  uint32_t* vals = buf + kStaticMax;
-  uint32_t* keys_alt = buf + 2 * kStaticMax;
-  uint32_t* scr = buf + 3 * kStaticMax;
-  const size_t scr_words = sort_scratch_words(n);
-  if (3 * kStaticMax + scr_words + 1 > (size_t)SG_CELL_SORT_STATIC_WORDS) {
-    set_error("sg_cell_sort_static: scan layout exceeds the fixed scratch capacity");
-    return SG_ERR_SIZE;
-  }
-  unsigned* status = (unsigned*)(scr + scr_words);
-  SG_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned), s));  // the one word that must start at zero
-  SortScratch sc;
-  sort_scratch_bind(sc, scr, n);
-  int st;
-  if (precision == SG_FP32) {
-    st = dim == 2 ? launch_keys_raw<float, 2>((const float* const*)u, n, level, keys, nullptr, nullptr, status, s)
-                  : launch_keys_raw<float, 3>((const float* const*)u, n, level, keys, nullptr, nullptr, status, s);
-  } else {
-    st = dim == 2 ? launch_keys_raw<double, 2>((const double* const*)u, n, level, keys, nullptr, nullptr, status, s)
-                  : launch_keys_raw<double, 3>((const double* const*)u, n, level, keys, nullptr, nullptr, status, s);
-  }
-  if (st != SG_OK) return st;
-  bool in_alt = false;
-  SG_TRY(radix_sort_pairs(keys, vals, keys_alt, perm, n, dim * level, true, sc, s, &in_alt));
-  const uint32_t* ks = in_alt ? keys_alt : keys;
-  const uint32_t* ps = in_alt ? perm : vals;
-  SG_CUDA(cudaMemcpyAsync(keys_sorted, ks, n * 4, cudaMemcpyDeviceToDevice, s));
-  if (ps != perm) SG_CUDA(cudaMemcpyAsync(perm, ps, n * 4, cudaMemcpyDeviceToDevice, s));
-  if (counts) {
-    SG_CUDA(cudaMemsetAsync(counts, 0, cells * 4, s));
-    SG_TRY(launch_counts(keys_sorted, n, counts, s));
-  }
-  return SG_OK;
+  return cell_sort(precision, dim, level, n, u, keys_sorted, perm, counts, buf, s);
 }

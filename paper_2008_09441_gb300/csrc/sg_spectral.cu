@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(512) k_rows_forward(const Tin* __restrict__ in
   const int N = 1 << logn, P = N / 2 + 1, total = C << logn;
   pdl_trigger();
   const cplx<real>* tws = stage_twiddles(tw, logn, tw_smem ? buf + fpad_size(total) : nullptr);
-  pdl_wait();
+  pdl_wait(in);
   const size_t row0 = (size_t)blockIdx.x * C * 2;
   double mx = 0.0;
   for (int e = threadIdx.x; e < total; e += blockDim.x) {
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(512) k_columns(cplx<real>* __restrict__ Z, Col
   cplx<real>* z = Z + blockIdx.y * zstride + T.base;
   pdl_trigger();
   const cplx<real>* tws = stage_twiddles(tw, a.logn, a.tw_smem ? buf + fpad_size((size_t)a.C << a.logn) : nullptr);
-  pdl_wait();
+  pdl_wait(z, vmax);
   bool any = false;
   for (int t = T.t0; t < N; t += T.dt) {
     cplx<real> v = {(real)0, (real)0};
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(512) k_est_columns(const cplx<double>* __restr
   const int mask = e.mask[blockIdx.y];
   pdl_trigger();
   const cplx<double>* tws = stage_twiddles(tw, a.logn, a.tw_smem ? buf + fpad_size((size_t)a.C << a.logn) : nullptr);
-  pdl_wait();
+  pdl_wait(Z, e.vmax, e.m2max);
   const double s = est_scale(e.vmax), eps2 = e.frac * e.frac * *e.m2max;
   double fl = 1.0;  // factors of the line's own axes
   if (mask & 1) {
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(512) k_est_columns(const cplx<double>* __restr
 __global__ void __launch_bounds__(256) k_est_modes(const cplx<double>* __restrict__ Z, int D, int logn, EstArgs e,
                                                    double* out) {
   pdl_trigger();
-  pdl_wait();
+  pdl_wait(Z, e.vmax, e.m2max);
   const int N = 1 << logn, P = N / 2 + 1;
   const size_t n = (size_t)P << ((D - 1) * logn);
   const double s = est_scale(e.vmax), eps2 = e.frac * e.frac * *e.m2max;
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(512) k_solve_columns(const cplx<real>* __restr
   const Tile T = make_tile(a, blockIdx.x);
   pdl_trigger();
   const cplx<real>* tws = stage_twiddles(tw, a.logn, a.tw_smem ? buf1 + nbuf : nullptr);
-  pdl_wait();
+  pdl_wait(Z);
   for (int t = T.t0; t < N; t += T.dt) {
     cplx<real> v = {(real)0, (real)0};
     if (T.valid) v = Z[T.base + t * T.stride];
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(512) k_est_rows(const cplx<double>* __restrict
   const int N = 1 << logn, P = N / 2 + 1;
   pdl_trigger();
   const cplx<double>* tws = stage_twiddles(tw, logn, tw_smem ? buf + fpad_size((size_t)C << logn) : nullptr);
-  pdl_wait();
+  pdl_wait(W);
   const cplx<double>* w = W + blockIdx.y * wstride + (size_t)blockIdx.x * C * 2 * P;
   for (int e = threadIdx.x; e < C * P; e += blockDim.x) {
     const int p = e / P, k = e - p * P;
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(512) k_field_rows(const cplx<real>* __restrict
   const int N = 1 << logn, P = N / 2 + 1;
   pdl_trigger();
   const cplx<real>* tws = stage_twiddles(tw, logn, tw_smem ? buf + fpad_size((size_t)C << logn) : nullptr);
-  pdl_wait();
+  pdl_wait(A, B);
   const size_t j0 = (size_t)blockIdx.x * C;  // first transform
   for (int e = threadIdx.x; e < C * P; e += blockDim.x) {
     const int p = e / P, k = e - p * P;
