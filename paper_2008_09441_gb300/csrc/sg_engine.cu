@@ -95,6 +95,57 @@ std::map<PartKey, PartEntry>& part_cache() {
   return m;
 }
 
+// The transforms' tables, made once per precision and size in the process
+// (n <= 12: 0.4 MB in all).
+template <typename real>
+const std::vector<cplx<real>>& twiddles(int n) {
+  static std::mutex mu;
+  static std::map<int, std::vector<cplx<real>>> tables;
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = tables.find(n);
+  if (it == tables.end()) it = tables.emplace(n, make_twiddles<real>(n)).first;
+  return it->second;
+}
+
+// Mapped pinned host blocks of the runs' small records, kept for the next run
+// (at most 64 of 8 KB; pinning and unpinning cost tens of microseconds each).
+// Larger records, and those beyond 64, come and go with their run.
+class PinnedPool {
+ public:
+  static constexpr size_t kBlock = 8192;
+  static PinnedPool& get() {
+    static PinnedPool* p = new PinnedPool;  // lives as long as the CUDA context
+    return *p;
+  }
+  cudaError_t take(void** p, size_t* bytes) {
+    if (*bytes <= kBlock) {
+      *bytes = kBlock;
+      std::lock_guard<std::mutex> lk(mu_);
+      if (!free_.empty()) {
+        *p = free_.back();
+        free_.pop_back();
+        return cudaSuccess;
+      }
+    }
+    return cudaHostAlloc(p, *bytes, cudaHostAllocMapped | cudaHostAllocPortable);
+  }
+  void give(void* p, size_t bytes) {
+    if (!p) return;
+    if (bytes == kBlock) {
+      std::lock_guard<std::mutex> lk(mu_);
+      if (free_.size() < 64) {
+        free_.push_back(p);
+        return;
+      }
+    }
+    cudaFreeHost(p);
+  }
+
+ private:
+  std::mutex mu_;
+  std::vector<void*> free_;
+};
+
 struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
@@ -126,70 +177,70 @@ class Engine final : public EngineBase {
     tau_ = cfg.tau == SG_TAU_ADAPTIVE ? 1 : cfg.tau;
     adaptive_ = cfg.tau == SG_TAU_ADAPTIVE;
 
-    // ---- particles (two sets for the sort's out-of-place permutation)
-    size_t pb = std::max<size_t>(np_, 1);
-    for (int set = 0; set < 2; ++set) {
+    // ---- the run's fixed arrays, one allocation for all of them (see Plan)
+    Plan plan;
+    const size_t pb = std::max<size_t>(np_, 1);
+    for (int set = 0; set < 2; ++set) {  // particles: two sets for the sort's out-of-place permutation
       for (int m = 0; m < D; ++m) {
-        SG_TRY(alloc((void**)&P_[set].u[m], pb * sizeof(real)));
-        SG_TRY(alloc((void**)&P_[set].v[m], pb * sizeof(real)));
+        plan.want(&P_[set].u[m], pb);
+        plan.want(&P_[set].v[m], pb);
       }
-      SG_TRY(alloc((void**)&P_[set].w, pb * sizeof(real)));
-      SG_TRY(alloc((void**)&P_[set].pid, pb * sizeof(uint32_t)));
+      plan.want(&P_[set].w, pb);
+      plan.want(&P_[set].pid, pb);
     }
-    // ---- small device records (the status word is written by the upload check)
-    SG_TRY(alloc((void**)&dd_, sizeof(DevDiag)));
-    SG_TRY(alloc((void**)&status_, sizeof(unsigned)));
-    SG_TRY(alloc((void**)&checksum_, sizeof(unsigned long long)));
-    SG_CUDA(cudaMemsetAsync(dd_, 0, sizeof(DevDiag), stream_));
-    SG_CUDA(cudaMemsetAsync(status_, 0, sizeof(unsigned), stream_));
-    SG_CUDA(cudaMemsetAsync(checksum_, 0, sizeof(unsigned long long), stream_));
-
-    cur_ = 0;
-    SG_TRY(upload_particles(parts));
-    SG_TRY(alloc((void**)&keys_, pb * 4));
-    SG_TRY(alloc((void**)&keys_alt_, pb * 4));
+    plan.want(&dd_, 1);  // small device records (the status word is written by the upload check)
+    plan.want(&status_, 1);
+    plan.want(&checksum_, 1);
+    plan.want(&comb_counter_, 1);
+    plan.want(&keys_, pb);
+    plan.want(&keys_alt_, pb);
     tile_shift_ = std::max(0, n_ - 12 / D);
     ntiles_ = (size_t)1 << (D * (n_ - tile_shift_));
-    SG_TRY(alloc((void**)&tile_count_, ntiles_ * 4));
-    SG_TRY(alloc((void**)&cursor_, ntiles_ * 4));
-    SG_TRY(alloc((void**)&scan_sums_, scan_block_sums_words(ntiles_) * 4));
+    plan.want(&tile_count_, ntiles_);
+    plan.want(&cursor_, ntiles_);
+    plan.want(&scan_sums_, scan_block_sums_words(ntiles_));
     // push grid: one resident wave by default; the tuner may take half or two
     // waves, so the kinetic-energy partials (one per block) fit two waves
     push_wave_ = push_blocks<real, D>(np_);
     push_blocks_ = push_wave_;
     nke_ = push_blocks_;
     win_cap_ = cfg_.win_cap;
-    SG_TRY(alloc((void**)&ke_partials_, (size_t)2 * push_wave_ * sizeof(double)));
-    SG_CUDA(cudaMemsetAsync(ke_partials_, 0, (size_t)2 * push_wave_ * sizeof(double), stream_));
-
-    // ---- regular grid, combined field, twiddles
-    SG_TRY(alloc((void**)&rho_reg_, ND_ * sizeof(real)));
-    SG_TRY(alloc((void**)&Ehi_, (size_t)ec_stride<D>() * ND_ * sizeof(real)));  // node-interleaved
-    if (sizeof(real) == 4) SG_TRY(alloc((void**)&Elo_, (size_t)D * ND_ * sizeof(float)));
+    plan.want(&ke_partials_, (size_t)2 * push_wave_);
+    // regular grid, combined field (node-interleaved), twiddles
+    plan.want(&rho_reg_, ND_);
+    plan.want(&Ehi_, (size_t)ec_stride<D>() * ND_);
+    if (sizeof(real) == 4) plan.want(&Elo_, (size_t)D * ND_);
     nrows_ = (int)(ND_ / (size_t)N_);
-    SG_TRY(alloc((void**)&fe_partials_, (size_t)nrows_ * D * sizeof(double)));  // per (line, component)
-    SG_TRY(alloc((void**)&comb_counter_, sizeof(unsigned)));
-    SG_CUDA(cudaMemsetAsync(comb_counter_, 0, sizeof(unsigned), stream_));
-    {
-      const std::vector<cplx<real>> tw = make_twiddles<real>(n_);
-      SG_TRY(alloc((void**)&tw_, tw.size() * sizeof(cplx<real>)));
-      // pageable source: staged when the call returns, no synchronisation needed
-      SG_CUDA(cudaMemcpyAsync(tw_, tw.data(), tw.size() * sizeof(cplx<real>), cudaMemcpyHostToDevice, stream_));
-    }
+    plan.want(&fe_partials_, (size_t)nrows_ * D);  // per (line, component)
+    const std::vector<cplx<real>>& tw = twiddles<real>(n_);
+    plan.want(&tw_, tw.size());
     filter_ = cfg.mode == SG_MODE_FILTER;
+    std::vector<real> kt;
     if (filter_) {
-      // the regular-grid solve has no low parts: the planes stay zero
-      if (Elo_) SG_CUDA(cudaMemsetAsync(Elo_, 0, (size_t)D * ND_ * sizeof(float), stream_));
-      SG_TRY(alloc((void**)&rho_f_, ND_ * sizeof(real)));
-      SG_TRY(alloc((void**)&regA_, half_spectrum(D, n_) * sizeof(cplx<real>)));
-      SG_TRY(alloc((void**)&regB_, D * half_spectrum(D, n_) * sizeof(cplx<real>)));
-      std::vector<real> kt((size_t)D * N_);
+      kt.resize((size_t)D * N_);
       for (int m = 0; m < D; ++m)
         for (int i = 0; i < N_; ++i)
           kt[(size_t)m * N_ + i] = (real)(2.0 * M_PI / cfg_.L[m] * (double)(i < N_ / 2 ? i : i - N_));
-      SG_TRY(alloc((void**)&ktab_, kt.size() * sizeof(real)));
+      plan.want(&rho_f_, ND_);
+      plan.want(&regA_, half_spectrum(D, n_));
+      plan.want(&regB_, D * half_spectrum(D, n_));
+      plan.want(&ktab_, kt.size());
+      plan.want(&reg_partials_, ND_ / N_ * 3 / 2);
+    }
+    SG_TRY(alloc_plan(plan));
+    SG_CUDA(cudaMemsetAsync(dd_, 0, sizeof(DevDiag), stream_));
+    SG_CUDA(cudaMemsetAsync(status_, 0, sizeof(unsigned), stream_));
+    SG_CUDA(cudaMemsetAsync(checksum_, 0, sizeof(unsigned long long), stream_));
+    SG_CUDA(cudaMemsetAsync(comb_counter_, 0, sizeof(unsigned), stream_));
+    SG_CUDA(cudaMemsetAsync(ke_partials_, 0, (size_t)2 * push_wave_ * sizeof(double), stream_));
+    cur_ = 0;
+    SG_TRY(upload_particles(parts));
+    // pageable sources: staged when the call returns, no synchronisation needed
+    SG_CUDA(cudaMemcpyAsync(tw_, tw.data(), tw.size() * sizeof(cplx<real>), cudaMemcpyHostToDevice, stream_));
+    if (filter_) {
+      // the regular-grid solve has no low parts: the planes stay zero
+      if (Elo_) SG_CUDA(cudaMemsetAsync(Elo_, 0, (size_t)D * ND_ * sizeof(float), stream_));
       SG_CUDA(cudaMemcpyAsync(ktab_, kt.data(), kt.size() * sizeof(real), cudaMemcpyHostToDevice, stream_));
-      SG_TRY(alloc((void**)&reg_partials_, (ND_ / N_ * 3 / 2) * sizeof(double)));
     }
 
     SG_TRY(particle_stats());
@@ -389,11 +440,12 @@ class Engine final : public EngineBase {
   // kernel writes a diagnostics record straight into it.
   int ensure_pinned(void** p, size_t* have, size_t need) {
     if (need <= *have) return SG_OK;
-    if (*p) cudaFreeHost(*p);
+    PinnedPool::get().give(*p, *have);
     *p = nullptr;
     *have = 0;
-    SG_CUDA(cudaHostAlloc(p, need, cudaHostAllocMapped));
-    *have = need;
+    size_t bytes = need;
+    SG_CUDA(PinnedPool::get().take(p, &bytes));
+    *have = bytes;
     return SG_OK;
   }
   // Enqueue the kernel that packs the record into the mapped host buffer h
@@ -911,6 +963,34 @@ class Engine final : public EngineBase {
     bytes_ += bytes;
     return SG_OK;
   }
+  // Several arrays in one allocation.  The stream-ordered allocator looks, at
+  // every call, at what earlier runs freed on other streams: with some forty
+  // calls per run, admitting eight served runs took 7.8 ms in a fresh process
+  // and 18.9 ms after nine other runs had come and gone; with one for the
+  // run's fixed arrays and one per grid set (and pinned blocks and twiddles
+  // kept for the next run) 2.6 and 3.2 ms.
+  struct Plan {
+    struct Item {
+      void** p;
+      size_t bytes;
+    };
+    std::vector<Item> items;
+    template <typename T>
+    void want(T** p, size_t count) {
+      items.push_back({reinterpret_cast<void**>(p), std::max<size_t>(count * sizeof(T), 16)});
+    }
+  };
+  int alloc_plan(const Plan& plan) {
+    size_t total = 0;
+    for (const auto& i : plan.items) total += (i.bytes + 255) / 256 * 256;
+    char* base = nullptr;
+    SG_TRY(alloc((void**)&base, total));
+    for (const auto& i : plan.items) {
+      *i.p = base;
+      base += (i.bytes + 255) / 256 * 256;
+    }
+    return SG_OK;
+  }
   // Once per device in the process: the default pool keeps up to 16 GB of
   // freed memory for reuse (process-local, released at exit).
   static void keep_pool_memory() {
@@ -941,17 +1021,17 @@ class Engine final : public EngineBase {
     for (auto& b : bufs_) cudaFreeAsync(b.p, stream_);
     if (stream_) cudaStreamSynchronize(stream_);
     bufs_.clear();
-    if (diag_host_) cudaFreeHost(diag_host_);
+    PinnedPool::get().give(diag_host_, diag_host_bytes_);
     diag_host_ = nullptr;
     diag_host_bytes_ = 0;
-    if (est_host_) cudaFreeHost(est_host_);
+    PinnedPool::get().give(est_host_, est_host_bytes_);
     est_host_ = nullptr;
     est_host_bytes_ = 0;
-    if (stats_host_) cudaFreeHost(stats_host_);
+    PinnedPool::get().give(stats_host_, stats_host_bytes_);
     stats_host_ = nullptr;
     stats_host_bytes_ = 0;
     for (auto& r : ring_) {
-      if (r.host) cudaFreeHost(r.host);
+      PinnedPool::get().give(r.host, r.bytes);
       if (r.ev) cudaEventDestroy(r.ev);
       r = DiagSlot();
     }
@@ -1055,38 +1135,87 @@ class Engine final : public EngineBase {
       off += (size_t)sz;
     }
     S_ = off;
-    // (re)allocate arenas
+    // The grid set's arrays and tables are measured first (the builders run
+    // without touching the device), then take one allocation and one copy.
     for (void* p : grid_bufs_) free_one(p);
     grid_bufs_.clear();
-    SG_TRY(galloc((void**)&grids_dev_, ngrids_ * sizeof(GridDesc)));
-    SG_TRY(build_combine_tables());
-    SG_TRY(galloc((void**)&rho_arena_, S_ * sizeof(real)));
-    SG_TRY(galloc((void**)&A_, S_ * sizeof(cplx<real>)));
-    SG_TRY(galloc((void**)&B_, (size_t)((D + 1) / 2) * S_ * sizeof(cplx<real>)));  // component pairs
-    SG_TRY(galloc((void**)&E_arena_, (size_t)ec_stride<D>() * S_ * sizeof(real)));  // node-interleaved
-    SG_CUDA(cudaMemcpyAsync(grids_dev_, gdesc_.data(), ngrids_ * sizeof(GridDesc), cudaMemcpyHostToDevice, stream_));
-    SG_TRY(build_restrict_jobs());
-    SG_TRY(build_fft_jobs());
-    if (D == 3) {
-      // The combination's pair scratch takes what the run's estimated
-      // footprint leaves (all planes at tau = 1: 6.3 MB at n = 7); larger tau,
-      // whose pairs grow towards the regular grid, go in several runs of
-      // planes instead of past the estimate that serving admits by (which
-      // leaves out the estimator's and the filter mode's arrays), in eight
-      // runs at most.
-      const size_t plane = (size_t)ec_stride<D>() * comb_.S2 * ((sizeof(real) == 8 || cfg_.combine_fp64) ? 8 : 4);
-      const size_t est = estimate_footprint(sizeof(real) == 8 ? SG_FP64 : SG_FP32, D, n_, tau_, np_);
-      const size_t used = bytes_ - est_bytes_;
-      const size_t left = std::max(est > used ? est - used : 0, plane * N_ / 8);
-      comb_.scratch_bytes = std::max(plane, std::min(plane * (size_t)N_, left));
-      SG_TRY(galloc(&comb_.scratch, comb_.scratch_bytes));
+    for (int pass = 0; pass < 2; ++pass) {
+      garena_.begin(pass == 0);
+      if (pass == 1) {
+        SG_TRY(alloc((void**)&garena_.base, garena_.total()));
+        grid_bufs_.push_back(garena_.base);
+      }
+      SG_TRY(gtable(&grids_dev_, gdesc_.data(), ngrids_));
+      SG_TRY(galloc((void**)&rho_arena_, S_ * sizeof(real)));
+      SG_TRY(galloc((void**)&A_, S_ * sizeof(cplx<real>)));
+      SG_TRY(galloc((void**)&B_, (size_t)((D + 1) / 2) * S_ * sizeof(cplx<real>)));  // component pairs
+      SG_TRY(galloc((void**)&E_arena_, (size_t)ec_stride<D>() * S_ * sizeof(real)));  // node-interleaved
+      SG_TRY(build_combine_tables());
+      SG_TRY(build_restrict_jobs());
+      SG_TRY(build_fft_jobs());
+      if (D == 3) {
+        // The combination's pair scratch takes what the run's estimated
+        // footprint leaves (all planes at tau = 1: 6.3 MB at n = 7); larger tau,
+        // whose pairs grow towards the regular grid, go in several runs of
+        // planes instead of past the estimate that serving admits by (which
+        // leaves out the estimator's and the filter mode's arrays), in eight
+        // runs at most.
+        const size_t plane = (size_t)ec_stride<D>() * comb_.S2 * ((sizeof(real) == 8 || cfg_.combine_fp64) ? 8 : 4);
+        if (pass == 0) {
+          const size_t est = estimate_footprint(sizeof(real) == 8 ? SG_FP64 : SG_FP32, D, n_, tau_, np_);
+          const size_t used = bytes_ - est_bytes_ + garena_.total();
+          const size_t left = std::max(est > used ? est - used : 0, plane * N_ / 8);
+          comb_scratch_bytes_ = std::max(plane, std::min(plane * (size_t)N_, left));
+        }
+        comb_.scratch_bytes = comb_scratch_bytes_;
+        SG_TRY(galloc(&comb_.scratch, comb_.scratch_bytes));
+      }
     }
+    // pageable source: staged when the call returns, no synchronisation needed
+    SG_CUDA(cudaMemcpyAsync(garena_.base, garena_.staging.data(), garena_.staging.size(), cudaMemcpyHostToDevice,
+                            stream_));
     SG_CUDA(cudaStreamSynchronize(stream_));
     return SG_OK;
   }
+  // Bump allocator of the grid set: tables (copied from `staging` together)
+  // in front, arrays behind.  While measuring, pointers are only offsets from
+  // an address that is never used.
+  struct GridArena {
+    bool measure = true;
+    size_t table_bytes = 0, array_bytes = 0, table_at = 0, array_at = 0;
+    char* base = nullptr;
+    std::vector<char> staging;
+    static size_t pad(size_t b) { return (std::max<size_t>(b, 16) + 255) / 256 * 256; }
+    size_t total() const { return table_bytes + array_bytes; }
+    void begin(bool m) {
+      measure = m;
+      table_at = array_at = 0;
+      if (m) {
+        table_bytes = array_bytes = 0;
+        base = reinterpret_cast<char*>((uintptr_t)1 << 20);
+      } else {
+        staging.assign(table_bytes, 0);
+      }
+    }
+  };
   int galloc(void** p, size_t bytes) {
-    SG_TRY(alloc(p, bytes));
-    grid_bufs_.push_back(*p);
+    const size_t b = GridArena::pad(bytes);
+    if (garena_.measure) {
+      garena_.array_bytes += b;
+      *p = garena_.base + garena_.array_at;
+    } else {
+      *p = garena_.base + garena_.table_bytes + garena_.array_at;
+    }
+    garena_.array_at += b;
+    return SG_OK;
+  }
+  template <typename T>
+  int gtable(T** p, const T* src, size_t count) {
+    const size_t bytes = count * sizeof(T), b = GridArena::pad(bytes);
+    *p = reinterpret_cast<T*>(garena_.base + garena_.table_at);
+    if (garena_.measure) garena_.table_bytes += b;
+    else std::memcpy(garena_.staging.data() + garena_.table_at, src, bytes);
+    garena_.table_at += b;
     return SG_OK;
   }
 
@@ -1136,13 +1265,11 @@ class Engine final : public EngineBase {
       return SG_ERR_UNSUPPORTED;
     }
     LineGrid* ld = nullptr;
-    SG_TRY(galloc((void**)&ld, lines.size() * sizeof(LineGrid)));
-    SG_CUDA(cudaMemcpyAsync(ld, lines.data(), lines.size() * sizeof(LineGrid), cudaMemcpyHostToDevice, stream_));
+    SG_TRY(gtable(&ld, lines.data(), lines.size()));
     comb_.lines = ld;
     if (D == 3) {
       PlanePair* pd = nullptr;
-      SG_TRY(galloc((void**)&pd, pairs.size() * sizeof(PlanePair)));
-      SG_CUDA(cudaMemcpyAsync(pd, pairs.data(), pairs.size() * sizeof(PlanePair), cudaMemcpyHostToDevice, stream_));
+      SG_TRY(gtable(&pd, pairs.data(), pairs.size()));
       comb_.pairs = pd;
       comb_.npairs = (int)pairs.size();
       comb_.S2 = S2;
@@ -1252,9 +1379,7 @@ class Engine final : public EngineBase {
       P.lpb = lpb;
       P.vpl = std::max(1, N_ / 32);
       P.smem = a == 0 ? 0 : (int)((size_t)lpb * S * sizeof(real));
-      SG_TRY(galloc((void**)&P.dev, jobs.size() * sizeof(LineJob)));
-      // pageable source: staged when the call returns, no synchronisation needed
-      SG_CUDA(cudaMemcpyAsync(P.dev, jobs.data(), jobs.size() * sizeof(LineJob), cudaMemcpyHostToDevice, stream_));
+      SG_TRY(gtable(&P.dev, jobs.data(), jobs.size()));
       rpasses_.push_back(P);
       prev.swap(next);
     }
@@ -1289,8 +1414,7 @@ class Engine final : public EngineBase {
       next[key] = dst;
       t.dst[g.l[0]][g.l[1]] = dst;
     }
-    SG_TRY(galloc((void**)&restrict_planes_, sizeof(t)));
-    SG_CUDA(cudaMemcpyAsync(restrict_planes_, &t, sizeof(t), cudaMemcpyHostToDevice, stream_));
+    SG_TRY(gtable(&restrict_planes_, &t, 1));
     restrict_lx_min_ = t.lx_min;
     prev->swap(next);
     *first = 2;
@@ -1345,9 +1469,7 @@ class Engine final : public EngineBase {
       P.njobs = (int)jobs.size();
       P.nblocks = blocks;
       P.smem = smem;
-      SG_TRY(galloc((void**)&P.dev, jobs.size() * sizeof(FftJob)));
-      // pageable source: staged when the call returns, no synchronisation needed
-      SG_CUDA(cudaMemcpyAsync(P.dev, jobs.data(), jobs.size() * sizeof(FftJob), cudaMemcpyHostToDevice, stream_));
+      SG_TRY(gtable(&P.dev, jobs.data(), jobs.size()));
       fpasses_.push_back(P);
     }
     return SG_OK;
@@ -1363,7 +1485,7 @@ class Engine final : public EngineBase {
     SG_TRY(alloc((void**)&est_z_, hs));
     SG_TRY(alloc((void**)&est_w_, est_wcount_ * hs));
     SG_TRY(alloc((void**)&est_scalar_, 16 * sizeof(double)));
-    const std::vector<cplx<double>> tw = make_twiddles<double>(n_);
+    const std::vector<cplx<double>>& tw = twiddles<double>(n_);
     SG_TRY(alloc((void**)&tw64_, tw.size() * sizeof(cplx<double>)));
     SG_CUDA(cudaMemcpyAsync(tw64_, tw.data(), tw.size() * sizeof(cplx<double>), cudaMemcpyHostToDevice, stream_));
     est_bytes_ = bytes_ - before;
@@ -2024,6 +2146,8 @@ class Engine final : public EngineBase {
   std::vector<GridDesc> gdesc_;
   int ngrids_ = 0;
   CombineTables comb_;
+  size_t comb_scratch_bytes_ = 0;
+  GridArena garena_;
   bool per_grid_ = false;
   int solve_mode_ = -1;  // -1 untuned, 0 per-axis passes, 1 one block per grid
   int force_mode_ = -1;  // solve variant fixed by the caller, -1 autotuned
