@@ -67,13 +67,28 @@ __device__ __forceinline__ void cell_frac(double s, int mask, int& c, double& f)
   f = s - fl;
 }
 
+// Division by a box's extents in the flush: r / n = (r ceil(2^32 / n)) >> 32,
+// exact while r n < 2^32 (a box has at most 51,200 nodes, 224 along an axis);
+// n = 1 is taken separately.
+constexpr int DEP_MAX_SIDE = 224;  // 200 KB of 32-bit nodes
+struct Reciprocals {
+  uint32_t m[DEP_MAX_SIDE + 1];
+  constexpr Reciprocals() : m() {
+    m[0] = m[1] = 0;
+    for (int n = 2; n <= DEP_MAX_SIDE; ++n) m[n] = 0xFFFFFFFFu / (uint32_t)n + 1u;
+  }
+};
+__constant__ const Reciprocals c_recip = Reciprocals();
+__device__ __forceinline__ int div_by(int r, int n, uint32_t m) { return n == 1 ? r : (int)__umulhi((unsigned)r, m); }
+
 // ---------------------------------------------------------------- deposit
 //
-// Persistent blocks walk chunks of 4 THREADS (DEP_CHUNK, or a quarter) consecutive particles
+// Persistent blocks walk chunks of THREADS x ITEMS (DEP_CHUNK; small runs a
+// quarter) consecutive particles
 // (consecutive in tile-key order after a sort, so a chunk covers a compact
 // group of cells).  Per chunk every thread reads the chunk's middle particle
 // and takes its cell as the anchor of a fixed window of side^d regular nodes
-// centred on it; its four particles (16-byte vector loads) add their CIC
+// centred on it; its particles (16-byte vector loads) add their CIC
 // weights into the window when all 2^d corners fall inside, else straight to
 // the global grid.  The window's touched box is then added to the global
 // grid row by row and cleared for the next chunk: two block barriers per
@@ -87,12 +102,12 @@ __device__ __forceinline__ void cell_frac(double s, int mask, int& c, double& f)
 // FP32: WinAcc fixed point with the run's scale 2^(20 - E), max_p |q_p|/V <=
 // 2^E (1 - 2^-11) (set at upload; charges do not change), so a window of at
 // most 2^11 particles cannot overflow.  FP64: plain double, scale 1.
-template <typename real, int D, int THREADS>
+template <typename real, int D, int THREADS, int ITEMS>
 __global__ void __launch_bounds__(THREADS) k_deposit(PArrays<real, D> p, size_t np, int n,
                                                          real inv_cell_vol, real* __restrict__ rho, int side,
                                                          real scale, real inv_scale, real shift) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int CHUNK = THREADS * DEP_ITEMS;
+  constexpr int CHUNK = THREADS * ITEMS;
   using W = WinAcc<real>;
   using T = typename W::T;
   T* win = reinterpret_cast<T*>(smem_raw);
@@ -118,10 +133,10 @@ __global__ void __launch_bounds__(THREADS) k_deposit(PArrays<real, D> p, size_t 
   int par = 0;
   for (size_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x, par ^= 1) {
     const size_t chunk = ch * CHUNK;
-    // ---- this thread's particles: DEP_ITEMS / 4 vectors of four
-    real ub[DEP_ITEMS][D], qb[DEP_ITEMS];
+    // ---- this thread's particles: ITEMS / 4 vectors of four
+    real ub[ITEMS][D], qb[ITEMS];
 #pragma unroll
-    for (int j = 0; j < DEP_ITEMS / 4; ++j) {
+    for (int j = 0; j < ITEMS / 4; ++j) {
       // Which four particles.  FP32: consecutive threads, consecutive vectors
       // (equal addresses of a warp's integer adds are merged; spreading them
       // cost 40%).  FP64: the shared double add is a compare-and-swap loop
@@ -174,7 +189,7 @@ __global__ void __launch_bounds__(THREADS) k_deposit(PArrays<real, D> p, size_t 
       hi[m] = INT_MIN;
     }
 #pragma unroll
-    for (int it = 0; it < DEP_ITEMS; ++it) {
+    for (int it = 0; it < ITEMS; ++it) {
       if (qb[it] == (real)0) continue;
       int c[D], l[D];
       real f[D];
@@ -263,11 +278,13 @@ __global__ void __launch_bounds__(THREADS) k_deposit(PArrays<real, D> p, size_t 
       const int x0 = W::fixed ? (blo[0] & ~3) : blo[0];
       const int nx = (bhi[0] - x0) / PER + 1;
       const int total = nrows * nx;
+      const uint32_t mx = c_recip.m[nx], my = c_recip.m[ny];
       for (int f = threadIdx.x; f < total; f += THREADS) {
-        const int r = f / nx;
+        const int r = div_by(f, nx, mx);
         const int x = x0 + (f - r * nx) * PER;
-        const int ly = blo[1 % D] + (D == 2 ? r : r % ny);
-        const int lz = D == 2 ? 0 : blo[D - 1] + r / ny;
+        const int rz = D == 2 ? 0 : div_by(r, ny, my);
+        const int ly = blo[1 % D] + r - rz * ny;
+        const int lz = D == 2 ? 0 : blo[D - 1] + rz;
         const size_t gy = (size_t)((origin[1 % D] + ly) & mask);
         const size_t grow = D == 2 ? gy * N : ((size_t)((origin[D - 1] + lz) & mask) * N + gy) * N;
         T* wrow = win + ((size_t)lz * side + ly) * side;
@@ -293,7 +310,7 @@ __global__ void __launch_bounds__(THREADS) k_deposit(PArrays<real, D> p, size_t 
   }
 }
 
-template <typename real, int D, int THREADS>
+template <typename real, int D, int THREADS, int ITEMS>
 static int launch_deposit_threads(const PArrays<real, D>& p, size_t np, int n, real inv_cell_vol, real* rho, int side,
                                   size_t smem, int sms, real scale, real inv_scale, real shift, cudaStream_t s) {
   // resident blocks per SM for each window size met so far (the autotuner
@@ -303,15 +320,15 @@ static int launch_deposit_threads(const PArrays<real, D>& p, size_t np, int n, r
   static int known_per_sm[8];
   static int nknown = 0;
   if (!attr_set) {
-    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS, ITEMS>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     attr_set = true;
   }
   int per_sm = 0;
   for (int i = 0; i < nknown; ++i)
     if (known_smem[i] == smem) per_sm = known_per_sm[i];
   if (!per_sm) {
-    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_deposit<real, D, THREADS>, THREADS, smem));
+    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_deposit<real, D, THREADS, ITEMS>, THREADS, smem));
     if (per_sm < 1) per_sm = 1;
     if (nknown < 8) {
       known_smem[nknown] = smem;
@@ -319,10 +336,10 @@ static int launch_deposit_threads(const PArrays<real, D>& p, size_t np, int n, r
       ++nknown;
     }
   }
-  constexpr int CHUNK = THREADS * DEP_ITEMS;
+  constexpr int CHUNK = THREADS * ITEMS;
   const size_t nchunks = (np + CHUNK - 1) / CHUNK;
   const unsigned blocks = (unsigned)std::min<size_t>(nchunks, (size_t)sms * per_sm);
-  k_deposit<real, D, THREADS><<<blocks, THREADS, smem, s>>>(p, np, n, inv_cell_vol, rho, side, scale, inv_scale, shift);
+  k_deposit<real, D, THREADS, ITEMS><<<blocks, THREADS, smem, s>>>(p, np, n, inv_cell_vol, rho, side, scale, inv_scale, shift);
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
@@ -362,10 +379,10 @@ int launch_deposit(const PArrays<real, D>& p, size_t np, int n, real inv_cell_vo
   // 3D n = 5 56.5 -> 28.3; FP32 3D n = 5, 100,003 particles 13.2 -> 11.6, 2D
   // n = 6 10.6 -> 8.8; no change from 500,000 particles on).
   if ((np + DEP_CHUNK - 1) / DEP_CHUNK < (size_t)2 * sms)
-    return launch_deposit_threads<real, D, DEP_THREADS / 4>(p, np, n, inv_cell_vol, rho, side, smem, sms, scale,
+    return launch_deposit_threads<real, D, DEP_SMALL_THREADS, DEP_SMALL_ITEMS>(p, np, n, inv_cell_vol, rho, side, smem, sms, scale,
                                                             inv_scale, shift, s);
-  return launch_deposit_threads<real, D, DEP_THREADS>(p, np, n, inv_cell_vol, rho, side, smem, sms, scale, inv_scale,
-                                                      shift, s);
+  return launch_deposit_threads<real, D, DEP_THREADS, DEP_ITEMS>(p, np, n, inv_cell_vol, rho, side, smem, sms, scale,
+                                                                 inv_scale, shift, s);
 }
 
 // ---------------------------------------------------------------- restriction

@@ -46,8 +46,15 @@ int exclusive_scan_u32(const uint32_t* in, uint32_t* out, size_t m, uint32_t* bl
 size_t scan_block_sums_words(size_t m);
 
 // ---------------------------------------------------------------- deposit
-constexpr int DEP_THREADS = 512;
-constexpr int DEP_ITEMS = 4;
+// Particles per thread: eight share the chunk's per-thread work (anchor, box,
+// barriers); four on twice the threads and sixteen on half as many were slower
+// (3D two-stream, 8,388,608 particles: 93.8 and 96.4 against 90.0 us, with
+// the flush's divisions as multiplications in all three; with real divisions
+// and four 102.7).  Small runs take 128 threads and four.
+constexpr int DEP_THREADS = 256;
+constexpr int DEP_ITEMS = 8;
+constexpr int DEP_SMALL_THREADS = 128;
+constexpr int DEP_SMALL_ITEMS = 4;
 constexpr int DEP_CHUNK = DEP_THREADS * DEP_ITEMS;
 
 // scale / inv_scale: the FP32 fixed-point scale of the window (WinAcc), 1 for FP64.
