@@ -1548,14 +1548,13 @@ class Engine final : public EngineBase {
   }
 
   // Step sort: counting sort of the particles by tile key (the Morton key of
-  // the level-(n - tile_shift) cell), in two halves: keys + tile counts
-  // (emitted by the push on sort steps, or by k_tile_keys), then the scan of
+  // the level-(n - tile_shift) cell), in two halves: cell keys (emitted by the
+  // push on sort steps, or by k_tile_keys), then the tile counts, the scan of
   // the counts and one scatter pass of the particle payload.
   SortFuse sort_fuse() const {
     SortFuse sf;
     sf.keys = keys_;
     sf.checksum = checksum_;
-    sf.tile_shift = tile_shift_;
     return sf;
   }
   int sort_reset() {
@@ -1565,9 +1564,9 @@ class Engine final : public EngineBase {
   }
   int sort_finish(cudaStream_t s = nullptr) {
     if (!s) s = stream_;
-    SG_TRY(launch_tile_hist(keys_, np_, tile_count_, s));
+    SG_TRY(launch_tile_hist(keys_, np_, D * tile_shift_, tile_count_, s));
     SG_TRY(exclusive_scan_u32(tile_count_, cursor_, ntiles_, scan_sums_, s));
-    SG_TRY(launch_tile_scatter<real, D>(P_[cur_], P_[cur_ ^ 1], keys_, cursor_, np_, s));
+    SG_TRY(launch_tile_scatter<real, D>(P_[cur_], P_[cur_ ^ 1], keys_, D * tile_shift_, cursor_, np_, s));
     cur_ ^= 1;
     return SG_OK;
   }

@@ -309,9 +309,8 @@ struct PushParams {
 
 // Sort work fused into the push on sort steps (keys == nullptr: none).
 struct SortFuse {
-  uint32_t* keys = nullptr;        // tile key per particle (storage order)
+  uint32_t* keys = nullptr;        // level-n Morton key per particle (storage order)
   unsigned long long* checksum = nullptr;
-  int tile_shift = 0;              // tile = level-n Morton key >> (D * tile_shift)
 };
 
 template <typename real, int D>
@@ -321,17 +320,17 @@ template <typename real, int D>
 int push_blocks(size_t np);  // grid of the push (size of its kinetic-energy partials)
 
 // ---------------------------------------------------------------- step sort (tile counting sort)
-// Tile keys and counts of the current positions (the push emits them on sort
-// steps; this kernel serves init and checkpoint load).
+// Cell keys of the current positions (the push emits them on sort steps; this
+// kernel serves init and checkpoint load).  A key's tile is key >> shift.
 template <typename real, int D>
 int launch_tile_keys(const PArrays<real, D>& p, size_t np, int n, const SortFuse& sf, unsigned* status,
                      cudaStream_t s);
-// tile_count[key] += 1 for every key (counts zeroed by the caller).
-int launch_tile_hist(const uint32_t* keys, size_t np, uint32_t* tile_count, cudaStream_t s);
-// Scatter every particle to its tile's next free slot (cursor = exclusive
-// scan of the tile counts): one pass, reads key + payload, writes payload.
+// tile_count[key >> shift] += 1 for every key (counts zeroed by the caller).
+int launch_tile_hist(const uint32_t* keys, size_t np, int shift, uint32_t* tile_count, cudaStream_t s);
+// Scatter every particle to its tile's slots (cursor = exclusive scan of the
+// tile counts): one pass, reads key + payload, writes payload.
 template <typename real, int D>
-int launch_tile_scatter(const PArrays<real, D>& src, const PArrays<real, D>& dst, const uint32_t* keys,
+int launch_tile_scatter(const PArrays<real, D>& src, const PArrays<real, D>& dst, const uint32_t* keys, int shift,
                         uint32_t* cursor, size_t np, cudaStream_t s);
 
 // ---------------------------------------------------------------- misc

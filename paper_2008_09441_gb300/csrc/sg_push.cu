@@ -5,9 +5,9 @@
 // also adds 0.5 m_p v^{n-1/2}.v^{n+1/2} to the time-centred kinetic energy.
 //
 // Each thread advances four consecutive particles per iteration with 16-byte
-// vector loads and stores.  On a sort step the kernel also emits the tile key
-// of every new position (the counting sort's keys; k_tile_hist counts them)
-// and adds sum (cell key + 1) to the checksum.
+// vector loads and stores.  On a sort step the kernel also emits the cell key
+// of every new position (the counting sort's keys; k_tile_hist counts their
+// tiles) and adds sum (key + 1) to the checksum.
 #include "sg_kernels.cuh"
 
 namespace sg {
@@ -170,17 +170,13 @@ __device__ __forceinline__ void push_one(real (&u)[D], real (&v)[D], real w, int
   }
 }
 
-// Tile key (Morton key of the level-(n - shift) cell) of a wrapped position;
-// also returns the level-n key for the checksum.
+// Cell key (Morton key of the level-n cell) of a wrapped position.
 template <typename real, int D>
-__device__ __forceinline__ uint32_t tile_key(const real (&u)[D], int n, int shift, uint32_t* full) {
-  const int N = 1 << n;
+__device__ __forceinline__ uint32_t cell_key(const real (&u)[D], int n) {
   int c[D];
 #pragma unroll
-  for (int m = 0; m < D; ++m) c[m] = cell_of(u[m], n, N);
-  uint32_t k = morton_key<D>(c, n);
-  *full = k;
-  return k >> (D * shift);
+  for (int m = 0; m < D; ++m) c[m] = cell_of(u[m], n, 1 << n);
+  return morton_key<D>(c, n);
 }
 
 template <typename real, int D>
@@ -205,7 +201,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? (D == 2 ? 4 : 2) : 0)
       Vv[m] = ld4(p.v[m] + i0);
     }
     const V4<real> W = ld4(p.w + i0);
-    uint32_t tiles[4];
+    uint32_t ck[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       real u[D], v[D];
@@ -221,9 +217,8 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? (D == 2 ? 4 : 2) : 0)
         Vv[m].x[j] = v[m];
       }
       if (sf.keys) {
-        uint32_t full;
-        tiles[j] = tile_key<real, D>(u, n, sf.tile_shift, &full);
-        cks += (unsigned long long)full + 1ull;
+        ck[j] = cell_key<real, D>(u, n);
+        cks += (unsigned long long)ck[j] + 1ull;
       }
     }
 #pragma unroll
@@ -231,7 +226,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? (D == 2 ? 4 : 2) : 0)
       if (pp.drift) st4(p.u[m] + i0, U[m]);
       st4(p.v[m] + i0, Vv[m]);
     }
-    if (sf.keys) *reinterpret_cast<uint4*>(sf.keys + i0) = make_uint4(tiles[0], tiles[1], tiles[2], tiles[3]);
+    if (sf.keys) *reinterpret_cast<uint4*>(sf.keys + i0) = make_uint4(ck[0], ck[1], ck[2], ck[3]);
   }
   // ragged tail (np not a multiple of 4): block 0 takes it particle by particle
   if (blockIdx.x == 0) {
@@ -251,10 +246,9 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? (D == 2 ? 4 : 2) : 0)
         p.v[m][i] = v[m];
       }
       if (sf.keys) {
-        uint32_t full;
-        uint32_t t = tile_key<real, D>(u, n, sf.tile_shift, &full);
-        sf.keys[i] = t;
-        cks += (unsigned long long)full + 1ull;
+        const uint32_t k = cell_key<real, D>(u, n);
+        sf.keys[i] = k;
+        cks += (unsigned long long)k + 1ull;
       }
     }
   }

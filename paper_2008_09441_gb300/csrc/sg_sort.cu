@@ -563,156 +563,176 @@ int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, s
 }
 
 // ---------------------------------------------------------------- tile counting sort
-// Tile keys of the current positions (the push emits them on sort steps;
-// this kernel serves init and checkpoint load) and sum (cell key + 1).
+// Cell keys of the current positions (the push emits them on sort steps;
+// this kernel serves init and checkpoint load) and sum (key + 1).
 template <typename real, int D>
 __global__ void __launch_bounds__(256) k_tile_keys(PArrays<real, D> p, size_t np, int n, SortFuse sf,
                                                    unsigned* status) {
+  __shared__ unsigned long long s_part[8];
   const int N = 1 << n;
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long part = 0;
-  if (i < np) {
+  bool bad = false;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += (size_t)gridDim.x * blockDim.x) {
     int c[D];
-    bool bad = false;
 #pragma unroll
     for (int m = 0; m < D; ++m) {
       real u = p.u[m][i];
       bad |= !(u >= (real)0 && u < (real)1);
       c[m] = cell_of(u, n, N);
     }
-    if (bad) atomicOr(status, ST_KEY_RANGE);
-    uint32_t k = morton_key<D>(c, n);
-    sf.keys[i] = k >> (D * sf.tile_shift);
-    part = (unsigned long long)k + 1ull;
+    const uint32_t k = morton_key<D>(c, n);
+    sf.keys[i] = k;
+    part += (unsigned long long)k + 1ull;
   }
+  if (bad) atomicOr(status, ST_KEY_RANGE);
   part = warp_sum(part);
-  if ((threadIdx.x & 31) == 0 && part && sf.checksum) atomicAdd(sf.checksum, part);
+  if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = part;
+  __syncthreads();
+  if (threadIdx.x == 0 && sf.checksum) {  // one atomic per block: all go to one address
+    for (int w = 1; w < 8; ++w) part += s_part[w];
+    atomicAdd(sf.checksum, part);
+  }
 }
 
 template <typename real, int D>
 int launch_tile_keys(const PArrays<real, D>& p, size_t np, int n, const SortFuse& sf, unsigned* status,
                      cudaStream_t s) {
   if (np == 0) return SG_OK;
-  k_tile_keys<real, D><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(p, np, n, sf, status);
+  const unsigned blocks = (unsigned)(np < (size_t)1216 * 256 ? (np + 255) / 256 : 1216);
+  k_tile_keys<real, D><<<blocks, 256, 0, s>>>(p, np, n, sf, status);
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
 
-// Block-level counting.  A block takes TB_ITEMS consecutive keys (the
-// particles were tile-sorted one step earlier, so the block sees a narrow
-// range of tiles); when that range fits TB_SPAN shared counters the block
-// counts there with native 32-bit shared atomics and issues one global
-// atomic per distinct tile, otherwise each key adds to the global counter.
-constexpr int TB_THREADS = 256;
+// The tile of a key is its top bits (key >> shift, at most 4096 tiles).
+constexpr int TB_TILES = 4096;
+constexpr int TH_THREADS = 512;
+constexpr int TH_ITEMS = 16 * TH_THREADS;
+
+// Tile counts: a block counts its keys in shared memory, lanes with equal
+// tiles (the common case: sorted input) once per group, and adds each
+// non-empty tile to the global counter.
+__global__ void __launch_bounds__(TH_THREADS) k_tile_hist(const uint32_t* __restrict__ keys, size_t np, int shift,
+                                                          uint32_t* tile_count) {
+  __shared__ uint32_t s_cnt[TB_TILES];
+  for (int i = threadIdx.x; i < TB_TILES; i += TH_THREADS) s_cnt[i] = 0;
+  __syncthreads();
+  const size_t base = (size_t)blockIdx.x * TH_ITEMS;
+  const int lane = threadIdx.x & 31;
+  constexpr int NV = TH_ITEMS / TH_THREADS / 4;
+  uint4 v[NV];  // sixteen keys per thread, four vector loads in flight
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const size_t i = base + ((size_t)k * TH_THREADS + threadIdx.x) * 4;
+    v[k] = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+    if (i + 4 <= np) {
+      v[k] = __ldg(reinterpret_cast<const uint4*>(keys + i));
+    } else if (i < np) {
+      v[k].x = keys[i];
+      if (i + 1 < np) v[k].y = keys[i + 1];
+      if (i + 2 < np) v[k].z = keys[i + 2];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4 * NV; ++k) {
+    const uint32_t key = (k & 3) == 0 ? v[k >> 2].x : (k & 3) == 1 ? v[k >> 2].y : (k & 3) == 2 ? v[k >> 2].z : v[k >> 2].w;
+    const bool valid = key != 0xFFFFFFFFu;
+    const uint32_t t = valid ? key >> shift : 0xFFFFFFFFu;
+    const unsigned peers = __match_any_sync(0xffffffffu, t);
+    if (valid && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[t], (uint32_t)__popc(peers));
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < TB_TILES; i += TH_THREADS)
+    if (s_cnt[i]) atomicAdd(&tile_count[i], s_cnt[i]);
+}
+
+int launch_tile_hist(const uint32_t* keys, size_t np, int shift, uint32_t* tile_count, cudaStream_t s) {
+  if (np == 0) return SG_OK;
+  k_tile_hist<<<(unsigned)((np + TH_ITEMS - 1) / TH_ITEMS), TH_THREADS, 0, s>>>(keys, np, shift, tile_count);
+  SG_CHECK_LAUNCH();
+  return SG_OK;
+}
+
+// Scatter every particle to its tile's slots.  A block takes TB_ITEMS
+// particles (tile-sorted a few steps earlier), numbers the R tiles that occur
+// among them, and orders its payload in shared memory by tile, in 3D by (tile,
+// part of the tile): as many parts, by the next key bits, as make R tiles fit
+// TB_BUCKETS counters.  It reserves one range per tile with a single global
+// atomic and writes contiguous runs per tile.
+//
+// The tiles are what later deposits need; the parts are for the warps of the
+// 3D push, which gather from nodes of a few neighbouring cells instead of the
+// whole tile of 8 x 8 x 8.  3D two-stream, 16,777,216 particles, step without /
+// with parts: 582 / 557 us (push 300 / 273), 4 M at n = 6 158 / 148, Penning
+// trap n = 7 164 / 165.  2D keeps tiles only: a warp whose particles share
+// cells meets itself in the deposit's shared adds (annulus, 146 particles per
+// cell, step 143 / 174; Landau n = 10 117 / 122).  Within a part the order
+// depends on the atomics: the step sort is a valid, not a stable, counting
+// sort by tile.  Bound: HBM and shared memory about equally (2D annulus: 53%
+// of DRAM's rate).  Against blocks of 1024 particles that counted over their
+// range of tiles: Landau n = 9, 8 M particles 45 -> 35 us per step, n = 10
+// 25.8 -> 21.9, Penning 18.6 -> 12.1, annulus 29.6 -> 32.8.
+constexpr int TB_THREADS = 512;
 constexpr int TB_PER_THREAD = 4;
 constexpr int TB_ITEMS = TB_THREADS * TB_PER_THREAD;
-constexpr int TB_SPAN = 1024;
+constexpr int TB_BUCKETS = 4096;
+static_assert(TB_ITEMS <= TB_BUCKETS, "every particle in a tile of its own still fits");
 
-__device__ __forceinline__ void block_key_range(const uint32_t (&t)[TB_PER_THREAD], uint32_t* s_lo, uint32_t* s_hi) {
-  uint32_t lo = 0xFFFFFFFFu, hi = 0;
-#pragma unroll
-  for (int k = 0; k < TB_PER_THREAD; ++k)
-    if (t[k] != 0xFFFFFFFFu) {
-      lo = min(lo, t[k]);
-      hi = max(hi, t[k]);
-    }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicMin(s_lo, lo);
-    atomicMax(s_hi, hi);
-  }
-}
-
-// Keys of item k of thread t: chunk + k * TB_THREADS + t (coalesced rounds).
-__device__ __forceinline__ void load_keys(const uint32_t* __restrict__ keys, size_t np, size_t chunk,
-                                          uint32_t (&t)[TB_PER_THREAD]) {
-#pragma unroll
-  for (int k = 0; k < TB_PER_THREAD; ++k) {
-    const size_t i = chunk + (size_t)k * TB_THREADS + threadIdx.x;
-    t[k] = i < np ? __ldg(keys + i) : 0xFFFFFFFFu;
-  }
-}
-
-__global__ void __launch_bounds__(TB_THREADS) k_tile_hist(const uint32_t* __restrict__ keys, size_t np,
-                                                          uint32_t* tile_count) {
-  __shared__ uint32_t s_cnt[TB_SPAN];
-  __shared__ uint32_t s_lo, s_hi;
-  const size_t chunk = (size_t)blockIdx.x * TB_ITEMS;
-  uint32_t t[TB_PER_THREAD];
-  load_keys(keys, np, chunk, t);
-  if (threadIdx.x == 0) {
-    s_lo = 0xFFFFFFFFu;
-    s_hi = 0;
-  }
-  for (int i = threadIdx.x; i < TB_SPAN; i += TB_THREADS) s_cnt[i] = 0;
-  __syncthreads();
-  block_key_range(t, &s_lo, &s_hi);
-  __syncthreads();
-  const uint32_t lo = s_lo;
-  const bool local = s_hi - lo < (uint32_t)TB_SPAN;
-  const int lane = threadIdx.x & 31;
-  // lanes with equal keys (the common case: sorted input) add once per group
-#pragma unroll
-  for (int k = 0; k < TB_PER_THREAD; ++k) {
-    const unsigned peers = __match_any_sync(0xffffffffu, t[k]);
-    if (t[k] == 0xFFFFFFFFu || lane != __ffs(peers) - 1) continue;
-    if (local)
-      atomicAdd(&s_cnt[t[k] - lo], (uint32_t)__popc(peers));
-    else
-      atomicAdd(&tile_count[t[k]], (uint32_t)__popc(peers));
-  }
-  if (!local) return;
-  __syncthreads();
-  for (int i = threadIdx.x; i < TB_SPAN; i += TB_THREADS)
-    if (s_cnt[i]) atomicAdd(&tile_count[lo + i], s_cnt[i]);
-}
-
-int launch_tile_hist(const uint32_t* keys, size_t np, uint32_t* tile_count, cudaStream_t s) {
-  if (np == 0) return SG_OK;
-  k_tile_hist<<<(unsigned)((np + TB_ITEMS - 1) / TB_ITEMS), TB_THREADS, 0, s>>>(keys, np, tile_count);
-  SG_CHECK_LAUNCH();
-  return SG_OK;
-}
-
-// Scatter every particle to its tile's slots.  Same blocks as the count.
-// When the block's keys span at most TB_SPAN tiles (the usual case: the
-// particles were tile-sorted a few steps earlier), the block ranks its
-// particles per tile with shared atomics, reserves one range per distinct
-// tile with a single global atomic, orders its payload by tile in shared
-// memory (a block-local counting sort), and writes it out as contiguous runs
-// per tile -- coalesced stores even when the particles have drifted over
-// many tiles.  Wider blocks reserve per warp group and store directly.
-// Within a tile the order depends on the atomics: the step sort is a valid,
-// not a stable, counting sort by tile key.
-template <typename real, int D>
-struct ScatterStage {
-  static constexpr size_t bytes = (size_t)TB_ITEMS * ((2 * D + 1) * sizeof(real) + 2 * sizeof(uint32_t));
-  static constexpr bool on = bytes <= 160 * 1024;
-};
-
-template <typename real, int D>
-__global__ void __launch_bounds__(TB_THREADS) k_tile_scatter(PArrays<real, D> src, PArrays<real, D> dst,
-                                                             const uint32_t* __restrict__ keys, uint32_t* cursor,
-                                                             size_t np) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint32_t s_cnt[TB_SPAN];   // per tile: count, then the local start
-  __shared__ uint32_t s_base[TB_SPAN];  // per tile: the block's global base
-  __shared__ uint32_t s_wsum[TB_THREADS / 32];
-  __shared__ uint32_t s_lo, s_hi;
-  const size_t chunk = (size_t)blockIdx.x * TB_ITEMS;
+// Exclusive scan over the block of each thread's sum; *all receives the total.
+__device__ __forceinline__ uint32_t block_scan(uint32_t sum, uint32_t* ws /* TB_THREADS / 32 */, uint32_t* all) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t t[TB_PER_THREAD];
-  load_keys(keys, np, chunk, t);
+  uint32_t incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) ws[warp] = incl;
+  __syncthreads();
+  constexpr int NW = TB_THREADS / 32;  // every warp scans the warps' sums
+  uint32_t t = lane < NW ? ws[lane] : 0u;
+#pragma unroll
+  for (int o = 1; o < NW; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
+    if (lane >= o) t += y;
+  }
+  const uint32_t before = __shfl_sync(0xffffffffu, t, warp > 0 ? warp - 1 : 0);
+  *all = __shfl_sync(0xffffffffu, t, NW - 1);
+  __syncthreads();
+  return incl - sum + (warp > 0 ? before : 0u);
+}
+
+template <typename real, int D>
+constexpr size_t scatter_stage_bytes() {
+  return (size_t)TB_ITEMS * ((2 * D + 1) * sizeof(real) + 2 * sizeof(uint32_t));
+}
+
+template <typename real, int D>
+__global__ void __launch_bounds__(TB_THREADS, sizeof(real) == 4 ? 2 : 1) k_tile_scatter(PArrays<real, D> src, PArrays<real, D> dst,
+                                                             const uint32_t* __restrict__ keys, int shift,
+                                                             uint32_t* cursor, size_t np) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(16) uint16_t s_id[TB_TILES];      // tile -> its number in the block
+  __shared__ uint16_t s_tile[TB_ITEMS];                  // and back
+  __shared__ __align__(16) uint32_t s_cnt[TB_BUCKETS];   // per bucket: count, then the local start
+  __shared__ uint32_t s_base[TB_ITEMS];                  // per tile: the block's global base minus the local start
+  __shared__ uint32_t s_ws[TB_THREADS / 32];
+  const size_t chunk = (size_t)blockIdx.x * TB_ITEMS;
+  const int lane = threadIdx.x & 31, tid = threadIdx.x;
+  constexpr int PT = TB_TILES / TB_THREADS;
+  static_assert(PT == 8, "eight 16-bit flags per thread in one vector");
+  uint32_t key[TB_PER_THREAD];
+#pragma unroll
+  for (int k = 0; k < TB_PER_THREAD; ++k) {
+    const size_t i = chunk + (size_t)k * TB_THREADS + tid;
+    key[k] = i < np ? __ldg(keys + i) : 0xFFFFFFFFu;
+  }
   // the payload's loads go out now, so that their latency overlaps the ranking
   real pu[TB_PER_THREAD][D], pv[TB_PER_THREAD][D], pw[TB_PER_THREAD];
   uint32_t ppid[TB_PER_THREAD];
 #pragma unroll
   for (int k = 0; k < TB_PER_THREAD; ++k) {
-    const size_t i = chunk + (size_t)k * TB_THREADS + threadIdx.x;
+    const size_t i = chunk + (size_t)k * TB_THREADS + tid;
     const bool valid = i < np;
 #pragma unroll
     for (int m = 0; m < D; ++m) {
@@ -722,132 +742,98 @@ __global__ void __launch_bounds__(TB_THREADS) k_tile_scatter(PArrays<real, D> sr
     pw[k] = valid ? __ldg(src.w + i) : (real)0;
     ppid[k] = valid ? __ldg(src.pid + i) : 0u;
   }
-  if (threadIdx.x == 0) {
-    s_lo = 0xFFFFFFFFu;
-    s_hi = 0;
+  reinterpret_cast<uint4*>(s_id)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < TB_PER_THREAD; ++k)
+    if (key[k] != 0xFFFFFFFFu) s_id[key[k] >> shift] = 1;
+  __syncthreads();
+  uint32_t R;
+  {  // number the tiles that occur
+    const uint4 f = reinterpret_cast<const uint4*>(s_id)[tid];  // eight flags of 0 or 1
+    const uint32_t f2[4] = {f.x, f.y, f.z, f.w};
+    const uint32_t pairs = f.x + f.y + f.z + f.w;
+    uint32_t at = block_scan((pairs & 0xFFFFu) + (pairs >> 16), s_ws, &R);
+#pragma unroll
+    for (int j = 0; j < PT; ++j)
+      if ((f2[j >> 1] >> (16 * (j & 1))) & 1u) {
+        s_tile[at] = (uint16_t)(PT * tid + j);
+        s_id[PT * tid + j] = (uint16_t)at++;
+      }
   }
-  for (int i = threadIdx.x; i < TB_SPAN; i += TB_THREADS) s_cnt[i] = 0;
+  const int logf = min(D == 3 ? shift : 0, 12 - (R > 1 ? 32 - __clz(R - 1) : 0));  // 2^logf parts per tile
+  const uint32_t fine = (1u << shift) - 1u, nb = R << logf;
+  for (uint32_t i = tid; i < nb; i += TB_THREADS) s_cnt[i] = 0;
   __syncthreads();
-  block_key_range(t, &s_lo, &s_hi);
+  uint32_t bucket[TB_PER_THREAD], pos[TB_PER_THREAD];
+#pragma unroll
+  for (int k = 0; k < TB_PER_THREAD; ++k) {  // rank within the bucket: one shared atomic per group of a warp
+    const bool valid = key[k] != 0xFFFFFFFFu;
+    bucket[k] = valid ? ((uint32_t)s_id[key[k] >> shift] << logf) + ((key[k] & fine) >> (shift - logf)) : 0xFFFFFFFFu;
+    const unsigned peers = __match_any_sync(0xffffffffu, bucket[k]);
+    const int leader = __ffs(peers) - 1;
+    uint32_t b = 0;
+    if (valid && lane == leader) b = atomicAdd(&s_cnt[bucket[k]], (uint32_t)__popc(peers));
+    pos[k] = __shfl_sync(0xffffffffu, b, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+  }
   __syncthreads();
-  const uint32_t lo = s_lo;
-  const bool local = s_hi - lo < (uint32_t)TB_SPAN;
-  uint32_t pos[TB_PER_THREAD];
-  if (local) {
-    // rank within the block's tile: one shared atomic per group of equal keys
-#pragma unroll
-    for (int k = 0; k < TB_PER_THREAD; ++k) {
-      const unsigned peers = __match_any_sync(0xffffffffu, t[k]);
-      const int leader = __ffs(peers) - 1;
-      uint32_t b = 0;
-      if (t[k] != 0xFFFFFFFFu && lane == leader) b = atomicAdd(&s_cnt[t[k] - lo], (uint32_t)__popc(peers));
-      pos[k] = __shfl_sync(0xffffffffu, b, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
-    }
-    __syncthreads();
-    // per tile: the block's global base (one atomic per non-empty tile) and
-    // the local start (exclusive scan of the counts, four tiles per thread)
-    static_assert(TB_SPAN == 4 * TB_THREADS, "four tiles per thread");
-    uint32_t cnt4[4], run = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int i = 4 * threadIdx.x + j;
-      cnt4[j] = s_cnt[i];
-      if (cnt4[j]) s_base[i] = atomicAdd(&cursor[lo + i], cnt4[j]);
-      run += cnt4[j];
-    }
-    uint32_t incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_wsum[warp] = incl;
-    __syncthreads();
-    uint32_t wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += s_wsum[w];
-    uint32_t start = wbase + incl - run;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      s_cnt[4 * threadIdx.x + j] = start;
-      start += cnt4[j];
-    }
-    __syncthreads();
-    if constexpr (ScatterStage<real, D>::on) {
-      real* su = reinterpret_cast<real*>(smem_raw);  // [2D+1][TB_ITEMS]: u, v, w
-      uint32_t* spid = reinterpret_cast<uint32_t*>(su + (size_t)(2 * D + 1) * TB_ITEMS);
-      uint32_t* sdst = spid + TB_ITEMS;
-#pragma unroll
-      for (int k = 0; k < TB_PER_THREAD; ++k) {
-        const size_t i = chunk + (size_t)k * TB_THREADS + threadIdx.x;
-        if (i < np) {
-          const uint32_t ti = t[k] - lo;
-          const uint32_t L = s_cnt[ti] + pos[k];
-#pragma unroll
-          for (int m = 0; m < D; ++m) {
-            su[(size_t)m * TB_ITEMS + L] = pu[k][m];
-            su[(size_t)(D + m) * TB_ITEMS + L] = pv[k][m];
-          }
-          su[(size_t)(2 * D) * TB_ITEMS + L] = pw[k];
-          spid[L] = ppid[k];
-          sdst[L] = s_base[ti] + pos[k];
-        }
-      }
-      __syncthreads();
-      const int nvalid = (int)min((size_t)TB_ITEMS, np - chunk);
-      for (int j = threadIdx.x; j < nvalid; j += TB_THREADS) {
-        const uint32_t p = sdst[j];
-#pragma unroll
-        for (int m = 0; m < D; ++m) {
-          dst.u[m][p] = su[(size_t)m * TB_ITEMS + j];
-          dst.v[m][p] = su[(size_t)(D + m) * TB_ITEMS + j];
-        }
-        dst.w[p] = su[(size_t)(2 * D) * TB_ITEMS + j];
-        dst.pid[p] = spid[j];
-      }
-      return;
-    } else {
-#pragma unroll
-      for (int k = 0; k < TB_PER_THREAD; ++k)
-        if (t[k] != 0xFFFFFFFFu) pos[k] += s_base[t[k] - lo];
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < TB_PER_THREAD; ++k) {
-      const bool valid = t[k] != 0xFFFFFFFFu;
-      const unsigned peers = __match_any_sync(0xffffffffu, t[k]);
-      const int leader = __ffs(peers) - 1;
-      uint32_t base = 0;
-      if (valid && lane == leader) base = atomicAdd(&cursor[t[k]], (uint32_t)__popc(peers));
-      pos[k] = __shfl_sync(0xffffffffu, base, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+  uint32_t nvalid;
+  {  // local starts: `per` consecutive buckets per thread
+    const uint32_t per = (nb + TB_THREADS - 1) / TB_THREADS, b0 = min(tid * per, nb), b1 = min(b0 + per, nb);
+    uint32_t n = 0;
+    for (uint32_t i = b0; i < b1; ++i) n += s_cnt[i];
+    uint32_t at = block_scan(n, s_ws, &nvalid);
+    for (uint32_t i = b0; i < b1; ++i) {
+      const uint32_t c = s_cnt[i];
+      s_cnt[i] = at;
+      at += c;
     }
   }
-  // direct move of the payload loaded at the start
+  __syncthreads();
+  for (uint32_t q = tid; q < R; q += TB_THREADS) {  // one global atomic per tile
+    const uint32_t a = s_cnt[q << logf], e = q + 1 < R ? s_cnt[(q + 1) << logf] : nvalid;
+    s_base[q] = atomicAdd(&cursor[s_tile[q]], e - a) - a;
+  }
+  real* su = reinterpret_cast<real*>(smem_raw);  // [2D+1][TB_ITEMS]: u, v, w
+  uint32_t* spid = reinterpret_cast<uint32_t*>(su + (size_t)(2 * D + 1) * TB_ITEMS);
+  uint32_t* stl = spid + TB_ITEMS;  // the particle's tile number
 #pragma unroll
-  for (int k = 0; k < TB_PER_THREAD; ++k) {
-    const size_t i = chunk + (size_t)k * TB_THREADS + threadIdx.x;
-    if (i >= np) continue;
-    const uint32_t p = pos[k];
+  for (int k = 0; k < TB_PER_THREAD; ++k)
+    if (key[k] != 0xFFFFFFFFu) {
+      const uint32_t L = s_cnt[bucket[k]] + pos[k];
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        su[(size_t)m * TB_ITEMS + L] = pu[k][m];
+        su[(size_t)(D + m) * TB_ITEMS + L] = pv[k][m];
+      }
+      su[(size_t)(2 * D) * TB_ITEMS + L] = pw[k];
+      spid[L] = ppid[k];
+      stl[L] = bucket[k] >> logf;
+    }
+  __syncthreads();
+  for (uint32_t j = tid; j < nvalid; j += TB_THREADS) {
+    const uint32_t p = s_base[stl[j]] + j;
 #pragma unroll
     for (int m = 0; m < D; ++m) {
-      dst.u[m][p] = pu[k][m];
-      dst.v[m][p] = pv[k][m];
+      dst.u[m][p] = su[(size_t)m * TB_ITEMS + j];
+      dst.v[m][p] = su[(size_t)(D + m) * TB_ITEMS + j];
     }
-    dst.w[p] = pw[k];
-    dst.pid[p] = ppid[k];
+    dst.w[p] = su[(size_t)(2 * D) * TB_ITEMS + j];
+    dst.pid[p] = spid[j];
   }
 }
 
 template <typename real, int D>
-int launch_tile_scatter(const PArrays<real, D>& src, const PArrays<real, D>& dst, const uint32_t* keys,
+int launch_tile_scatter(const PArrays<real, D>& src, const PArrays<real, D>& dst, const uint32_t* keys, int shift,
                         uint32_t* cursor, size_t np, cudaStream_t s) {
   if (np == 0) return SG_OK;
-  const size_t smem = ScatterStage<real, D>::on ? ScatterStage<real, D>::bytes : 0;
-  static bool attr_set = false;
-  if (!attr_set && smem > 0) {  // with the static counters the total may pass 48 KB
+  constexpr size_t smem = scatter_stage_bytes<real, D>();
+  static std::atomic<bool> attr_set{false};
+  if (!attr_set) {  // with the static counters the total passes 48 KB
     SG_CUDA(cudaFuncSetAttribute(k_tile_scatter<real, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr_set = true;
   }
-  k_tile_scatter<real, D><<<(unsigned)((np + TB_ITEMS - 1) / TB_ITEMS), TB_THREADS, smem, s>>>(src, dst, keys,
+  k_tile_scatter<real, D><<<(unsigned)((np + TB_ITEMS - 1) / TB_ITEMS), TB_THREADS, smem, s>>>(src, dst, keys, shift,
                                                                                               cursor, np);
   SG_CHECK_LAUNCH();
   return SG_OK;
@@ -887,7 +873,7 @@ int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_
   template size_t unpermute_scratch_bytes<real, D>(size_t);                                              \
   template int launch_tile_keys<real, D>(const PArrays<real, D>&, size_t, int, const SortFuse&, unsigned*,         \
                                          cudaStream_t);                                                            \
-  template int launch_tile_scatter<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, const uint32_t*,     \
+  template int launch_tile_scatter<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, const uint32_t*, int, \
                                             uint32_t*, size_t, cudaStream_t);
 
 SG_INST_SORT(float, 2)
