@@ -5,9 +5,10 @@
 // also adds 0.5 m_p v^{n-1/2}.v^{n+1/2} to the time-centred kinetic energy.
 //
 // Each thread advances four consecutive particles per iteration with 16-byte
-// vector loads and stores.  On a sort step the kernel also emits the cell key
-// of every new position (the counting sort's keys; k_tile_hist counts their
-// tiles) and adds sum (key + 1) to the checksum.
+// vector loads and stores; in 3D FP32 two, a warp's width apart.  On a sort
+// step the kernel also emits the cell key of every new position (the counting
+// sort's keys; k_tile_hist counts their tiles) and adds sum (key + 1) to the
+// checksum.
 #include "sg_kernels.cuh"
 
 namespace sg {
@@ -179,8 +180,22 @@ __device__ __forceinline__ uint32_t cell_key(const real (&u)[D], int n) {
   return morton_key<D>(c, n);
 }
 
+// The 3D FP32 push is bound by the gather's passes through L1 (eight 16-byte
+// node records a particle; 73% of that pipe's rate with 24% of the warps
+// resident).  Consecutive particles in consecutive lanes and two particles
+// per thread in 64 registers double the resident warps: 16.7M two-stream
+// particles at n = 7 273 -> 254 us, 2.1M in a Penning trap 48.2 -> 47.8.  Four
+// per thread in 85 registers: 252 and 50.2.  In 2D (8-byte records) the same
+// layout costs 4 to 30%, in registers and in four times the requests for the
+// particles, so the quads stay there, and in FP64.
 template <typename real, int D>
-__global__ void __launch_bounds__(256, sizeof(real) == 4 ? (D == 2 ? 4 : 2) : 0) k_push(PArrays<real, D> p, size_t np, int n, const real* __restrict__ Ec,
+constexpr bool push_lanes() {
+  return sizeof(real) == 4 && D == 3;
+}
+constexpr int PUSH_LANE_ITEMS = 2;
+
+template <typename real, int D>
+__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 0) k_push(PArrays<real, D> p, size_t np, int n, const real* __restrict__ Ec,
                                               PushParams<real> pp, double* __restrict__ ke_partials,
                                               unsigned* status, SortFuse sf) {
   __shared__ double red[32];
@@ -190,47 +205,87 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? (D == 2 ? 4 : 2) : 0)
   KeAcc<real> ke;
   bool bad = false;
   unsigned long long cks = 0;
-  const size_t nvec = np >> 2;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t iv = (size_t)blockIdx.x * blockDim.x + threadIdx.x; iv < nvec; iv += stride) {
-    const size_t i0 = iv << 2;
-    V4<real> U[D], Vv[D];
-#pragma unroll
-    for (int m = 0; m < D; ++m) {
-      U[m] = ld4(p.u[m] + i0);
-      Vv[m] = ld4(p.v[m] + i0);
-    }
-    const V4<real> W = ld4(p.w + i0);
-    uint32_t ck[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      real u[D], v[D];
+  size_t done;  // particles taken in whole groups
+  if constexpr (push_lanes<real, D>()) {
+    constexpr int ITEMS = PUSH_LANE_ITEMS;
+    constexpr int GROUP = 32 * ITEMS;  // one warp and iteration
+    const size_t ngroups = np / GROUP;
+    done = ngroups * GROUP;
+    const size_t stride = (size_t)gridDim.x * (blockDim.x >> 5);
+    for (size_t g = (size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); g < ngroups; g += stride) {
+      const size_t i0 = g * GROUP + (threadIdx.x & 31);
+      real U[ITEMS][D], V[ITEMS][D], W[ITEMS];
 #pragma unroll
       for (int m = 0; m < D; ++m) {
-        u[m] = U[m].x[j];
-        v[m] = Vv[m].x[j];
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+          U[j][m] = p.u[m][i0 + 32 * j];
+          V[j][m] = p.v[m][i0 + 32 * j];
+        }
       }
-      push_one<real, D>(u, v, W.x[j], n, Ec, ND, pp, ke, bad);
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) W[j] = p.w[i0 + 32 * j];
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        push_one<real, D>(U[j], V[j], W[j], n, Ec, ND, pp, ke, bad);
+        if (sf.keys) {
+          const uint32_t k = cell_key<real, D>(U[j], n);
+          sf.keys[i0 + 32 * j] = k;
+          cks += (unsigned long long)k + 1ull;
+        }
+      }
 #pragma unroll
       for (int m = 0; m < D; ++m) {
-        U[m].x[j] = u[m];
-        Vv[m].x[j] = v[m];
-      }
-      if (sf.keys) {
-        ck[j] = cell_key<real, D>(u, n);
-        cks += (unsigned long long)ck[j] + 1ull;
-      }
-    }
 #pragma unroll
-    for (int m = 0; m < D; ++m) {
-      if (pp.drift) st4(p.u[m] + i0, U[m]);
-      st4(p.v[m] + i0, Vv[m]);
+        for (int j = 0; j < ITEMS; ++j) {
+          if (pp.drift) p.u[m][i0 + 32 * j] = U[j][m];
+          p.v[m][i0 + 32 * j] = V[j][m];
+        }
+      }
     }
-    if (sf.keys) *reinterpret_cast<uint4*>(sf.keys + i0) = make_uint4(ck[0], ck[1], ck[2], ck[3]);
+  } else {
+    done = np & ~(size_t)3;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t iv = (size_t)blockIdx.x * blockDim.x + threadIdx.x; iv < (np >> 2); iv += stride) {
+      const size_t i0 = iv << 2;
+      V4<real> U[D], Vv[D];
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        U[m] = ld4(p.u[m] + i0);
+        Vv[m] = ld4(p.v[m] + i0);
+      }
+      const V4<real> W = ld4(p.w + i0);
+      uint32_t ck[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        real u[D], v[D];
+#pragma unroll
+        for (int m = 0; m < D; ++m) {
+          u[m] = U[m].x[j];
+          v[m] = Vv[m].x[j];
+        }
+        push_one<real, D>(u, v, W.x[j], n, Ec, ND, pp, ke, bad);
+#pragma unroll
+        for (int m = 0; m < D; ++m) {
+          U[m].x[j] = u[m];
+          Vv[m].x[j] = v[m];
+        }
+        if (sf.keys) {
+          ck[j] = cell_key<real, D>(u, n);
+          cks += (unsigned long long)ck[j] + 1ull;
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        if (pp.drift) st4(p.u[m] + i0, U[m]);
+        st4(p.v[m] + i0, Vv[m]);
+      }
+      if (sf.keys) *reinterpret_cast<uint4*>(sf.keys + i0) = make_uint4(ck[0], ck[1], ck[2], ck[3]);
+    }
   }
-  // ragged tail (np not a multiple of 4): block 0 takes it particle by particle
+  // the ragged tail (at most 63 particles): block 0, one per thread
   if (blockIdx.x == 0) {
-    const size_t i = (nvec << 2) + threadIdx.x;
+    const size_t i = done + threadIdx.x;
     const bool valid = i < np;
     if (valid) {
       real u[D], v[D];
