@@ -609,9 +609,12 @@ constexpr int TB_TILES = 4096;
 constexpr int TH_THREADS = 512;
 constexpr int TH_ITEMS = 16 * TH_THREADS;
 
-// Tile counts: a block counts its keys in shared memory, lanes with equal
-// tiles (the common case: sorted input) once per group, and adds each
-// non-empty tile to the global counter.
+// Tile counts: a block counts its keys in shared memory and adds each
+// non-empty tile to the global counter.  Four consecutive keys of one tile
+// (the common case: input sorted a few steps earlier) count once per group of
+// lanes of that tile, the others one by one.  Matching every key's lanes
+// instead: the sort per step, one sort in four, 2D n = 9, 8 M particles 36 ->
+// 32 us, n = 10, 4 M 22.4 -> 19.7, 3D n = 7, 16.7 M 61.6 -> 60.5.
 __global__ void __launch_bounds__(TH_THREADS) k_tile_hist(const uint32_t* __restrict__ keys, size_t np, int shift,
                                                           uint32_t* tile_count) {
   __shared__ uint32_t s_cnt[TB_TILES];
@@ -634,12 +637,18 @@ __global__ void __launch_bounds__(TH_THREADS) k_tile_hist(const uint32_t* __rest
     }
   }
 #pragma unroll
-  for (int k = 0; k < 4 * NV; ++k) {
-    const uint32_t key = (k & 3) == 0 ? v[k >> 2].x : (k & 3) == 1 ? v[k >> 2].y : (k & 3) == 2 ? v[k >> 2].z : v[k >> 2].w;
-    const bool valid = key != 0xFFFFFFFFu;
-    const uint32_t t = valid ? key >> shift : 0xFFFFFFFFu;
-    const unsigned peers = __match_any_sync(0xffffffffu, t);
-    if (valid && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[t], (uint32_t)__popc(peers));
+  for (int k = 0; k < NV; ++k) {
+    const uint32_t t[4] = {v[k].x >> shift, v[k].y >> shift, v[k].z >> shift, v[k].w >> shift};
+    const bool whole = v[k].w != 0xFFFFFFFFu && t[0] == t[1] && t[1] == t[2] && t[2] == t[3];
+    const unsigned peers = __match_any_sync(0xffffffffu, whole ? t[0] : 0xFFFFFFFFu);
+    if (whole) {
+      if (lane == __ffs(peers) - 1) atomicAdd(&s_cnt[t[0]], 4u * (uint32_t)__popc(peers));
+    } else {
+      if (v[k].x != 0xFFFFFFFFu) atomicAdd(&s_cnt[t[0]], 1u);
+      if (v[k].y != 0xFFFFFFFFu) atomicAdd(&s_cnt[t[1]], 1u);
+      if (v[k].z != 0xFFFFFFFFu) atomicAdd(&s_cnt[t[2]], 1u);
+      if (v[k].w != 0xFFFFFFFFu) atomicAdd(&s_cnt[t[3]], 1u);
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < TB_TILES; i += TH_THREADS)
