@@ -1535,6 +1535,9 @@ class Engine final : public EngineBase {
       boris |= cfg_.B[m] != 0.0;
       eext |= (m < D && cfg_.eext_lin[m] != 0.0);
     }
+    const real tt = D == 2 ? pp.tB[2] * pp.tB[2]
+                           : std::fma(pp.tB[2], pp.tB[2], std::fma(pp.tB[1], pp.tB[1], pp.tB[0] * pp.tB[0]));
+    for (int m = 0; m < 3; ++m) pp.sB[m] = (real)2 * pp.tB[m] / ((real)1 + tt);
     pp.boris = boris ? 1 : 0;
     pp.has_eext = eext ? 1 : 0;
     pp.drift = drift ? 1 : 0;

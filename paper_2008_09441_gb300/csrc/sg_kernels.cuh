@@ -301,6 +301,7 @@ struct PushParams {
   real dt_over_L[3];
   real eext[3];   // E_ext,m = eext[m] * (u_m - 1/2)   (eext = Eext_lin * L)
   real tB[3];     // q/m * B * dt / 2 (Boris t vector)
+  real sB[3];     // 2 t / (1 + t . t); 2D: only t_z turns the plane's velocities
   int boris;
   int has_eext;
   int drift;      // 0: velocity only (initial half kick), 1: kick + drift

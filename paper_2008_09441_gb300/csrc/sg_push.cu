@@ -133,16 +133,14 @@ __device__ __forceinline__ void push_one(real (&u)[D], real (&v)[D], real w, int
   if (pp.boris) {
     if (D == 2) {
       const real tz = pp.tB[2];
-      const real sz = (real)2 * tz / ((real)1 + tz * tz);
+      const real sz = pp.sB[2];
       const real px = vm[0] + vm[1] * tz;
       const real py = vm[1] - vm[0] * tz;
       vm[0] = vm[0] + py * sz;
       vm[1] = vm[1] - px * sz;
     } else {
       const real t0 = pp.tB[0], t1 = pp.tB[1], t2 = pp.tB[2];
-      const real tt = t0 * t0 + t1 * t1 + t2 * t2;
-      const real s0 = (real)2 * t0 / ((real)1 + tt), s1 = (real)2 * t1 / ((real)1 + tt),
-                 s2 = (real)2 * t2 / ((real)1 + tt);
+      const real s0 = pp.sB[0], s1 = pp.sB[1], s2 = pp.sB[2];
       const real a0 = vm[0], a1 = vm[1], a2 = vm[D - 1];
       const real p0 = a0 + (a1 * t2 - a2 * t1);
       const real p1 = a1 + (a2 * t0 - a0 * t2);
