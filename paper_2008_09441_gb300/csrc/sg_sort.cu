@@ -672,7 +672,7 @@ int launch_tile_hist(const uint32_t* keys, size_t np, int shift, uint32_t* tile_
 // The tiles are what later deposits need; the parts are for the warps of the
 // 3D push, which gather from nodes of a few neighbouring cells instead of the
 // whole tile of 8 x 8 x 8.  3D two-stream, 16,777,216 particles, step without /
-// with parts: 582 / 557 us (push 300 / 273), 4 M at n = 6 158 / 148, Penning
+// with parts: 582 / 557 us (push, then four particles per thread, 300 / 273), 4 M at n = 6 158 / 148, Penning
 // trap n = 7 164 / 165.  2D keeps tiles only: a warp whose particles share
 // cells meets itself in the deposit's shared adds (annulus, 146 particles per
 // cell, step 143 / 174; Landau n = 10 117 / 122).  Within a part the order
