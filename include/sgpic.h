@@ -194,7 +194,11 @@ int sg_pic_diagnostics_collect(sg_pic* h, sg_diag* out);
 int sg_pic_select_tau(sg_pic* h, int* tau, double* est_grid, double* est_noise, int cap);
 
 /* Switch the truncation parameter (1..n) for the following steps: rebuilds
- * the component-grid set and re-deposits / re-solves the current state. */
+ * the component-grid set and re-deposits / re-solves the current state.
+ * SG_ERR_OOM leaves the run without a grid set: calls that need one return
+ * SG_ERR_STATE until sg_pic_set_tau or sg_pic_load succeeds.  The same after
+ * an adaptive step that could not get its new tau's arrays; that step is then
+ * finished by sg_pic_set_tau and sg_pic_step_fields. */
 int sg_pic_set_tau(sg_pic* h, int tau);
 
 /* Copy particle states to caller buffers in the ORIGINAL particle order

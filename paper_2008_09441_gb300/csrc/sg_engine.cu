@@ -326,6 +326,7 @@ class Engine final : public EngineBase {
       set_error("sg_pic_start: the run was not created by sg_pic_init_deferred, or has started");
       return SG_ERR_STATE;
     }
+    SG_TRY(need_grids("sg_pic_start"));
     SG_TRY(enqueue_restrict_solve_combine());
     if (!filter_) {
       SG_TRY(tune_solve());
@@ -342,6 +343,7 @@ class Engine final : public EngineBase {
                           : "sg_pic_step_deposit: the run is not between steps");
       return adaptive_ ? SG_ERR_UNSUPPORTED : SG_ERR_STATE;
     }
+    SG_TRY(need_grids("sg_pic_step_deposit"));
     const bool do_sort = ((step_ + 1) % sort_every_) == 0;
     const unsigned long long l0 = launches_so_far();
     SG_TRY(enqueue_push(cfg_.dt, true, ke_partials_, do_sort));
@@ -356,6 +358,7 @@ class Engine final : public EngineBase {
       set_error("sg_pic_step_fields: sg_pic_step_deposit must come first");
       return SG_ERR_STATE;
     }
+    SG_TRY(need_grids("sg_pic_step_fields"));
     const unsigned long long l0 = launches_so_far();
     SG_TRY(enqueue_restrict_solve_combine(ke_partials_));
     launches_ += launches_so_far() - l0;
@@ -396,6 +399,7 @@ class Engine final : public EngineBase {
                                       : "sg_pic_step: finish the split step with sg_pic_step_fields first");
       return SG_ERR_STATE;
     }
+    SG_TRY(need_grids("sg_pic_step"));
     if (profiling_) std::fill(stage_ms_, stage_ms_ + 6, 0.0);
     for (int k = 0; k < nsteps; ++k) {
       bool do_sort = ((step_ + 1) % sort_every_) == 0;
@@ -496,6 +500,7 @@ class Engine final : public EngineBase {
   }
 
   int diagnostics(sg_diag* out) override {
+    SG_TRY(need_grids("sg_pic_diagnostics"));
     // one synchronisation for the whole record
     SG_TRY(ensure_pinned(&diag_host_, &diag_host_bytes_, diag_bytes()));
     char* h = static_cast<char*>(diag_host_);
@@ -507,6 +512,7 @@ class Engine final : public EngineBase {
   // Pipelined diagnostics: records enqueued into a ring of pinned slots and
   // read in order, so that a monitor reads step k while step k+1 runs.
   int diagnostics_post() override {
+    SG_TRY(need_grids("sg_pic_diagnostics_post"));
     if (ring_count_ == kDiagRing) {
       set_error("sg_pic_diagnostics_post: every slot holds a record not yet collected");
       return SG_ERR_STATE;
@@ -618,7 +624,7 @@ class Engine final : public EngineBase {
       set_error("sg_pic_set_tau: tau outside [1, n]");
       return SG_ERR_INVALID;
     }
-    if (tau == tau_) return SG_OK;
+    if (tau == tau_ && grids_ok_) return SG_OK;
     SG_CUDA(cudaStreamSynchronize(stream_));
     SG_TRY(build_grid_set(tau));
     SG_TRY(enqueue_restrict());
@@ -710,6 +716,7 @@ class Engine final : public EngineBase {
   }
 
   int get_grid_charge(double* rho, size_t cap) override {
+    SG_TRY(need_grids("sg_pic_get_grid_charge"));
     if (cap < S_) return size_error("sg_pic_get_grid_charge");
     SG_TRY(copy_to_host_double(rho_arena_, rho, S_));
     return add_mean(rho, S_);
@@ -720,6 +727,7 @@ class Engine final : public EngineBase {
       set_error("sg_pic_get_grid_field: the filter mode solves no component fields");
       return SG_ERR_STATE;
     }
+    SG_TRY(need_grids("sg_pic_get_grid_field"));
     if (cap < (size_t)D * S_) return size_error("sg_pic_get_grid_field");
     constexpr size_t st = ec_stride<D>();
     std::vector<double> all(st * S_);
@@ -756,6 +764,7 @@ class Engine final : public EngineBase {
       SG_TRY(copy_to_host_double(rho_f_, rho, ND_));
       return add_mean(rho, ND_);
     }
+    SG_TRY(need_grids("sg_pic_get_density"));
     real* tmp = nullptr;
     SG_TRY(alloc((void**)&tmp, ND_ * sizeof(real)));
     CombineFinal off;
@@ -852,7 +861,7 @@ class Engine final : public EngineBase {
     cur_ = 0;
     SG_TRY(upload_particles(&in));
     SG_TRY(particle_stats());
-    if (hd.tau != tau_) SG_TRY(build_grid_set(hd.tau));
+    if (hd.tau != tau_ || !grids_ok_) SG_TRY(build_grid_set(hd.tau));
     adaptive_ = hd.adaptive != 0;
     SG_TRY(enqueue_sort());
     SG_TRY(enqueue_fields());
@@ -891,6 +900,7 @@ class Engine final : public EngineBase {
       set_error("sg_pic_set_solve_variant: variant must be -1, 0 or 1");
       return SG_ERR_INVALID;
     }
+    SG_TRY(need_grids("sg_pic_set_solve_variant"));
     if (variant == 1 && !small_solve_fits()) {
       set_error("sg_pic_set_solve_variant: a component grid is too large for the one-block solve");
       return SG_ERR_UNSUPPORTED;
@@ -933,6 +943,7 @@ class Engine final : public EngineBase {
   long long steps_done() const override { return step_; }
   bool next_step_sorts() const { return ((step_ + 1) % sort_every_) == 0; }
   int step_plain() override {
+    SG_TRY(need_grids("step_plain"));
     const bool do_sort = next_step_sorts();
     const unsigned long long l0 = launches_so_far();
     per_grid_ = true;
@@ -1109,7 +1120,36 @@ class Engine final : public EngineBase {
   }
 
   // ------------------------------------------------------------ grid set
+  // The arrays of one tau make room for those of the next, so a failed
+  // allocation leaves the run without any: what launches on them is refused
+  // (need_grids) until set_tau or load has built a set.
   int build_grid_set(int tau) {
+    const int st = make_grid_set(tau);
+    grids_ok_ = st == SG_OK;
+    if (!grids_ok_) {  // keep no address of what is not there
+      for (void* p : grid_bufs_) free_one(p);
+      grid_bufs_.clear();
+      grids_.clear();
+      gdesc_.clear();
+      ngrids_ = 0;
+      S_ = 0;
+      comb_ = CombineTables();
+      rpasses_.clear();
+      fpasses_.clear();
+      grids_dev_ = nullptr;
+      restrict_planes_ = nullptr;
+      rho_arena_ = E_arena_ = nullptr;
+      A_ = B_ = nullptr;
+    }
+    return st;
+  }
+  int need_grids(const char* who) const {
+    if (grids_ok_) return SG_OK;
+    set_error(std::string(who) + ": the run has no grid set since an allocation failed (sg_pic_set_tau or "
+                                 "sg_pic_load builds one)");
+    return SG_ERR_STATE;
+  }
+  int make_grid_set(int tau) {
     invalidate_graphs();
     solve_mode_ = -1;
     tau_ = tau;
@@ -1982,7 +2022,7 @@ class Engine final : public EngineBase {
   // bookkeeping).  Runs of the combination mode with a fixed tau whose grids
   // all fit one block take part.
   bool solve_batchable() const override {
-    return !adaptive_ && !filter_ && !profiling_ && phase_ == kReady && small_solve_fits();
+    return !adaptive_ && !filter_ && !profiling_ && phase_ == kReady && grids_ok_ && small_solve_fits();
   }
   int real_bytes() const override { return (int)sizeof(real); }
   int enqueue_step_pre(bool do_sort) {
@@ -2078,8 +2118,10 @@ class Engine final : public EngineBase {
     int st = select_tau(&t, nullptr, nullptr, 0);
     if (st == SG_OK && t != tau_) {
       SG_CUDA(cudaStreamSynchronize(stream_));
-      SG_TRY(build_grid_set(t));
-    } else if (st != SG_OK && st != SG_ERR_RANGE) {
+      st = build_grid_set(t);
+    }
+    if (st != SG_OK && st != SG_ERR_RANGE) {
+      phase_ = kHalfStep;  // pushed and deposited: sg_pic_step_fields finishes the step
       return st;
     }
     SG_TRY(enqueue_restrict_solve_combine(ke_partials_));
@@ -2147,6 +2189,7 @@ class Engine final : public EngineBase {
   std::vector<GridSpec> grids_;
   std::vector<GridDesc> gdesc_;
   int ngrids_ = 0;
+  bool grids_ok_ = false;  // the grid set's arrays and tables are there
   CombineTables comb_;
   size_t comb_scratch_bytes_ = 0;
   GridArena garena_;

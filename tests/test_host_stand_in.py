@@ -1,0 +1,97 @@
+"""The library's host code against a stand-in for the CUDA runtime
+(fake_cudart.cpp): failing allocations, device memory, launches.  No GPU and
+no kernel: each script runs in a child process with the stand-in preloaded.
+"""
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes as C
+import numpy as np
+from paper_2008_09441_gb300 import SGError, _lib as L
+from paper_2008_09441_gb300.sgpic import Run, Server, sg_estimate_footprint
+fake = C.CDLL(None)
+for f in ("fake_peak", "fake_in_use"):
+    getattr(fake, f).restype = C.c_size_t
+fake.fake_launches.restype = C.c_longlong
+fake.fake_fail_malloc.argtypes = [C.c_longlong]
+launches = lambda part="": fake.fake_launches(part.encode())
+rng = np.random.default_rng(1)
+
+def run(d=2, n=6, np_=1000, **kw):
+    u, v = rng.random((np_, d)), rng.normal(size=(np_, d))
+    return Run((1.0,) * d, n, u, v, np.full(np_, -1.0 / np_), 0.1, **kw)
+
+def status(call, *args):
+    try:
+        call(*args)
+    except SGError as e:
+        return e.status
+    return L.SG_OK
+"""
+
+
+@pytest.fixture(scope="module")
+def stand_in(tmp_path_factory):
+    from paper_2008_09441_gb300 import build
+    so = tmp_path_factory.mktemp("stand_in") / "fake_cudart.so"
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+    subprocess.run(["g++", "-O1", "-fPIC", "-shared", "-std=c++17", "-I", include, "-o", str(so),
+                    os.path.join(HERE, "fake_cudart.cpp")], check=True)
+
+    def script(body):
+        r = subprocess.run([sys.executable, "-c", PRELUDE + body], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                           env={**os.environ, "LD_PRELOAD": str(so)})
+        assert r.returncode == 0, r.stdout + r.stderr
+    return script
+
+
+@pytest.mark.parametrize("d,n,t0,t1", [(2, 6, 1, 3), (3, 4, 1, 2)])
+def test_failed_grid_set_leaves_no_launchable_run(stand_in, d, n, t0, t1):
+    """No memory for a new tau's arrays: nothing that reads them may launch
+    until a grid set is there again."""
+    stand_in(f"""
+r = run({d}, {n}, tau={t0})
+r.step(3)
+blob = r.save()
+fake.fake_fail_malloc(0)
+assert status(r.set_tau, {t1}) == L.SG_ERR_OOM
+before = launches()
+for call in (lambda: r.step(1), r.step_deposit, r.diagnostics, r.post_diagnostics, r.grid_charges, r.grid_fields,
+             r.density, lambda: r.set_solve_variant("passes")):
+    assert status(call) == L.SG_ERR_STATE
+assert launches() == before
+assert r.particles()[0].shape == (1000, {d})
+fake.fake_fail_malloc(0)
+assert status(r.set_tau, {t1}) == L.SG_ERR_OOM  # the tau that failed is not taken for the current one
+r.set_tau({t1})
+assert r.grids() and len(r.grids()) == len(run({d}, {n}, tau={t1}).grids())
+r.step(2)
+r.diagnostics()
+fake.fake_fail_malloc(0)
+assert status(r.set_tau, {t0}) == L.SG_ERR_OOM
+r.load(blob)  # a checkpoint restores the run, whatever its tau
+r.step(1)
+assert r.diagnostics()["tau"] == {t0}
+""")
+
+
+def test_adaptive_step_without_memory_for_its_tau_can_be_finished(stand_in):
+    stand_in("""
+r = run(2, 6, tau=L.SG_TAU_ADAPTIVE)
+r.set_tau(3)
+fake.fake_fail_malloc(0)
+assert status(r.step, 1) == L.SG_ERR_OOM  # pushed and deposited, then no room for the selected tau
+assert status(r.step, 1) == L.SG_ERR_STATE and status(r.step_fields) == L.SG_ERR_STATE
+r.set_tau(2)
+r.step_fields()
+assert r.diagnostics()["step"] == 1
+r.step(2)
+assert r.diagnostics()["step"] == 3
+""")
