@@ -1516,19 +1516,24 @@ class Engine final : public EngineBase {
   }
 
   int ensure_estimator_buffers() {
-    if (est_z_) return SG_OK;
-    const size_t before = bytes_;
+    if (est_ready_) return SG_OK;
     // half spectra: the density's, and as many derivatives' as 256 MB hold
     // (all of them up to 3D n = 7), at least two
     const size_t hs = half_spectrum(D, n_) * sizeof(cplx<double>);
     est_wcount_ = (int)std::max<size_t>(2, std::min<size_t>(D == 2 ? 3 : 7, ((size_t)256 << 20) / hs));
-    SG_TRY(alloc((void**)&est_z_, hs));
-    SG_TRY(alloc((void**)&est_w_, est_wcount_ * hs));
-    SG_TRY(alloc((void**)&est_scalar_, 16 * sizeof(double)));
     const std::vector<cplx<double>>& tw = twiddles<double>(n_);
-    SG_TRY(alloc((void**)&tw64_, tw.size() * sizeof(cplx<double>)));
+    if (!est_z_) {  // all or nothing
+      const size_t before = bytes_;
+      Plan plan;
+      plan.want(&est_z_, half_spectrum(D, n_));
+      plan.want(&est_w_, est_wcount_ * half_spectrum(D, n_));
+      plan.want(&est_scalar_, 16);
+      plan.want(&tw64_, tw.size());
+      SG_TRY(alloc_plan(plan));
+      est_bytes_ = bytes_ - before;
+    }
     SG_CUDA(cudaMemcpyAsync(tw64_, tw.data(), tw.size() * sizeof(cplx<double>), cudaMemcpyHostToDevice, stream_));
-    est_bytes_ = bytes_ - before;
+    est_ready_ = true;
     return SG_OK;
   }
 
@@ -2221,6 +2226,7 @@ class Engine final : public EngineBase {
   std::vector<Pass> rpasses_;
   std::vector<FPass> fpasses_;
 
+  bool est_ready_ = false;
   int est_wcount_ = 0;
   void* est_host_ = nullptr;  // pinned: the estimator's reductions
   size_t est_host_bytes_ = 0;

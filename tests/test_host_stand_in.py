@@ -95,3 +95,22 @@ assert r.diagnostics()["step"] == 1
 r.step(2)
 assert r.diagnostics()["step"] == 3
 """)
+
+
+def test_failed_estimator_buffers_are_not_taken_for_ready(stand_in):
+    stand_in("""
+def select_after_failure(nth):
+    r = run(3, 4, tau=1)
+    base, before = fake.fake_in_use(), launches()
+    if nth >= 0:
+        fake.fake_fail_malloc(nth)
+        if status(r.select_tau) != L.SG_OK:
+            assert launches() == before and fake.fake_in_use() == base
+    fake.fake_fail_malloc(-1)
+    r.select_tau()
+    return fake.fake_in_use() - base
+whole = select_after_failure(-1)
+assert whole > 0
+for nth in range(5):
+    assert select_after_failure(nth) == whole
+""")
