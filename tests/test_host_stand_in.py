@@ -114,3 +114,17 @@ assert whole > 0
 for nth in range(5):
     assert select_after_failure(nth) == whole
 """)
+
+
+def test_failed_admission_launches_no_record(stand_in):
+    """The server ends a request whose init failed: nothing reads the arrays
+    that the init did not get."""
+    stand_in("""
+n = 500
+for nth in range(2):  # the run's fixed arrays, then its grid set
+    s = Server(1 << 30, 2)
+    t = s.submit((1.0, 1.0), 5, rng.random((n, 2)), np.zeros((n, 2)), np.full(n, -1.0 / n), 0.1, 2)
+    fake.fake_fail_malloc(nth)
+    assert status(s.tick) == L.SG_ERR_OOM
+    assert s.poll(t)[0] == L.SG_REQ_FAILED and launches("k_diag_record") == 0
+""")
