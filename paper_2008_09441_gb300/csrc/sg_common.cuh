@@ -57,9 +57,11 @@ unsigned long long launches_so_far();
 // call pdl_wait() before touching anything the predecessor writes (the wait
 // returns once the predecessor has completed and its writes are visible).
 // pdl_trigger() lets the successor start launching early.
-// The same for loads through the given pointers: each is re-defined after the
-// wait.  A load the compiler takes for invariant (const __restrict__, __ldg)
-// may otherwise move up past it, whatever the wait's memory clobber says.
+//
+// pdl_wait(p, ...) re-defines the given pointers after the wait.  A load that
+// the compiler takes for invariant (const __restrict__, __ldg) may otherwise
+// move up past it, whatever the wait's memory clobber says; ordinary loads
+// (load4) stay behind it.
 template <typename P>
 __device__ __forceinline__ void pdl_renew(P& p) {
   asm volatile("" : "+l"(p)::"memory");
@@ -251,6 +253,15 @@ __device__ __forceinline__ V4<float> ld4(const float* p) {
 __device__ __forceinline__ V4<double> ld4(const double* p) {
   double2 a = __ldg(reinterpret_cast<const double2*>(p));
   double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  return {{a.x, a.y, b.x, b.y}};
+}
+// The same as ordinary loads (see pdl_wait).
+__device__ __forceinline__ V4<float> load4(const float* p) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  return {{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ V4<double> load4(const double* p) {
+  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
   return {{a.x, a.y, b.x, b.y}};
 }
 __device__ __forceinline__ void st4(float* p, const V4<float>& v) {

@@ -520,13 +520,13 @@ __global__ void __launch_bounds__(256) k_restrict_warp(const LineJob* __restrict
   pdl_trigger();
   const int jb = find_job(jobs, njobs);  // job tables are written once, at set-up
   const LineJob* J = jobs + jb;
-  pdl_wait();
+  const real* src = reinterpret_cast<const real*>(J->src);
+  pdl_wait(src);  // the density, or the previous pass's output
   const int lpb = blockDim.x >> 5;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int top = J->top, len = 1 << top;
   const int inner = J->inner;
   const int b = blockIdx.x - J->block_begin;
-  const real* src = reinterpret_cast<const real*>(J->src);
   real v[VPL];
   size_t o;
   int i;

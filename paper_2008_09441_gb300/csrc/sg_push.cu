@@ -199,7 +199,10 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 0) k_push(PArrays
   __shared__ double red[32];
   const int N = 1 << n;
   const size_t ND = (size_t)N * (D == 2 ? N : (size_t)N * N);
-  pdl_wait();  // the combined field (no-op when launched without the attribute)
+  // The combined field (no wait when launched without the attribute).  The
+  // particles, which an earlier push or sort wrote, are read with ordinary
+  // loads: renewing their pointers would take them out of the parameter bank.
+  pdl_wait(Ec);
   KeAcc<real> ke;
   bool bad = false;
   unsigned long long cks = 0;
@@ -249,10 +252,10 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 0) k_push(PArrays
       V4<real> U[D], Vv[D];
 #pragma unroll
       for (int m = 0; m < D; ++m) {
-        U[m] = ld4(p.u[m] + i0);
-        Vv[m] = ld4(p.v[m] + i0);
+        U[m] = load4(p.u[m] + i0);
+        Vv[m] = load4(p.v[m] + i0);
       }
-      const V4<real> W = ld4(p.w + i0);
+      const V4<real> W = load4(p.w + i0);
       uint32_t ck[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
