@@ -60,8 +60,8 @@ unsigned long long launches_so_far();
 //
 // pdl_wait(p, ...) re-defines the given pointers after the wait.  A load that
 // the compiler takes for invariant (const __restrict__, __ldg) may otherwise
-// move up past it, whatever the wait's memory clobber says; ordinary loads
-// (load4) stay behind it.
+// move up past it, whatever the wait's memory clobber says; ordinary loads and
+// volatile ones (load4) stay behind it.
 template <typename P>
 __device__ __forceinline__ void pdl_renew(P& p) {
   asm volatile("" : "+l"(p)::"memory");
@@ -255,14 +255,20 @@ __device__ __forceinline__ V4<double> ld4(const double* p) {
   double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
   return {{a.x, a.y, b.x, b.y}};
 }
-// The same as ordinary loads (see pdl_wait).
+// The same loads as volatile instructions, which keep their place behind the
+// wait (see pdl_wait).
 __device__ __forceinline__ V4<float> load4(const float* p) {
-  const float4 t = *reinterpret_cast<const float4*>(p);
-  return {{t.x, t.y, t.z, t.w}};
+  V4<float> r;
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(r.x[0]), "=f"(r.x[1]), "=f"(r.x[2]), "=f"(r.x[3])
+               : "l"(p));
+  return r;
 }
 __device__ __forceinline__ V4<double> load4(const double* p) {
-  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
-  return {{a.x, a.y, b.x, b.y}};
+  V4<double> r;
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(r.x[0]), "=d"(r.x[1]) : "l"(p));
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(r.x[2]), "=d"(r.x[3]) : "l"(p + 2));
+  return r;
 }
 __device__ __forceinline__ void st4(float* p, const V4<float>& v) {
   *reinterpret_cast<float4*>(p) = make_float4(v.x[0], v.x[1], v.x[2], v.x[3]);

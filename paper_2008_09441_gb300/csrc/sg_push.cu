@@ -201,7 +201,9 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 0) k_push(PArrays
   const size_t ND = (size_t)N * (D == 2 ? N : (size_t)N * N);
   // The combined field (no wait when launched without the attribute).  The
   // particles, which an earlier push or sort wrote, are read with ordinary
-  // loads: renewing their pointers would take them out of the parameter bank.
+  // (3D) and volatile loads: renewing their pointers would take them out of the
+  // parameter bank.  Ordinary vector loads in 2D: annulus, 8,388,608 particles,
+  // 61.1 us instead of 58.4.
   pdl_wait(Ec);
   KeAcc<real> ke;
   bool bad = false;
