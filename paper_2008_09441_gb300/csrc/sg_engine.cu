@@ -180,7 +180,13 @@ class Engine final : public EngineBase {
     // ---- the run's fixed arrays, one allocation for all of them (see Plan)
     Plan plan;
     const size_t pb = std::max<size_t>(np_, 1);
-    for (int set = 0; set < 2; ++set) {  // particles: two sets for the sort's out-of-place permutation
+    // particles: two sets for the sort's out-of-place permutation, the keys
+    // between them (read_back_space)
+    for (int set = 0; set < 2; ++set) {
+      if (set == 1) {
+        plan.want(&keys_, pb);
+        plan.want(&keys_alt_, pb);
+      }
       for (int m = 0; m < D; ++m) {
         plan.want(&P_[set].u[m], pb);
         plan.want(&P_[set].v[m], pb);
@@ -192,8 +198,6 @@ class Engine final : public EngineBase {
     plan.want(&status_, 1);
     plan.want(&checksum_, 1);
     plan.want(&comb_counter_, 1);
-    plan.want(&keys_, pb);
-    plan.want(&keys_alt_, pb);
     tile_shift_ = std::max(0, n_ - 12 / D);
     ntiles_ = (size_t)1 << (D * (n_ - tile_shift_));
     plan.want(&tile_count_, ntiles_);
@@ -657,18 +661,14 @@ class Engine final : public EngineBase {
       }
       dst.w = P_[o].w;
     }
-    // Destinations beyond half of the 129 MB L2 go through full-sector records
-    // (with sector-sized scratch from the pool), smaller ones are scattered
-    // directly.  Direct / records, us: 40 MB 81 / 86, 59 MB 106 / 93, 84 MB
-    // 155 / 151, 168 MB 1091 / 282, 470 MB 4180 / 600.  Without memory for
-    // the scratch the direct scatter serves every size.
+    // Device destinations beyond half of the 129 MB L2 go through full-sector
+    // records, smaller ones are scattered directly.  Direct / records, us:
+    // 40 MB 81 / 86, 59 MB 106 / 93, 84 MB 155 / 151, 168 MB 1091 / 282, 470 MB
+    // 4180 / 600.  Host destinations are scattered too: their staging takes the
+    // records' place, and the copy to the host is ten times the difference.
     void* rec = nullptr;
-    if ((2 * D + 1) * np_ * sizeof(real) >= ((size_t)64 << 20) &&
-        alloc(&rec, unpermute_scratch_bytes<real, D>(np_)) != SG_OK)
-      rec = nullptr;
-    const int st = launch_unpermute<real, D>(P_[cur_], dst, np_, rec, stream_);
-    free_one(rec);
-    SG_TRY(st);
+    if (out->on_device && (2 * D + 1) * np_ * sizeof(real) >= ((size_t)64 << 20)) rec = read_back_space(dst);
+    SG_TRY(launch_unpermute<real, D>(P_[cur_], dst, np_, rec, stream_));
     if (!out->on_device) {
       for (int m = 0; m < D; ++m) {
         if (out->u[m]) SG_CUDA(cudaMemcpyAsync(out->u[m], dst.u[m], np_ * sizeof(real), cudaMemcpyDeviceToHost, stream_));
@@ -678,6 +678,23 @@ class Engine final : public EngineBase {
     }
     SG_CUDA(cudaStreamSynchronize(stream_));
     return SG_OK;
+  }
+
+  // Room for the read-back's records between steps: the idle particle set and
+  // the keys next to it, so that a read-back adds nothing to the memory that
+  // the run was admitted by.  nullptr if a destination lies there (arrays that
+  // device_particles once returned).
+  void* read_back_space(const PArrays<real, D>& dst) const {
+    char* p = reinterpret_cast<char*>(cur_ == 0 ? static_cast<void*>(keys_) : static_cast<void*>(P_[0].u[0]));
+    char* end = cur_ == 0 ? reinterpret_cast<char*>(P_[1].pid + np_) : reinterpret_cast<char*>(P_[1].u[0]);
+    if ((size_t)(end - p) < unpermute_scratch_bytes<real, D>(np_)) return nullptr;
+    auto inside = [&](const real* a) {
+      const char* b = reinterpret_cast<const char*>(a);
+      return b < end && b + np_ * sizeof(real) > p;
+    };
+    for (int m = 0; m < D; ++m)
+      if (inside(dst.u[m]) || inside(dst.v[m])) return nullptr;
+    return inside(dst.w) ? nullptr : p;
   }
 
   int get_keys(uint32_t* keys, uint32_t* counts, size_t cap_keys, size_t cap_counts) override {

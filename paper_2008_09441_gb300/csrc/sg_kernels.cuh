@@ -28,8 +28,8 @@ int cell_sort(int precision, int dim, int level, size_t n, const void* const* u,
               uint32_t* counts, uint32_t* scratch, cudaStream_t s);
 
 // dst[pid[i]] = src[i] for every particle array (back to the original order;
-// dst's pid is not written).  scratch: unpermute_scratch_bytes(np) bytes
-// aligned to 32, or nullptr for the direct scatter.
+// dst's pid is not used).  scratch: unpermute_scratch_bytes(np) bytes aligned
+// to 32, or nullptr for the direct scatter.
 template <typename real, int D>
 int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, size_t np, void* scratch,
                      cudaStream_t s);

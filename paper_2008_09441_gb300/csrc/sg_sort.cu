@@ -467,7 +467,6 @@ __global__ void __launch_bounds__(256) k_unpermute(PArrays<real, D> src, PArrays
     dst.v[m][j] = src.v[m][i];
   }
   dst.w[j] = src.w[i];
-  if (dst.pid) dst.pid[j] = j;
 }
 
 // The same in two passes through an array of records, one per particle in
@@ -478,10 +477,13 @@ __global__ void __launch_bounds__(256) k_unpermute(PArrays<real, D> src, PArrays
 // longer fits L2.  The second pass reads the records in order and writes
 // the arrays.  Bound: HBM (the payload read, the records written in random
 // 32-byte sectors and read back, the payload written).  16,777,216 particles
-// in 3D: 600 us in all against 4180 us direct.
+// in 3D: 600 us in all against 4180 us direct.  In 2D FP64 the record is one
+// sector of u and v, and the charge is scattered directly: two sectors would
+// not fit the place that the records have (Engine::read_back_space).
 template <typename real, int D>
 struct __align__(32) ParticleRecord {
-  static constexpr int words = ((2 * D + 1) * (int)sizeof(real) + 31) / 32 * (32 / (int)sizeof(real));
+  static constexpr bool charge = !(D == 2 && sizeof(real) == 8);
+  static constexpr int words = ((2 * D + charge) * (int)sizeof(real) + 31) / 32 * (32 / (int)sizeof(real));
   real x[words];
 };
 
@@ -504,7 +506,8 @@ __device__ __forceinline__ void ld_sector(const double* p, double* x) {
 }
 
 template <typename real, int D>
-__global__ void __launch_bounds__(256) k_unpermute_pack(PArrays<real, D> src, ParticleRecord<real, D>* rec, size_t np) {
+__global__ void __launch_bounds__(256) k_unpermute_pack(PArrays<real, D> src, ParticleRecord<real, D>* rec,
+                                                        PArrays<real, D> dst, size_t np) {
   constexpr int PER = 32 / (int)sizeof(real), W = ParticleRecord<real, D>::words;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= np) return;
@@ -516,8 +519,10 @@ __global__ void __launch_bounds__(256) k_unpermute_pack(PArrays<real, D> src, Pa
     x[m] = src.u[m][i];
     x[D + m] = src.v[m][i];
   }
-  x[2 * D] = src.w[i];
-  real* d = rec[src.pid[i]].x;
+  const uint32_t j = src.pid[i];
+  if constexpr (ParticleRecord<real, D>::charge) x[2 * D] = src.w[i];
+  else dst.w[j] = src.w[i];
+  real* d = rec[j].x;
 #pragma unroll
   for (int k = 0; k < W; k += PER) st_sector(d + k, x + k);
 }
@@ -536,7 +541,7 @@ __global__ void __launch_bounds__(256) k_unpermute_unpack(const ParticleRecord<r
     dst.u[m][i] = x[m];
     dst.v[m][i] = x[D + m];
   }
-  dst.w[i] = x[2 * D];
+  if constexpr (ParticleRecord<real, D>::charge) dst.w[i] = x[2 * D];
 }
 
 template <typename real, int D>
@@ -555,7 +560,7 @@ int launch_unpermute(const PArrays<real, D>& src, const PArrays<real, D>& dst, s
     return SG_OK;
   }
   auto* rec = static_cast<ParticleRecord<real, D>*>(scratch);
-  k_unpermute_pack<real, D><<<blocks, 256, 0, s>>>(src, rec, np);
+  k_unpermute_pack<real, D><<<blocks, 256, 0, s>>>(src, rec, dst, np);
   SG_CHECK_LAUNCH();
   k_unpermute_unpack<real, D><<<blocks, 256, 0, s>>>(rec, dst, np);
   SG_CHECK_LAUNCH();

@@ -128,3 +128,27 @@ for nth in range(2):  # the run's fixed arrays, then its grid set
     assert status(s.tick) == L.SG_ERR_OOM
     assert s.poll(t)[0] == L.SG_REQ_FAILED and launches("k_diag_record") == 0
 """)
+
+
+@pytest.mark.parametrize("d,prec", [(2, "fp32"), (3, "fp32"), (2, "fp64"), (3, "fp64")])
+@pytest.mark.parametrize("sorts", [0, 1])
+def test_read_back_takes_no_device_memory(stand_in, d, prec, sorts):
+    """Payloads beyond 64 MiB included: a server admits runs by the memory they
+    hold between steps, so a read-back may not add to it."""
+    np_ = (64 << 20) // ((2 * d + 1) * (4 if prec == "fp32" else 8)) + 259
+    stand_in(f"""
+d, n = {d}, {np_}
+r = run(d, 4, n, precision="{prec}", sort_every=1)
+r.step({sorts})  # the current particle set is the second or the first one
+a = [np.empty(n, r.dtype) for _ in range(2 * d + 1)]
+o = L.sg_particles_out()
+o.n, o.w = n, a[2 * d].ctypes.data
+for m in range(d):
+    o.u[m], o.v[m] = a[m].ctypes.data, a[d + m].ctypes.data
+for on_device in (1, 0):
+    o.on_device = on_device
+    fake.fake_peak(1)
+    assert L.lib().sg_pic_get_particles(r.h, C.byref(o)) == L.SG_OK
+    assert fake.fake_peak(1) == fake.fake_in_use()
+assert launches("k_unpermute_pack") == 1  # the device's own records: in the idle particle set and the keys
+""")
