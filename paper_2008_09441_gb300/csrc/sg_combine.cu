@@ -3,16 +3,17 @@
 // (eq. sparse_filter's c_i and P_i of eq. restriction, applied to the
 // fields).  P_i is a product of one prolongation per axis, so the sum is taken
 // axis by axis, the last axis first:
-//   3D: k_combine_planes prolongs along z.  The grids that share the levels
-//       (l_1, l_2) -- at most three, of coefficients +1, -2, +1 -- collapse
-//       into one "pair" array on 2^l_1 x 2^l_2 x N nodes.
-//   2D, and every z plane of a 3D run: k_combine_line interpolates each array
-//       (2D: the component grids, 3D: the plane's pairs) between the two
-//       coarse lines that bracket a regular line, and prolongs along x by
-//       Horner's scheme (prolong level l to l + 1, add the arrays of x level
-//       l + 1, ...), exact for nested node-centred grids.
-// Arrays per regular line drop from the 64 component grids with four
-// brackets each to 28 pairs with two (3D, n = 7, tau = 1).
+//   3D: k_combine_planes prolongs every grid along z, to 2^l_1 x 2^l_2 x N
+//       nodes.
+//   2D, and every z plane of a 3D run: k_combine_line interpolates each grid
+//       between the two coarse lines that bracket a regular line, and prolongs
+//       along x by Horner's scheme (prolong level l to l + 1, add the grids of
+//       x level l + 1, ...), exact for nested node-centred grids.
+// A regular line reads two brackets of every grid instead of four.  Summing the
+// grids that share (l_1, l_2) along z first (28 arrays instead of 64 at n = 7,
+// tau = 1) would round partial sums to floats between the kernels, or pass
+// them as float pairs, whose interpolation costs as much as the grids' own (3D
+// n = 7 80 us, the grids 77).
 //
 // The fields are stored node-interleaved, from the solve's output to the
 // combined field, so one load brings all components of a node and one thread
@@ -162,10 +163,6 @@ struct Sum {  // FP64 accumulation
 #pragma unroll
     for (int p = 0; p < W; ++p) v[p] += t.v[p];
   }
-  __device__ __forceinline__ void value(T* x) const {
-#pragma unroll
-    for (int p = 0; p < W; ++p) x[p] = v[p];
-  }
 };
 template <int W>
 struct __align__(16) Sum<float, W> {  // float pairs
@@ -243,10 +240,6 @@ struct __align__(16) Sum<float, W> {  // float pairs
       }
     }
   }
-  __device__ __forceinline__ void value(float* x) const {
-    float l[W];
-    split(x, l);
-  }
 };
 
 // The two level-lev nodes that bracket regular node y along one axis and
@@ -280,12 +273,10 @@ constexpr int carried() { return sizeof(T) == 4 ? node_stride<NC>() : 1; }
 
 // ---------------------------------------------------------------- 3D: prolongation along z
 //
-// out[z][off_p + e] = sum over the pair's grids of c_i times the linear
-// interpolation along z of in-plane node e.  The sum runs in the accumulator
-// and is rounded once to the type of the grids' terms, as a grid's own
-// interpolated term is in k_combine_line.  One thread per in-plane node
-// walks PL_Z planes; loads are consecutive in e.  Bound: latency (9400
-// cycles, about 5 us, at n = 7, tau = 1: 394 K nodes from 64 grids).
+// out[z][off_i + e] = c_i times the linear interpolation along z of in-plane
+// node e of grid i.  One thread per in-plane node walks PL_Z planes; loads are
+// consecutive in e.  Bound: latency (7 us at n = 7, tau = 1: 624 K nodes from 64
+// grids).
 constexpr int PL_Z = 4;
 constexpr int PL_LEVELS = 9;  // 3D levels 0..8
 template <typename T>
@@ -294,18 +285,18 @@ struct __align__(16) PlaneBracket {
   T w0, w1;
 };
 template <typename real, typename T, int NC, bool CELL>
-__global__ void __launch_bounds__(256) k_combine_planes(const PlanePair* __restrict__ pairs, int npairs,
+__global__ void __launch_bounds__(256) k_combine_planes(const PlaneGrid* __restrict__ grids, int ngrids,
                                                         const real* __restrict__ E, int S2, int n, int z0, int nz,
                                                         T* __restrict__ out) {
   constexpr int DP = node_stride<NC>(), W = sizeof(T) == 4 ? DP : NC;
-  __shared__ PlanePair sp[CB_MAX_GRIDS];
+  __shared__ PlaneGrid sp[CB_MAX_GRIDS];
   __shared__ PlaneBracket<T> sb[PL_LEVELS][PL_Z];
   pdl_trigger();
   const int zb = blockIdx.y * PL_Z;
   {
-    const int* src = reinterpret_cast<const int*>(pairs);
+    const int* src = reinterpret_cast<const int*>(grids);
     int* dst = reinterpret_cast<int*>(sp);
-    for (int i = threadIdx.x; i < npairs * (int)(sizeof(PlanePair) / 4); i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < ngrids * (int)(sizeof(PlaneGrid) / 4); i += blockDim.x) dst[i] = src[i];
     if (threadIdx.x < (n + 1) * PL_Z) {
       const int l = threadIdx.x / PL_Z, z = threadIdx.x % PL_Z;
       PlaneBracket<T> t;
@@ -318,38 +309,29 @@ __global__ void __launch_bounds__(256) k_combine_planes(const PlanePair* __restr
   pdl_wait(E);  // the solve's fields
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= S2) return;
-  int lo = 0, hi = npairs;  // the last pair with off <= e
+  int lo = 0, hi = ngrids;  // the last grid with off <= e
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (sp[mid].off <= e) lo = mid;
     else hi = mid;
   }
-  const PlanePair P = sp[lo];
-  const int le = e - P.off;
+  const PlaneGrid P = sp[lo];
+  const int le = e - P.off, g = P.goff + le;
+  const T c = (T)P.coeff;
   const int x = le & ((1 << P.lx) - 1);
   const int at = e - x + line_pos(x, P.lx, n);
 #pragma unroll
   for (int z = 0; z < PL_Z; ++z) {
     if (zb + z >= nz) break;
-    Sum<T, W> acc = Sum<T, W>::zero();
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      if (q < P.ng) {
-        const PlaneBracket<T> t = sb[P.lz[q]][z];
-        const T c = (T)P.coeff[q];
-        const int g = P.goff[q] + le;
-        acc.add_term(Term<T, W>::lerp(c * t.w0, load_node<T, W, DP>(E, g + (t.k0 << P.logs)), c * t.w1,
-                                      load_node<T, W, DP>(E, g + (t.k1 << P.logs))));
-      }
-    }
-    T xv[W];
-    acc.value(xv);
+    const PlaneBracket<T> t = sb[P.lz][z];
+    const Term<T, W> v = Term<T, W>::lerp(c * t.w0, load_node<T, W, DP>(E, g + (t.k0 << P.logs)), c * t.w1,
+                                          load_node<T, W, DP>(E, g + (t.k1 << P.logs)));
     T* d = out + ((size_t)(zb + z) * S2 + at) * DP;
     if constexpr (sizeof(T) == 4 && W == 4) {
-      *reinterpret_cast<float4*>(d) = make_float4(xv[0], xv[1], xv[2], xv[3]);
+      *reinterpret_cast<ulonglong2*>(d) = make_ulonglong2(v.v[0], v.v[1]);
     } else {
 #pragma unroll
-      for (int w = 0; w < W; ++w) d[w] = xv[w];
+      for (int w = 0; w < W; ++w) d[w] = v.v[w];
     }
   }
 }
@@ -363,11 +345,12 @@ __global__ void __launch_bounds__(256) k_combine_planes(const PlanePair* __restr
 // computes K consecutive nodes: it needs 2 nodes of the shared level, then
 // 3, 5, ..., K + 1, and prolongs that cone by itself, which spares the
 // barriers of the widest levels for a few values computed twice.  Bound:
-// 3D, the L1 data pipe (53% busy) and latency at 31% occupancy; 2D, the
-// latency of the block's phases (36% of issue slots).  With profiling events,
-// before (one warp per line, all grids) -> now, planes included: 3D n = 7
-// 151 -> 59 us, tau = 2 137 -> 69, n = 6 cell-centred 64 -> 25; 2D n = 11
-// 134 -> 51, n = 10 27 -> 20.5, n = 8 14.3 -> 12.3 us.
+// 3D, latency (four loads in flight instead of two: 88 -> 84 us) and the
+// seven pair operations of every grid's node; 2D, the latency of the block's
+// phases (36% of issue slots).  With profiling events, before (one warp per
+// line, four brackets) -> now, planes included: 3D n = 7 151 -> 77 us, tau = 2
+// 137 -> 74, n = 6 cell-centred 64 -> 28; 2D n = 11 134 -> 51, n = 10 27 -> 22,
+// n = 8 14.3 -> 12.3 us.
 
 // Transverse interpolation of one array at regular line y: the two coarse
 // lines that bracket it, each weight times the coefficient (dyadic: exact).
@@ -439,7 +422,7 @@ __device__ __forceinline__ Sum<T, W> entering(const GT* __restrict__ G, const Ro
   const int mask = (1 << l) - 1;
   const int i1 = CELL ? x >> 1 : x;
   const int end = start[l + 1];
-#pragma unroll 2
+#pragma unroll DP == 4 ? 4 : 2  // loads in flight (3D n = 7: two 88 us, four 84)
   for (int gi = start[l]; gi < end; ++gi) {
     const RowTerm<T> rt = tab[gi];
     Term<T, W> t = row_node<T, W, DP>(G, rt, i1);
@@ -552,7 +535,7 @@ __global__ void __launch_bounds__(CL_THREADS, sizeof(T) == 8 ? 2 : NC == 3 ? 3 :
     tab[e] = rt;
   }
   __syncthreads();
-  pdl_wait(G);  // the fields (3D: their pairs)
+  pdl_wait(G);  // the fields (3D: their planes)
   const int ntask = lpb * MG * ipl;
   const GT* Gz = G + (size_t)((brow - row0) >> n) * zstride;  // lpb <= N: the block's lines lie in one plane
   int level = min(CELL ? lmin + 1 : lmin, n - LK);
@@ -661,15 +644,16 @@ static int launch_lines(const CombineTables& ct, const GT* G, size_t zstride, in
   const int N = 1 << n, ipl = N / CB_RUN;
   constexpr int W = carried<T, NC>(), MG = W >= NC ? 1 : NC;
   // Threads per block and tasks to share among them.  From 2^18 tasks on
-  // (2D n = 10, 3D n = 7) a block takes 384 or more, two per thread, which
-  // spreads its tables and barriers: 3D n = 7 59 us against 71 us with 128
-  // and 128, 2D n = 10 20.5 against 21.2.  Below, small blocks reach more SMs:
-  // 3D n = 6 25 against 43 us, 2D n = 8 12.3 against 14.5.  Doubles on tiny
-  // grids go smaller still (2D n = 6: 13.5 against 14.3 us).
+  // (2D n = 10, 3D n = 7) a block takes 384 or more (3D fields 192, whose
+  // tables are three times as long), two per thread, which spreads its tables
+  // and barriers: 3D n = 7 77 us against 86 with 128 and 128, 84 with 384; 2D
+  // n = 10 20.5 against 21.2.  Below, small blocks reach more SMs: 3D n = 6 25
+  // against 43 us, 2D n = 8 12.3 against 14.5.  Doubles on tiny grids go smaller
+  // still (2D n = 6: 13.5 against 14.3 us).
   const size_t tasks = nd * MG / CB_RUN;
   const bool large = sizeof(T) == 4 && tasks >= ((size_t)1 << 18);
-  const int ft = large ? 384 : sizeof(T) == 8 && tasks < ((size_t)1 << 14) ? 64 : 128;
-  const int fthr = large ? 192 : ft;
+  const int ft = large ? (NC == 3 ? 192 : 384) : sizeof(T) == 8 && tasks < ((size_t)1 << 14) ? 64 : 128;
+  const int fthr = large ? ft / 2 : ft;
   int lpb = 1;
   while (2 * lpb <= std::min(rows, N) && lpb * MG * ipl < ft) lpb *= 2;
   const int ngl = ct.ls.start[17];
@@ -698,21 +682,21 @@ static int launch_combine_nc(const CombineTables& ct, const real* E, int n, real
   if constexpr (D == 2) {
     return launch_lines<real, real, T, NC, CELL, (NC > 1)>(ct, E, 0, n, 0, N, nd, Ehi, Elo, partials, &part0, fin, s);
   } else {
-    // as many planes at a time as the pair scratch holds (a power of two, so
+    // as many planes at a time as the scratch holds (a power of two, so
     // that every launch has whole blocks); the last launch closes the step
     constexpr int DP = node_stride<NC>();
     const size_t plane = (size_t)DP * ct.S2;
     int nz = N;
     while (nz > 1 && (size_t)nz * plane * sizeof(T) > ct.scratch_bytes) nz >>= 1;
     if ((size_t)nz * plane * sizeof(T) > ct.scratch_bytes) {
-      set_error("combination: pair scratch smaller than one plane");
+      set_error("combination: scratch smaller than one plane");
       return SG_ERR_SIZE;
     }
     T* G = static_cast<T*>(ct.scratch);
     for (int z0 = 0; z0 < N; z0 += nz) {
       SG_CUDA(launch_pdl(k_combine_planes<real, T, NC, CELL>,
                          dim3((unsigned)((ct.S2 + 255) / 256), (unsigned)((nz + PL_Z - 1) / PL_Z)), dim3(256), 0, s,
-                         ct.pairs, ct.npairs, E, ct.S2, n, z0, nz, G));
+                         ct.planes, ct.ls.start[17], E, ct.S2, n, z0, nz, G));
       SG_CHECK_LAUNCH();
       CombineFinal f = fin;
       if (z0 + nz < N) f.active = 0;

@@ -1211,9 +1211,9 @@ class Engine final : public EngineBase {
       SG_TRY(build_restrict_jobs());
       SG_TRY(build_fft_jobs());
       if (D == 3) {
-        // The combination's pair scratch takes what the run's estimated
-        // footprint leaves (all planes at tau = 1: 6.3 MB at n = 7); larger tau,
-        // whose pairs grow towards the regular grid, go in several runs of
+        // The combination's scratch takes what the run's estimated footprint
+        // leaves (all planes at tau = 1: 10 MB at n = 7); larger tau, whose
+        // planes grow towards the regular grid, go in several runs of
         // planes instead of past the estimate that serving admits by (which
         // leaves out the estimator's and the filter mode's arrays), in eight
         // runs at most.
@@ -1276,11 +1276,11 @@ class Engine final : public EngineBase {
     return SG_OK;
   }
 
-  // The combination's arrays grouped by x level: 2D, the component grids;
-  // 3D, the pairs (l_1, l_2) whose grids the z prolongation collapses.
+  // The combination's arrays grouped by x level: the component grids, in 3D
+  // their planes after the z prolongation.
   int build_combine_tables() {
     std::vector<LineGrid> lines;
-    std::vector<PlanePair> pairs;
+    std::vector<PlaneGrid> planes;
     comb_ = CombineTables();
     comb_.lmin = n_;
     int S2 = 0;
@@ -1294,26 +1294,9 @@ class Engine final : public EngineBase {
           lines.push_back({d.l[0], d.l[1], d.offset, d.coeff});
           continue;
         }
-        size_t p = (size_t)comb_.ls.start[l];
-        while (p < lines.size() && lines[p].ly != d.l[1]) ++p;
-        if (p == lines.size()) {
-          lines.push_back({d.l[0], d.l[1], S2, 1});
-          PlanePair q;
-          std::memset(&q, 0, sizeof(q));
-          q.off = S2;
-          q.logs = d.l[0] + d.l[1];
-          q.lx = l;
-          pairs.push_back(q);
-          S2 += 1 << q.logs;
-        }
-        PlanePair& q = pairs[p];
-        if (q.ng == 3) {
-          set_error("combination: more than three grids share two levels");
-          return SG_ERR_UNSUPPORTED;
-        }
-        q.goff[q.ng] = d.offset;
-        q.lz[q.ng] = d.l[D - 1];
-        q.coeff[q.ng++] = d.coeff;
+        lines.push_back({d.l[0], d.l[1], S2, 1});  // the coefficient goes into the planes
+        planes.push_back({S2, d.l[0] + d.l[1], l, d.l[D - 1], d.offset, d.coeff});
+        S2 += 1 << (d.l[0] + d.l[1]);
       }
     }
     for (int l = n_ + 1; l < 18; ++l) comb_.ls.start[l] = (int)lines.size();
@@ -1325,10 +1308,9 @@ class Engine final : public EngineBase {
     SG_TRY(gtable(&ld, lines.data(), lines.size()));
     comb_.lines = ld;
     if (D == 3) {
-      PlanePair* pd = nullptr;
-      SG_TRY(gtable(&pd, pairs.data(), pairs.size()));
-      comb_.pairs = pd;
-      comb_.npairs = (int)pairs.size();
+      PlaneGrid* pd = nullptr;
+      SG_TRY(gtable(&pd, planes.data(), planes.size()));
+      comb_.planes = pd;
       comb_.S2 = S2;
     }
     return SG_OK;

@@ -251,7 +251,7 @@ int launch_estimator(const real* rho, cplx<double>* Z, cplx<double>* W, int wcou
 
 // ---------------------------------------------------------------- combine
 // Place of node x of a level-l line in the arrays the line kernel reads (2D:
-// the component fields, 3D: the planes of pairs).  A thread of that kernel
+// the component fields, 3D: the planes).  A thread of that kernel
 // takes CB_RUN consecutive nodes of a level-n line and half as many one
 // level below; node j of every thread's run is stored next to the other
 // threads' node j, so that a warp's loads are consecutive.
@@ -259,9 +259,9 @@ constexpr int CB_RUN = 4;
 __host__ __device__ __forceinline__ int line_pos(int x, int l, int n) {
   return l == n ? ((x & 3) << (l - 2)) + (x >> 2) : l == n - 1 ? ((x & 1) << (l - 1)) + (x >> 1) : x;
 }
-// The arrays the line kernel combines: 2D, the component grids; 3D, the pairs
-// (l_1, l_2) with the z axis already prolonged.  Grouped by x level:
-// start[l] .. start[l+1] have l_1 = l; start[l] for l > n holds the count.
+// The arrays the line kernel combines: the component grids, in 3D with the z
+// axis already prolonged.  Grouped by x level: start[l] .. start[l+1] have
+// l_1 = l; start[l] for l > n holds the count.
 constexpr int CB_MAX_GRIDS = 128;
 struct LineGrid {
   int lx, ly, off, coeff;
@@ -269,19 +269,18 @@ struct LineGrid {
 struct LevelStarts {
   int start[18];
 };
-// 3D: the grids of one pair, and the pair's place in a plane of pairs.
-struct PlanePair {
-  int off, logs, ng, lx;  // offset in the plane, l_1 + l_2, number of grids, l_1
-  int goff[3], lz[3], coeff[3];
-  int pad2[3];
+// 3D: a grid and its place in a plane.
+struct PlaneGrid {
+  int off, logs, lx, lz;  // offset in the plane, l_1 + l_2, l_1, l_3
+  int goff, coeff;        // offset in the arena, coefficient
 };
 struct CombineTables {
   const LineGrid* lines = nullptr;
   LevelStarts ls{};
   int lmin = 0;  // smallest x level
   // 3D only
-  const PlanePair* pairs = nullptr;
-  int npairs = 0, S2 = 0;  // S2: values of one plane and component
+  const PlaneGrid* planes = nullptr;
+  int S2 = 0;  // values of one plane and component
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
 };
