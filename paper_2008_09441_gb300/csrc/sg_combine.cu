@@ -99,22 +99,6 @@ struct Term {
     }
     return r;
   }
-  static __device__ __forceinline__ Term mid(const Term& a, const Term& b) {  // (a + b) / 2
-    Term r;
-    const E h = splat((T)0.5);
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-      if constexpr (packed) r.v[p] = f2_mul(h, f2_add(a.v[p], b.v[p]));
-      else r.v[p] = h * (a.v[p] + b.v[p]);
-    }
-    return r;
-  }
-  static __device__ __forceinline__ Term select(bool c, const Term& a, const Term& b) {
-    Term r;
-#pragma unroll
-    for (int p = 0; p < P; ++p) r.v[p] = c ? a.v[p] : b.v[p];
-    return r;
-  }
 };
 
 // Loads node i of an array stored with DP values per node.
@@ -162,6 +146,10 @@ struct Sum {  // FP64 accumulation
   __device__ __forceinline__ void add_term(const Tm& t) {
 #pragma unroll
     for (int p = 0; p < W; ++p) v[p] += t.v[p];
+  }
+  __device__ __forceinline__ void add_mid(const Tm& a, const Tm& b) {  // (a + b) / 2
+#pragma unroll
+    for (int p = 0; p < W; ++p) v[p] += (T)0.5 * (a.v[p] + b.v[p]);
   }
 };
 template <int W>
@@ -223,6 +211,22 @@ struct __align__(16) Sum<float, W> {  // float pairs
       E err;
       hi[p] = two_sum_e(hi[p], t.v[p], err);
       lo[p] = add_e(lo[p], err);
+    }
+  }
+  // (a + b) / 2 without rounding it: the sum and its error go into the pair
+  __device__ __forceinline__ void add_mid(const Tm& a, const Tm& b) {
+    const E h = Tm::splat(0.5f);
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+      E e1, e2;
+      const E s = two_sum_e(a.v[p], b.v[p], e1);
+      if constexpr (Tm::packed) {
+        hi[p] = f2_two_sum(hi[p], f2_mul(h, s), e2);
+        lo[p] = f2_fma(h, e1, f2_add(lo[p], e2));
+      } else {
+        hi[p] = two_sum_e(hi[p], h * s, e2);
+        lo[p] = fmaf(h, e1, lo[p] + e2);
+      }
     }
   }
   // the normalised hi and lo parts, by component
@@ -425,13 +429,14 @@ __device__ __forceinline__ Sum<T, W> entering(const GT* __restrict__ G, const Ro
 #pragma unroll DP == 4 ? 4 : 2  // loads in flight (3D n = 7: two 88 us, four 84)
   for (int gi = start[l]; gi < end; ++gi) {
     const RowTerm<T> rt = tab[gi];
-    Term<T, W> t = row_node<T, W, DP>(G, rt, i1);
+    const Term<T, W> t = row_node<T, W, DP>(G, rt, i1);
     if constexpr (CELL) {  // an even node: the midpoint of two centres
       const int i0 = (x & 1) ? i1 : (i1 - 1) & mask;
       const Term<T, W> t0 = row_node<T, W, DP>(G, rt, i0);
-      t = Term<T, W>::select(x & 1, t, Term<T, W>::mid(t0, t));
+      acc.add_mid(t0, t);  // of a centre and itself: the centre
+    } else {
+      acc.add_term(t);
     }
-    acc.add_term(t);
   }
   return acc;
 }
@@ -465,7 +470,7 @@ __device__ __forceinline__ void expand(Sum<T, W>* v, const GT* __restrict__ G, c
         t[0] = row_node<T, W, DP>(G, rt, PERM && C == 2 ? ((b & 1) << (l - 1)) + (b >> 1) : b);
         row_run<T, W, DP, C, 1, PERM && C == 2>(G, rt, a, l, t + 1);
 #pragma unroll
-        for (int j = 0; j <= C; ++j) v[2 * j].add_term(Term<T, W>::mid(t[j], t[j + 1]));
+        for (int j = 0; j <= C; ++j) v[2 * j].add_mid(t[j], t[j + 1]);
 #pragma unroll
         for (int j = 0; j < C; ++j) v[2 * j + 1].add_term(t[j + 1]);
       } else {

@@ -66,7 +66,7 @@ def make_run(torch, d, n, tau, cell, mode="combine", np_=20011):
 CASES = [(2, 2, 1), (2, 5, 1), (2, 6, 2), (2, 8, 1), (2, 10, 3), (2, 11, 1), (3, 2, 1), (3, 4, 1), (3, 5, 2), (3, 6, 1)]
 
 
-@pytest.mark.parametrize("cell", [False])
+@pytest.mark.parametrize("cell", [False, True])
 @pytest.mark.parametrize("d,n,tau", CASES)
 def test_field_is_the_pair_sum(torch_cuda, d, n, tau, cell):
     r = make_run(torch_cuda, d, n, tau, cell)
@@ -79,7 +79,7 @@ def test_field_is_the_pair_sum(torch_cuda, d, n, tau, cell):
     r.close()
 
 
-@pytest.mark.parametrize("cell", [False])
+@pytest.mark.parametrize("cell", [False, True])
 @pytest.mark.parametrize("d,n,tau", [(2, 6, 1), (2, 9, 2), (3, 5, 1), (3, 6, 2)])
 def test_filtered_density_is_the_pair_sum(torch_cuda, d, n, tau, cell):
     """The same kernels on one component, whose result is stored as one float:
