@@ -229,17 +229,17 @@ struct __align__(16) Sum<float, W> {  // float pairs
       }
     }
   }
-  // the normalised hi and lo parts, by component
-  __device__ __forceinline__ void split(float* h, float* l) const {
+  // the normalised hi and lo parts, by component; the hi parts also as they are
+  __device__ __forceinline__ void split(float* h, float* l, E* s) const {
 #pragma unroll
     for (int p = 0; p < P; ++p) {
       E err;
-      const E s = two_sum_e(hi[p], lo[p], err);
+      s[p] = two_sum_e(hi[p], lo[p], err);
       if constexpr (Tm::packed) {
-        f2_unpack(s, h[2 * p], h[2 * p + 1]);
+        f2_unpack(s[p], h[2 * p], h[2 * p + 1]);
         f2_unpack(err, l[2 * p], l[2 * p + 1]);
       } else {
-        h[p] = s;
+        h[p] = s[p];
         l[p] = err;
       }
     }
@@ -484,16 +484,34 @@ __device__ __forceinline__ void expand(Sum<T, W>* v, const GT* __restrict__ G, c
   }
 }
 
-// Sum of one value per warp (the same in all its lanes), valid in thread 0.
-__device__ __forceinline__ double block_sum_warps(double w, double* sh) {
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = w;
-  __syncthreads();
-  double r = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) r += sh[k];
-  return r;
-}
+// SquareSum of the combined field's high parts, W components at a time.
+template <int W>
+struct Energy {
+  using Tm = Term<float, W>;
+  using E = typename Tm::E;
+  E hi, lo;
+  __device__ __forceinline__ Energy() : hi(Tm::splat(0.f)), lo(Tm::splat(0.f)) {}
+  __device__ __forceinline__ void add(const E* x) {
+#pragma unroll
+    for (int p = 0; p < Tm::P; ++p) {
+      E err;
+      if constexpr (Tm::packed) hi = f2_two_sum(hi, f2_mul(x[p], x[p]), err);
+      else hi = Sum<float, W>::two_sum_e(hi, __fmul_rn(x[p], x[p]), err);
+      lo = Sum<float, W>::add_e(lo, err);
+    }
+  }
+  __device__ __forceinline__ double value() const {
+    if constexpr (Tm::packed) {
+      float h0, h1, l0, l1;
+      f2_unpack(hi, h0, h1);
+      f2_unpack(lo, l0, l1);
+      const ff s = two_sum(h0, h1);
+      return (double)s.hi + (double)(s.lo + (l0 + l1));
+    } else {
+      return (double)hi + (double)lo;
+    }
+  }
+};
 
 constexpr int CL_THREADS = 256;
 
@@ -562,8 +580,8 @@ __global__ void __launch_bounds__(CL_THREADS, sizeof(T) == 8 ? 2 : NC == 3 ? 3 :
     }
     __syncthreads();
   }
-  real energy = (real)0;
-  double energy_d = 0.0;  // FP64 accumulation: the squares of the double results
+  Energy<W> energy;       // float pairs
+  double energy_d = 0.0;  // double accumulation: the squares of the double results
   for (int task = threadIdx.x; task < ntask; task += blockDim.x) {
     const int item = task & (ipl - 1);
     const int q = task >> (n - LK), r = q / MG, m0 = q % MG;
@@ -596,9 +614,9 @@ __global__ void __launch_bounds__(CL_THREADS, sizeof(T) == 8 ? 2 : NC == 3 ? 3 :
       for (int k = 0; k < K; ++k) {
         float l[W];
         if constexpr (sizeof(T) == 4) {
-          v[k].split(hi[k], l);
-#pragma unroll
-          for (int m = 0; m < WO; ++m) energy = fmaf(hi[k][m], hi[k][m], energy);
+          typename Term<float, W>::E s[Term<float, W>::P];
+          v[k].split(hi[k], l, s);
+          energy.add(s);  // a padding component is zero
         } else {
           hi[k][0] = (float)v[k].v[0];
           l[0] = (float)(v[k].v[0] - (double)hi[k][0]);
@@ -626,17 +644,11 @@ __global__ void __launch_bounds__(CL_THREADS, sizeof(T) == 8 ? 2 : NC == 3 ? 3 :
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         dst[k * DP] = v[k].v[0];
-        energy = fma(v[k].v[0], v[k].v[0], energy);
+        energy_d = fma(v[k].v[0], v[k].v[0], energy_d);
       }
     }
   }
-  double tot;
-  if constexpr (sizeof(T) == 4) {  // float pairs within the warp, double across warps
-    const ff w = warp_sum_ff(ff{energy, 0.f});
-    tot = block_sum_warps(ff_to_double(w), red);
-  } else {
-    tot = block_sum_double((double)energy + energy_d, red);
-  }
+  const double tot = block_sum_double(sizeof(T) == 4 ? energy.value() : energy_d, red);
   if (threadIdx.x == 0) partials[blockIdx.x] = tot;
   if (!fin.active) return;
   combine_finalize(partials - (n_part - (int)gridDim.x), n_part, fin, red);

@@ -346,6 +346,24 @@ int launch_diag_record(const GridDesc* grids, int ngrids, const real* rho, const
                        const unsigned long long* cks, const unsigned* st, void* out, size_t o_cks, size_t o_ch,
                        cudaStream_t s);
 
+// Sum of squares of one thread's field values: floats, every square rounded
+// once, in a float pair; doubles plainly.
+template <typename real>
+struct SquareSum {
+  ff v{0.f, 0.f};
+  __device__ __forceinline__ void add(float x) {
+    const ff s = two_sum(v.hi, __fmul_rn(x, x));
+    v = {s.hi, __fadd_rn(v.lo, s.lo)};
+  }
+  __device__ __forceinline__ double value() const { return (double)v.hi + (double)v.lo; }
+};
+template <>
+struct SquareSum<double> {
+  double v = 0.0;
+  __device__ __forceinline__ void add(double x) { v = fma(x, x, v); }
+  __device__ __forceinline__ double value() const { return v; }
+};
+
 // The last block of a field kernel to finish reduces the energy partials (and the push's kinetic-energy partials) in FP64, in a
 // fixed order, so the step needs no separate bookkeeping launch.
 __device__ __forceinline__ void combine_finalize(const double* partials, int n_part, const CombineFinal& fin,

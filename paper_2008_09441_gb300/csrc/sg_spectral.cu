@@ -398,11 +398,11 @@ __global__ void __launch_bounds__(512) k_field_rows(const cplx<real>* __restrict
   }
   __syncthreads();
   fft_smem<real>(buf, C, logn, true, tws);
-  real energy = (real)0;
+  SquareSum<real> energy;
   for (int e = threadIdx.x; e < (C << logn); e += blockDim.x) {
     const cplx<real> v = buf[fpad(e)];
-    energy = fma(v.x, v.x, energy);
-    energy = fma(v.y, v.y, energy);
+    energy.add(v.x);
+    energy.add(v.y);
     if constexpr (TWO) {
       *reinterpret_cast<cplx<real>*>(Ehi + ((j0 << logn) + e) * stride) = v;
     } else {
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(512) k_field_rows(const cplx<real>* __restrict
       Ehi[(node + N) * stride + m] = v.y;
     }
   }
-  const double tot = block_sum_double((double)energy, red);
+  const double tot = block_sum_double(energy.value(), red);
   if (threadIdx.x == 0) partials[part0 + blockIdx.x] = tot;
   if (fin.active) combine_finalize(partials, part0 + (int)gridDim.x, fin, red);
 }

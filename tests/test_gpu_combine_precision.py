@@ -4,7 +4,9 @@ Everything after it -- the sum over the grids, cell midpoints, the prolongation
 along x -- runs in float pairs, so the combined field equals the same
 expression in 64 bits up to 2^-42 of the terms' magnitudes (a pair carries 48
 bits, and fewer than 2^5 rounded pair operations follow one another on the way
-to a node).  The component fields are read back from the run itself."""
+to a node).  The field energy adds the squares of the high parts, each rounded
+once, in float pairs and doubles.  The component fields are read back from the
+run itself."""
 import numpy as np
 import pytest
 
@@ -63,6 +65,12 @@ def make_run(torch, d, n, tau, cell, mode="combine", np_=20011):
     return Run((2.0,) * d, n, u, v, -rng.random(np_), 0.01, tau=tau, centring="cell" if cell else "node", mode=mode)
 
 
+def check_energy(r, E):
+    hi = E.astype(np.float32)
+    h = (2.0 / 2 ** r.n) ** r.d
+    assert abs(r.diagnostics()["field_energy"] / (0.5 * h * np.sum((hi * hi).astype(np.float64))) - 1) <= 2.0 ** -42
+
+
 CASES = [(2, 2, 1), (2, 5, 1), (2, 6, 2), (2, 8, 1), (2, 10, 3), (2, 11, 1), (3, 2, 1), (3, 4, 1), (3, 5, 2), (3, 6, 1)]
 
 
@@ -76,6 +84,7 @@ def test_field_is_the_pair_sum(torch_cuda, d, n, tau, cell):
     for m in range(d):
         ref, mag = ref_combination({l: (coeff[l], e[m].astype(np.float32)) for l, e in fields.items()}, n, cell)
         assert np.abs(E[m] - ref).max() <= 2.0 ** -42 * mag, (m, np.abs(E[m] - ref).max() / mag)
+    check_energy(r, E)
     r.close()
 
 
@@ -91,4 +100,12 @@ def test_filtered_density_is_the_pair_sum(torch_cuda, d, n, tau, cell):
                                cell)
     assert np.all(np.abs(rho - mean - ref) <= 2.0 ** -24 * (1 + 2.0 ** -10) * np.abs(ref) + 2.0 ** -42 * mag
                   + 2.0 ** -52 * abs(mean))
+    r.close()
+
+
+@pytest.mark.parametrize("d,n", [(2, 5), (2, 9), (2, 11), (3, 4), (3, 6)])
+def test_filter_mode_energy(torch_cuda, d, n):
+    r = make_run(torch_cuda, d, n, 1, False, mode="filter")
+    r.step(1)
+    check_energy(r, r.field())
     r.close()
