@@ -14,9 +14,8 @@
 // a non-zero mode skip their transform (its result is zero).
 //
 // Bound: the estimator by the double-precision pipe (GB300: two operations
-// per clock and SM), which half spectra, skipped tiles and six-operation
-// butterflies (sg_fft.cuh) spare; the filter's solve by latency (one or two
-// blocks per SM, five barriers per transform).  Before, with whole complex
+// per clock and SM), which half spectra and skipped tiles spare; the filter's
+// solve by latency (one or two blocks per SM, five barriers per transform).  Before, with whole complex
 // arrays and a pass per operation: estimator and step 427 -> 181 us (2D
 // n = 9, adaptive), 815 -> 237 us (3D n = 6); the filter's solve with
 // profiling events 100 -> 55 us (2D n = 10).
