@@ -20,7 +20,6 @@
 // carries them through the same operations two at a time (f32x2
 // instructions; 3D pads the third component with a zero fourth).
 #include <algorithm>
-#include <atomic>
 #include <type_traits>
 
 #include "sg_kernels.cuh"
@@ -677,12 +676,9 @@ static int launch_lines(const CombineTables& ct, const GT* G, size_t zstride, in
   const unsigned blocks = (unsigned)(rows / lpb);  // both powers of two
   const unsigned threads = (unsigned)std::min(fthr, (lpb * MG * ipl + 31) / 32 * 32);
   const size_t smem = (size_t)lpb * ngl * sizeof(RowTerm<T>) + (size_t)2 * lpb * MG * ipl * sizeof(Sum<T, W>);
-  static std::atomic<bool> attr_set{false};
-  if (smem > 40 * 1024 && !attr_set) {  // with the static part the total may pass 48 KB
-    SG_CUDA(cudaFuncSetAttribute(k_combine_line<real, GT, T, NC, CELL, PERM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 200 * 1024));
-    attr_set = true;
-  }
+  static DeviceSet allowed{0};
+  if (smem > 40 * 1024)  // with the static part the total may pass 48 KB
+    SG_TRY(allow_smem(k_combine_line<real, GT, T, NC, CELL, PERM>, allowed, 200 * 1024));
   SG_CUDA(launch_pdl(k_combine_line<real, GT, T, NC, CELL, PERM>, dim3(blocks), dim3(threads), smem, s, ct.lines, ct.ls,
                      ct.lmin, G, zstride, n, lpb, row0, nd, Ehi, Elo, partials + *part0, *part0 + (int)blocks, fin));
   *part0 += (int)blocks;

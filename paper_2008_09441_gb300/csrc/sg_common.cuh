@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <utility>
 
@@ -51,6 +52,24 @@ unsigned long long launches_so_far();
     ::sg::count_launch(); \
     SG_CUDA(cudaGetLastError()); \
   } while (0)
+
+// Sets a kernel's attribute once per device (attributes belong to the kernel
+// on the current device); allow_smem: its limit of dynamic shared memory.
+using DeviceSet = std::atomic<unsigned long long>;
+template <typename K>
+int set_on_device(K* kernel, DeviceSet& done, cudaFuncAttribute attribute, int value) {
+  int dev = 0;
+  SG_CUDA(cudaGetDevice(&dev));
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load(std::memory_order_relaxed) & bit) return SG_OK;
+  SG_CUDA(cudaFuncSetAttribute(kernel, attribute, value));
+  done.fetch_or(bit, std::memory_order_relaxed);
+  return SG_OK;
+}
+template <typename K>
+int allow_smem(K* kernel, DeviceSet& done, int bytes) {
+  return set_on_device(kernel, done, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
 
 // Programmatic dependent launch (sm_90+).  A kernel launched with
 // launch_pdl may start while its predecessor in the stream drains; it must

@@ -10,7 +10,6 @@
 #include <limits.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "sg_kernels.cuh"
 
@@ -315,15 +314,12 @@ static int launch_deposit_threads(const PArrays<real, D>& p, size_t np, int n, r
                                   size_t smem, int sms, real scale, real inv_scale, real shift, cudaStream_t s) {
   // resident blocks per SM for each window size met so far (the autotuner
   // tries several capacities; the answer depends on the window's bytes)
-  static bool attr_set = false;
+  static DeviceSet allowed{0}, carved{0};
   static size_t known_smem[8];
   static int known_per_sm[8];
   static int nknown = 0;
-  if (!attr_set) {
-    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    SG_CUDA(cudaFuncSetAttribute(k_deposit<real, D, THREADS, ITEMS>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    attr_set = true;
-  }
+  SG_TRY(allow_smem(k_deposit<real, D, THREADS, ITEMS>, allowed, 200 * 1024));
+  SG_TRY(set_on_device(k_deposit<real, D, THREADS, ITEMS>, carved, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   int per_sm = 0;
   for (int i = 0; i < nknown; ++i)
     if (known_smem[i] == smem) per_sm = known_per_sm[i];
@@ -783,12 +779,8 @@ template <typename real>
 int launch_restrict_planes(const real* rho, const PlaneTargets* tgt, int n, int lx_min, bool cell, real mean,
                            cudaStream_t s) {
   const size_t smem = restrict_planes_smem<real>(n, lx_min, cell);
-  static std::atomic<bool> attr[2] = {{false}, {false}};
-  if (!attr[cell]) {
-    SG_CUDA(cudaFuncSetAttribute(cell ? k_restrict_planes<real, true> : k_restrict_planes<real, false>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, RJ_PLANE_SMEM));
-    attr[cell] = true;
-  }
+  static DeviceSet allowed[2] = {{0}, {0}};
+  SG_TRY(allow_smem(cell ? k_restrict_planes<real, true> : k_restrict_planes<real, false>, allowed[cell], RJ_PLANE_SMEM));
   const int N = 1 << n;
   const unsigned threads = (unsigned)std::max(32, std::min(1024, N * N / 4));
   if (cell)
@@ -810,12 +802,8 @@ int launch_restrict_pass(const LineJob* jobs_dev, int njobs, int nblocks, int li
   const unsigned threads = 32u * (unsigned)lines_per_block;
 #define SG_RJ_LAUNCH(V, C)                                                                                   \
   {                                                                                                          \
-    static bool attr_set = false;                                                                            \
-    if (!attr_set) {                                                                                         \
-      SG_CUDA(cudaFuncSetAttribute(k_restrict_warp<real, V, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                   200 * 1024));                                                             \
-      attr_set = true;                                                                                       \
-    }                                                                                                        \
+    static DeviceSet allowed{0};                                                                             \
+    SG_TRY(allow_smem(k_restrict_warp<real, V, C>, allowed, 200 * 1024));                                    \
     SG_CUDA(launch_pdl(k_restrict_warp<real, V, C>, dim3(nblocks), dim3(threads), smem_bytes, s, jobs_dev,   \
                        njobs, mean));                                                                        \
   }

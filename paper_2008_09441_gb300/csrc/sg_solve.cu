@@ -155,11 +155,8 @@ template <typename real>
 int launch_fft_pass(int kind, const SolveArena<real>& a, const FftJob* jobs_dev, int njobs, int nblocks,
                     int smem_bytes, cudaStream_t s) {
   if (njobs == 0 || nblocks == 0) return SG_OK;
-  static bool attr_set = false;
-  if (!attr_set) {
-    SG_CUDA(cudaFuncSetAttribute(k_fft_pass<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set = true;
-  }
+  static DeviceSet allowed{0};
+  SG_TRY(allow_smem(k_fft_pass<real>, allowed, 200 * 1024));
   SG_CUDA(launch_pdl(k_fft_pass<real>, dim3(nblocks), dim3(FFT_BLOCK_VALUES / 2),
                      smem_bytes + (size_t)twiddle_count(a.log_nmax) * sizeof(cplx<real>), s, kind, a, jobs_dev,
                      njobs));
@@ -344,11 +341,8 @@ int launch_solve_small(const SolveArena<real>& a, int ngrids, int max_size, cuda
   if (ngrids == 0) return SG_OK;
   const int threads = solve_block_threads(max_size);
   const size_t smem = solve_block_smem<real>(a.dim, max_size, a.log_nmax);
-  static bool attr_set = false;
-  if (!attr_set) {
-    SG_CUDA(cudaFuncSetAttribute(k_solve_small<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set = true;
-  }
+  static DeviceSet allowed{0};
+  SG_TRY(allow_smem(k_solve_small<real>, allowed, 200 * 1024));
   SG_CUDA(launch_pdl(k_solve_small<real>, dim3(ngrids), dim3(threads), smem, s, a, max_size, grid0));
   SG_CHECK_LAUNCH();
   return SG_OK;
@@ -366,11 +360,8 @@ int launch_solve_batch(const SolveJob<real>* jobs, int njobs, int max_size, int 
   }
   const int threads = solve_block_threads(max_size);
   const size_t smem = solve_block_smem<real>(3, max_size, max_log);  // runs of either dimension
-  static bool attr_set = false;
-  if (!attr_set) {
-    SG_CUDA(cudaFuncSetAttribute(k_solve_batch<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set = true;
-  }
+  static DeviceSet allowed{0};
+  SG_TRY(allow_smem(k_solve_batch<real>, allowed, 200 * 1024));
   k_solve_batch<real><<<njobs, threads, smem, s>>>(jobs, max_size);
   SG_CHECK_LAUNCH();
   return SG_OK;

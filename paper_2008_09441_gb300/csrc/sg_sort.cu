@@ -2,8 +2,6 @@
 // level-n cells, permutation, per-cell counts; integer work, bit-exact), the
 // step's tile counting sort, and the particles' way back to their original
 // order.
-#include <atomic>
-
 #include "sg_kernels.cuh"
 
 namespace sg {
@@ -391,12 +389,8 @@ static int cell_keys(const void* const* u, size_t n, int level, uint32_t* keys, 
 template <int BITS>
 static int radix_scatter(const uint32_t* ki, const uint32_t* vi, size_t n, int shift, const uint32_t* hist,
                          const uint32_t* total, size_t ntiles, uint32_t* ko, uint32_t* vo, cudaStream_t s) {
-  static std::atomic<bool> attr_set{false};
-  if (!attr_set) {  // with the static part the total may pass 48 KB
-    SG_CUDA(cudaFuncSetAttribute(k_radix_scatter<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 2 * RS_TILE * (int)sizeof(uint32_t)));
-    attr_set = true;
-  }
+  static DeviceSet allowed{0};  // with the static part the total may pass 48 KB
+  SG_TRY(allow_smem(k_radix_scatter<BITS>, allowed, 2 * RS_TILE * (int)sizeof(uint32_t)));
   SG_CUDA(launch_pdl(k_radix_scatter<BITS>, dim3((unsigned)ntiles), dim3(RS_THREADS), 2 * RS_TILE * sizeof(uint32_t), s,
                      ki, vi, n, shift, hist, total, ntiles, ko, vo));
   SG_CHECK_LAUNCH();
@@ -842,11 +836,8 @@ int launch_tile_scatter(const PArrays<real, D>& src, const PArrays<real, D>& dst
                         uint32_t* cursor, size_t np, cudaStream_t s) {
   if (np == 0) return SG_OK;
   constexpr size_t smem = scatter_stage_bytes<real, D>();
-  static std::atomic<bool> attr_set{false};
-  if (!attr_set) {  // with the static counters the total passes 48 KB
-    SG_CUDA(cudaFuncSetAttribute(k_tile_scatter<real, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr_set = true;
-  }
+  static DeviceSet allowed{0};  // with the static counters the total passes 48 KB
+  SG_TRY(allow_smem(k_tile_scatter<real, D>, allowed, (int)smem));
   k_tile_scatter<real, D><<<(unsigned)((np + TB_ITEMS - 1) / TB_ITEMS), TB_THREADS, smem, s>>>(src, dst, keys, shift,
                                                                                               cursor, np);
   SG_CHECK_LAUNCH();

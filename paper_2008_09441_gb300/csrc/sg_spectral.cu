@@ -20,7 +20,6 @@
 // n = 9, adaptive), 815 -> 237 us (3D n = 6); the filter's solve with
 // profiling events 100 -> 55 us (2D n = 10).
 #include <algorithm>
-#include <atomic>
 
 #include "sg_fft.cuh"
 
@@ -447,12 +446,8 @@ int line_shape(long long lines, int logn, int cmin, int nbuf, bool divide, Shape
   return SG_OK;
 }
 template <typename K>
-int allow_smem(K kernel, std::atomic<bool>& done, size_t smem) {
-  if (smem > 40 * 1024 && !done) {  // with the static part the total may pass 48 KB
-    SG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SP_SMEM));
-    done = true;
-  }
-  return SG_OK;
+int allow_lines(K* kernel, DeviceSet& done, size_t smem) {
+  return smem > 40 * 1024 ? allow_smem(kernel, done, SP_SMEM) : SG_OK;  // with the static part the total may pass 48 KB
 }
 
 template <typename Tin, typename real>
@@ -460,8 +455,8 @@ int rows_forward(const Tin* in, cplx<real>* H, int D, int n, real scale, const c
                  cudaStream_t s) {
   Shape sh;
   SG_TRY(line_shape<real>(1ll << ((D - 1) * n - 1), n, 1, 1, true, &sh));
-  static std::atomic<bool> done{false};
-  SG_TRY(allow_smem(k_rows_forward<Tin, real>, done, sh.smem));
+  static DeviceSet done{0};
+  SG_TRY(allow_lines(k_rows_forward<Tin, real>, done, sh.smem));
   SG_CUDA(launch_pdl(k_rows_forward<Tin, real>, dim3(sh.blocks), dim3(sh.threads), sh.smem, s, in, H, n, sh.C, scale, tw, sh.tw_smem, vmax));
   SG_CHECK_LAUNCH();
   return SG_OK;
@@ -484,8 +479,8 @@ int columns(cplx<real>* Z, int D, int n, int axis, bool inverse, int count, size
   Shape sh;
   const long long lines = (long long)((1 << n) / 2 + 1) << ((D - 2) * n);
   SG_TRY(line_shape<real>(lines, n, 2, 1, false, &sh));
-  static std::atomic<bool> done{false};
-  SG_TRY(allow_smem(k_columns<real>, done, sh.smem));
+  static DeviceSet done{0};
+  SG_TRY(allow_lines(k_columns<real>, done, sh.smem));
   SG_CUDA(launch_pdl(k_columns<real>, dim3(sh.blocks, count), dim3(sh.threads), sh.smem, s, Z, column_args<real>(D, n, axis, sh), inverse ? 1 : 0, zstride, tw, vmax, max2));
   SG_CHECK_LAUNCH();
   return SG_OK;
@@ -505,16 +500,16 @@ int launch_regular_solve(const real* rho_f, cplx<real>* Z, cplx<real>* W, const 
   Shape sh;
   const long long lines = (long long)((1 << n) / 2 + 1) << ((dim - 2) * n);
   SG_TRY(line_shape<real>(lines, n, 2, 2, false, &sh));
-  static std::atomic<bool> done{false};
-  SG_TRY(allow_smem(k_solve_columns<real>, done, sh.smem));
+  static DeviceSet done{0};
+  SG_TRY(allow_lines(k_solve_columns<real>, done, sh.smem));
   const unsigned groups = sh.blocks < 4 * 152 ? dim : 1;
   SG_CUDA(launch_pdl(k_solve_columns<real>, dim3(sh.blocks, groups), dim3(sh.threads), sh.smem, s, Z, W, hs, column_args<real>(dim, n, dim - 1, sh), ktab, (real)(1.0 / (double)nd), tw));
   SG_CHECK_LAUNCH();
   if (dim == 3) SG_TRY(columns<real>(W, dim, n, 1, true, 3, hs, tw, nullptr, nullptr, s));
   const long long rows = 1ll << ((dim - 1) * n);
   SG_TRY(line_shape<real>(rows, n, 1, 1, true, &sh));
-  static std::atomic<bool> done2{false}, done1{false};
-  SG_TRY(allow_smem(k_field_rows<real, true>, done2, sh.smem));
+  static DeviceSet done2{0}, done1{0};
+  SG_TRY(allow_lines(k_field_rows<real, true>, done2, sh.smem));
   CombineFinal f = fin;
   if (dim == 3) f.active = 0;
   SG_CUDA(launch_pdl(k_field_rows<real, true>, dim3(sh.blocks), dim3(sh.threads), sh.smem, s, W, W + hs, n, sh.C, tw,
@@ -523,7 +518,7 @@ int launch_regular_solve(const real* rho_f, cplx<real>* Z, cplx<real>* W, const 
   if (dim == 3) {
     const int part0 = (int)sh.blocks;
     SG_TRY(line_shape<real>(rows / 2, n, 1, 1, true, &sh));
-    SG_TRY(allow_smem(k_field_rows<real, false>, done1, sh.smem));
+    SG_TRY(allow_lines(k_field_rows<real, false>, done1, sh.smem));
     SG_CUDA(launch_pdl(k_field_rows<real, false>, dim3(sh.blocks), dim3(sh.threads), sh.smem, s, W + 2 * hs, W, n, sh.C,
                        tw, sh.tw_smem, Ehi, stride, 2, partials, part0, fin));
     SG_CHECK_LAUNCH();
@@ -560,18 +555,18 @@ int launch_estimator(const real* rho, cplx<double>* Z, cplx<double>* W, int wcou
     return SG_OK;
   }
   Shape sh;
-  static std::atomic<bool> done{false}, done2{false};
+  static DeviceSet done{0}, done2{0};
   for (int q0 = 0; q0 < nmask; q0 += wcount) {  // as many masks at a time as W holds
     e.nmask = std::min(wcount, nmask - q0);
     for (int q = 0; q < e.nmask; ++q) e.mask[q] = masks[q0 + q];
     const long long lines = (long long)((1 << n) / 2 + 1) << ((dim - 2) * n);
     SG_TRY(line_shape<double>(lines, n, 2, 1, false, &sh));
-    SG_TRY(allow_smem(k_est_columns, done, sh.smem));
+    SG_TRY(allow_lines(k_est_columns, done, sh.smem));
     SG_CUDA(launch_pdl(k_est_columns, dim3(sh.blocks, e.nmask), dim3(sh.threads), sh.smem, s, Z, W, column_args<double>(dim, n, dim - 1, sh), e, tw));
     SG_CHECK_LAUNCH();
     if (dim == 3) SG_TRY(columns<double>(W, dim, n, 1, true, e.nmask, hs, tw, nullptr, nullptr, s));
     SG_TRY(line_shape<double>(1ll << ((dim - 1) * n - 1), n, 1, 1, true, &sh));
-    SG_TRY(allow_smem(k_est_rows, done2, sh.smem));
+    SG_TRY(allow_lines(k_est_rows, done2, sh.smem));
     SG_CUDA(launch_pdl(k_est_rows, dim3(sh.blocks, e.nmask), dim3(sh.threads), sh.smem, s, W, hs, n, sh.C, tw, sh.tw_smem, out + q0));
     SG_CHECK_LAUNCH();
   }

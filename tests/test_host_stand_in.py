@@ -152,3 +152,26 @@ for on_device in (1, 0):
     assert fake.fake_peak(1) == fake.fake_in_use()
 assert launches("k_unpermute_pack") == 1  # the device's own records: in the idle particle set and the keys
 """)
+
+
+def test_every_device_raises_the_shared_memory_limits_it_needs(stand_in):
+    """The limit is a property of the kernel on one device: what a first device
+    set does not hold on the next."""
+    stand_in("""
+n, level = 4096, 8
+a = [np.zeros(n, np.float32), np.zeros(n, np.float32)]
+out = [np.zeros(n, np.uint32) for _ in range(2)] + [np.zeros(1 << (2 * level), np.uint32)]
+arr = (C.c_void_p * 3)(a[0].ctypes.data, a[1].ctypes.data, None)
+def sort(fn):
+    assert fn(L.SG_FP32, 2, level, n, arr, *(C.c_void_p(o.ctypes.data) for o in out), None) == L.SG_OK
+for device in (0, 1, 0, 2):
+    fake.fake_set_device(device)
+    sort(L.lib().sg_cell_sort)
+    sort(L.lib().sg_cell_sort_static)
+    for kw in (dict(d=2, n=10), dict(d=2, n=11, mode="filter"), dict(d=3, n=6), dict(d=3, n=7, centring="cell"),
+               dict(d=2, n=7, precision="fp64"), dict(d=3, n=5, tau=L.SG_TAU_ADAPTIVE)):
+        r = run(**kw)
+        r.step(7)
+        r.close()
+    assert fake.fake_missing_opt_in() == 0, device
+""")
