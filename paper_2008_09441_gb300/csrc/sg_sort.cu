@@ -161,7 +161,7 @@ constexpr int RS_WARP_KEYS = RS_TILE / RS_WARPS;
 static_assert(RS_WARP_KEYS == 32 * RS_ITEMS, "one key per lane per chunk");
 
 static size_t cell_sort_tiles(size_t n) { return (n + RS_TILE - 1) / RS_TILE; }
-size_t cell_sort_words(size_t n) { return 2 * n + 256 * cell_sort_tiles(n) + 256; }
+size_t cell_sort_words(size_t n) { return 3 * n + 256 * cell_sort_tiles(n) + 256; }
 
 template <typename real, int D>
 struct RawU {
@@ -399,14 +399,18 @@ static int radix_scatter(const uint32_t* ki, const uint32_t* vi, size_t n, int s
 
 int cell_sort(int precision, int dim, int level, size_t n, const void* const* u, uint32_t* keys_sorted, uint32_t* perm,
               uint32_t* counts, uint32_t* scratch, cudaStream_t s) {
-  if (counts) SG_CUDA(cudaMemsetAsync(counts, 0, ((size_t)1 << (dim * level)) * 4, s));
-  if (n == 0) return SG_OK;
+  const size_t count_bytes = ((size_t)1 << (dim * level)) * 4;
+  if (n == 0) {
+    if (counts) SG_CUDA(cudaMemsetAsync(counts, 0, count_bytes, s));
+    return SG_OK;
+  }
   const size_t ntiles = cell_sort_tiles(n);
-  uint32_t *tk = scratch, *tv = scratch + n, *hist = scratch + 2 * n, *total = hist + 256 * ntiles;
+  uint32_t *tk = scratch, *tv = scratch + n, *hist = scratch + 3 * n, *total = hist + 256 * ntiles;
   const int bits = dim * level, passes = (bits + 7) / 8;
   // passes alternate between the scratch and the result, which the last one
-  // writes; the unsorted keys start where the first pass does not write
-  uint32_t* ki = passes & 1 ? tk : keys_sorted;
+  // writes.  The unsorted keys have a place of their own and the counts are
+  // cleared after it is filled: the outputs may lie over the positions.
+  uint32_t* ki = scratch + 2 * n;
   const uint32_t* vi = nullptr;  // the first pass's values are the input indices
   int shift = 0;
   for (int p = 0; p < passes; ++p) {
@@ -418,6 +422,7 @@ int cell_sort(int precision, int dim, int level, size_t n, const void* const* u,
       else
         SG_TRY(dim == 2 ? cell_keys<double, 2>(u, n, level, ki, bins, hist, ntiles, s)
                         : cell_keys<double, 3>(u, n, level, ki, bins, hist, ntiles, s));
+      if (counts) SG_CUDA(cudaMemsetAsync(counts, 0, count_bytes, s));
     } else {
       SG_CUDA(launch_pdl(k_radix_hist, dim3((unsigned)ntiles), dim3(RS_THREADS), 0, s, ki, n, shift, bins, hist, ntiles));
       SG_CHECK_LAUNCH();

@@ -24,10 +24,10 @@
 
 namespace sg {
 
-// Keys and indices of the radix sort's alternate passes (2 x max), digit
-// histograms and totals.
+// Keys and indices of the radix sort's alternate passes and the unsorted keys
+// (3 x max), digit histograms and totals.
 constexpr size_t kStaticMax = SG_CELL_SORT_STATIC_MAX;
-constexpr size_t kStaticWords = 2 * kStaticMax + 256 * ((kStaticMax + RS_TILE - 1) / RS_TILE) + 256;  // cell_sort_words
+constexpr size_t kStaticWords = 3 * kStaticMax + 256 * ((kStaticMax + RS_TILE - 1) / RS_TILE) + 256;  // cell_sort_words
 static_assert(kStaticWords <= SG_CELL_SORT_STATIC_WORDS, "scratch layout exceeds the declared size");
 
 static __device__ __align__(256) uint32_t g_cell_sort_scratch[SG_CELL_SORT_STATIC_WORDS];
