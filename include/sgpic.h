@@ -203,7 +203,8 @@ int sg_pic_set_tau(sg_pic* h, int tau);
 
 /* Copy particle states to caller buffers in the ORIGINAL particle order
  * (the order given at init), whatever sorts happened since.  out->n must
- * equal the run's particle count; buffers are host or device per on_device. */
+ * equal the run's particle count; buffers are host or device per on_device.
+ * NULL host buffers are skipped; a NULL device buffer is SG_ERR_INVALID. */
 int sg_pic_get_particles(sg_pic* h, const sg_particles_out* out);
 
 /* Cell keys (Morton order of the level-n cell, x lowest bit) of the particles

@@ -645,12 +645,17 @@ class Engine final : public EngineBase {
     }
     if (np_ == 0) return SG_OK;
     PArrays<real, D> dst;
-    std::vector<void*> temps;
+    bool whole = out->w != nullptr;
     for (int m = 0; m < D; ++m) {
       dst.u[m] = (real*)out->u[m];
       dst.v[m] = (real*)out->v[m];
+      whole &= dst.u[m] && dst.v[m];
     }
     dst.w = (real*)out->w;
+    if (out->on_device && !whole) {
+      set_error("sg_pic_get_particles: NULL device array");
+      return SG_ERR_INVALID;
+    }
     dst.pid = nullptr;
     if (!out->on_device) {
       // stage in the other particle set (free between steps)

@@ -175,3 +175,21 @@ for device in (0, 1, 0, 2):
         r.close()
     assert fake.fake_missing_opt_in() == 0, device
 """)
+
+
+def test_device_read_back_needs_every_array(stand_in):
+    """Host destinations may be left out; a kernel cannot skip a missing device array."""
+    stand_in("""
+r = run(3, 4)
+a = [np.empty(1000, r.dtype) for _ in range(7)]
+for missing in range(7):
+    o = L.sg_particles_out()
+    o.n = 1000
+    p = [None if k == missing else x.ctypes.data for k, x in enumerate(a)]
+    o.u[0], o.u[1], o.u[2], o.v[0], o.v[1], o.v[2], o.w = p
+    o.on_device = 1
+    before = launches("k_unpermute")
+    assert L.lib().sg_pic_get_particles(r.h, C.byref(o)) == L.SG_ERR_INVALID and launches("k_unpermute") == before
+    o.on_device = 0
+    assert L.lib().sg_pic_get_particles(r.h, C.byref(o)) == L.SG_OK
+""")
