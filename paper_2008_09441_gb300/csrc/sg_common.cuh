@@ -10,9 +10,6 @@
 
 #include "../../include/sgpic.h"
 
-#define SG_MAX_DIM 3
-#define SG_THREADS 256
-
 namespace sg {
 
 // ---------------------------------------------------------------------------
@@ -21,11 +18,6 @@ namespace sg {
 // ---------------------------------------------------------------------------
 void set_error(const std::string& msg);
 const char* last_error();
-
-struct Status {
-  int code = SG_OK;
-  explicit operator bool() const { return code != SG_OK; }
-};
 
 #define SG_CUDA(call)                                                              \
   do {                                                                             \
@@ -112,7 +104,6 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 enum : unsigned {
   ST_NONFINITE = 1u,
   ST_KEY_RANGE = 2u,
-  ST_BOUNDS = 4u,
 };
 
 // ---------------------------------------------------------------------------
@@ -188,8 +179,7 @@ __device__ __forceinline__ real wrap_unit(real u) {
 // ---------------------------------------------------------------------------
 // Float-float ("double-float") arithmetic: an unevaluated sum hi + lo of two
 // floats carrying ~48 significant bits, used for the signed combination and
-// the energy sums of the FP32 path.  Error-free transformations after Knuth
-// (TwoSum) and the fused-multiply-add product (TwoProd).
+// the energy sums of the FP32 path.  Error-free sum after Knuth (TwoSum).
 // ---------------------------------------------------------------------------
 struct ff {
   float hi, lo;
@@ -201,62 +191,6 @@ __device__ __forceinline__ ff two_sum(float a, float b) {
   float err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
   return {s, err};
 }
-
-__device__ __forceinline__ ff two_prod(float a, float b) {
-  float p = __fmul_rn(a, b);
-  float e = __fmaf_rn(a, b, -p);
-  return {p, e};
-}
-
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-  ff s = two_sum(a.hi, b.hi);
-  float lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
-  return two_sum(s.hi, lo);  // renormalise
-}
-
-__device__ __forceinline__ ff ff_add_f(ff a, float b) {
-  ff s = two_sum(a.hi, b);
-  return two_sum(s.hi, __fadd_rn(s.lo, a.lo));
-}
-
-__device__ __forceinline__ ff ff_scale(ff a, float s) {  // s a power of two: exact
-  return {a.hi * s, a.lo * s};
-}
-
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
-
-__device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
-
-// Accumulator selection: float-float for the FP32 path, plain double for the
-// FP64 path.
-template <typename real>
-struct Acc;
-
-template <>
-struct Acc<float> {
-  using term = float;
-  ff v{0.f, 0.f};
-  __device__ __forceinline__ void add_prod(float a, float b) { v = ff_add(v, two_prod(a, b)); }
-  __device__ __forceinline__ void add(float a) { v = ff_add_f(v, a); }
-  __device__ __forceinline__ void add_acc(const Acc<float>& o) { v = ff_add(v, o.v); }
-  __device__ __forceinline__ void scale(float s) { v = ff_scale(v, s); }
-  __device__ __forceinline__ double to_double() const { return ff_to_double(v); }
-  __device__ __forceinline__ float hi() const { return v.hi; }
-  __device__ __forceinline__ float lo() const { return v.lo; }
-};
-
-template <>
-struct Acc<double> {
-  using term = double;
-  double v = 0.0;
-  __device__ __forceinline__ void add_prod(double a, double b) { v = fma(a, b, v); }
-  __device__ __forceinline__ void add(double a) { v += a; }
-  __device__ __forceinline__ void add_acc(const Acc<double>& o) { v += o.v; }
-  __device__ __forceinline__ void scale(double s) { v *= s; }
-  __device__ __forceinline__ double to_double() const { return v; }
-  __device__ __forceinline__ double hi() const { return v; }
-  __device__ __forceinline__ double lo() const { return 0.0; }
-};
 
 // Four consecutive values with 16-byte vector loads / stores (the arrays
 // come from cudaMalloc and every vector index is a multiple of 4).
@@ -310,15 +244,6 @@ template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ ff warp_sum_ff(ff v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ff w{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
-    v = ff_add(v, w);
-  }
   return v;
 }
 

@@ -711,7 +711,7 @@ class Engine final : public EngineBase {
       set_error("sg_pic_get_keys: count buffer too small");
       return SG_ERR_SIZE;
     }
-    SG_TRY(launch_keys<real, D>(P_[cur_], np_, n_, keys_alt_, nullptr, nullptr, status_, stream_));
+    SG_TRY(launch_keys<real, D>(P_[cur_], np_, n_, keys_alt_, status_, stream_));
     if (keys) SG_CUDA(cudaMemcpyAsync(keys, keys_alt_, np_ * 4, cudaMemcpyDeviceToHost, stream_));
     if (counts) {
       uint32_t* dcounts = nullptr;

@@ -14,11 +14,9 @@ constexpr int RS_THREADS = 512;
 constexpr int RS_ITEMS = 8;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;  // keys per tile
 
-// keys[i] = Morton key of particle i's level-n cell, idx[i] = i,
-// *checksum += sum_i (keys[i] + 1).
+// keys[i] = Morton key of particle i's level-n cell.
 template <typename real, int D>
-int launch_keys(const PArrays<real, D>& p, size_t np, int n, uint32_t* keys, uint32_t* idx,
-                unsigned long long* checksum, unsigned* status, cudaStream_t s);
+int launch_keys(const PArrays<real, D>& p, size_t np, int n, uint32_t* keys, unsigned* status, cudaStream_t s);
 
 // The stand-alone cell sort of positions u (dim device arrays in the given
 // precision): sorted keys, stable permutation, counts per cell (may be NULL).

@@ -9,36 +9,26 @@ namespace sg {
 
 // ---------------------------------------------------------------- keys
 template <typename real, int D>
-__global__ void __launch_bounds__(256) k_keys(PArrays<real, D> p, size_t np, int n, uint32_t* keys,
-                                              uint32_t* idx, unsigned long long* checksum,
-                                              unsigned* status) {
+__global__ void __launch_bounds__(256) k_keys(PArrays<real, D> p, size_t np, int n, uint32_t* keys, unsigned* status) {
   const int N = 1 << n;
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long part = 0;
-  if (i < np) {
-    int c[D];
-    bool bad = false;
+  if (i >= np) return;
+  int c[D];
+  bool bad = false;
 #pragma unroll
-    for (int m = 0; m < D; ++m) {
-      real u = p.u[m][i];
-      bad |= !(u >= (real)0 && u < (real)1);
-      c[m] = cell_of(u, n, N);
-    }
-    if (bad) atomicOr(status, ST_KEY_RANGE);
-    uint32_t k = morton_key<D>(c, n);
-    keys[i] = k;
-    if (idx) idx[i] = (uint32_t)i;
-    part = (unsigned long long)k + 1ull;
+  for (int m = 0; m < D; ++m) {
+    real u = p.u[m][i];
+    bad |= !(u >= (real)0 && u < (real)1);
+    c[m] = cell_of(u, n, N);
   }
-  part = warp_sum(part);
-  if ((threadIdx.x & 31) == 0 && checksum && part) atomicAdd(checksum, part);
+  if (bad) atomicOr(status, ST_KEY_RANGE);
+  keys[i] = morton_key<D>(c, n);
 }
 
 template <typename real, int D>
-int launch_keys(const PArrays<real, D>& p, size_t np, int n, uint32_t* keys, uint32_t* idx,
-                unsigned long long* checksum, unsigned* status, cudaStream_t s) {
+int launch_keys(const PArrays<real, D>& p, size_t np, int n, uint32_t* keys, unsigned* status, cudaStream_t s) {
   if (np == 0) return SG_OK;
-  k_keys<real, D><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(p, np, n, keys, idx, checksum, status);
+  k_keys<real, D><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(p, np, n, keys, status);
   SG_CHECK_LAUNCH();
   return SG_OK;
 }
@@ -876,8 +866,7 @@ int launch_counts(const uint32_t* keys, size_t np, uint32_t* counts, cudaStream_
 }
 
 #define SG_INST_SORT(real, D)                                                                           \
-  template int launch_keys<real, D>(const PArrays<real, D>&, size_t, int, uint32_t*, uint32_t*,        \
-                                    unsigned long long*, unsigned*, cudaStream_t);                      \
+  template int launch_keys<real, D>(const PArrays<real, D>&, size_t, int, uint32_t*, unsigned*, cudaStream_t); \
   template int launch_unpermute<real, D>(const PArrays<real, D>&, const PArrays<real, D>&, size_t, void*,        \
                                          cudaStream_t);                                                          \
   template size_t unpermute_scratch_bytes<real, D>(size_t);                                              \

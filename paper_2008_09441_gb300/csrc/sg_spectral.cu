@@ -268,8 +268,8 @@ __global__ void __launch_bounds__(256) k_est_modes(const cplx<double>* __restric
     if (q < e.nmask) block_max_store(mx[q], out + q);
 }
 
-// Components blockIdx.y, blockIdx.y + gridDim.y, ...
-// Filter mode: forward along the last axis, E^_m = -i k_m rho^ / |k|^2 (k = 0
+// Filter mode, components blockIdx.y, blockIdx.y + gridDim.y, ...: forward
+// along the last axis, E^_m = -i k_m rho^ / |k|^2 (k = 0
 // and the Nyquist plane of axis m -> 0, the component-grid rules), inverse
 // along the last axis, Z -> W[m] for every component.
 // ktab[m * N + i] = 2 pi / L_m * (i < N/2 ? i : i - N), in the run's precision.
