@@ -4,16 +4,16 @@
 // fields).  P_i is a product of one prolongation per axis, so the sum is taken
 // axis by axis, the last axis first:
 //   3D: k_combine_planes prolongs every grid along z, to 2^l_1 x 2^l_2 x N
-//       nodes.
+//       nodes; where sums run in double, the grids that share (l_1, l_2) -- at
+//       most three, of coefficients +1, -2, +1 -- collapse into one array.
 //   2D, and every z plane of a 3D run: k_combine_line interpolates each grid
 //       between the two coarse lines that bracket a regular line, and prolongs
 //       along x by Horner's scheme (prolong level l to l + 1, add the grids of
 //       x level l + 1, ...), exact for nested node-centred grids.
-// A regular line reads two brackets of every grid instead of four.  Summing the
-// grids that share (l_1, l_2) along z first (28 arrays instead of 64 at n = 7,
-// tau = 1) would round partial sums to floats between the kernels, or pass
-// them as float pairs, whose interpolation costs as much as the grids' own (3D
-// n = 7 80 us, the grids 77).
+// A regular line reads two brackets of every grid instead of four.  In FP32 the
+// collapse (28 arrays instead of 64 at n = 7, tau = 1) would round partial sums
+// to floats between the kernels, or pass them as float pairs, whose
+// interpolation costs as much as the grids' own (3D n = 7 80 us, the grids 77).
 //
 // The fields are stored node-interleaved, from the solve's output to the
 // combined field, so one load brings all components of a node and one thread
@@ -276,10 +276,10 @@ constexpr int carried() { return sizeof(T) == 4 ? node_stride<NC>() : 1; }
 
 // ---------------------------------------------------------------- 3D: prolongation along z
 //
-// out[z][off_i + e] = c_i times the linear interpolation along z of in-plane
-// node e of grid i.  One thread per in-plane node walks PL_Z planes; loads are
-// consecutive in e.  Bound: latency (7 us at n = 7, tau = 1: 624 K nodes from 64
-// grids).
+// out[z][off + e] = sum over an array's grids of c_i times the linear
+// interpolation along z of in-plane node e.  One thread per in-plane node walks
+// PL_Z planes; loads are consecutive in e.  Bound: latency (7 us at n = 7, tau =
+// 1: 624 K nodes from 64 grids).
 constexpr int PL_Z = 4;
 constexpr int PL_LEVELS = 9;  // 3D levels 0..8
 template <typename T>
@@ -288,18 +288,18 @@ struct __align__(16) PlaneBracket {
   T w0, w1;
 };
 template <typename real, typename T, int NC, bool CELL>
-__global__ void __launch_bounds__(256) k_combine_planes(const PlaneGrid* __restrict__ grids, int ngrids,
+__global__ void __launch_bounds__(256) k_combine_planes(const PlaneArray* __restrict__ arrays, int narrays,
                                                         const real* __restrict__ E, int S2, int n, int z0, int nz,
                                                         T* __restrict__ out) {
   constexpr int DP = node_stride<NC>(), W = sizeof(T) == 4 ? DP : NC;
-  __shared__ PlaneGrid sp[CB_MAX_GRIDS];
+  __shared__ PlaneArray sp[CB_MAX_GRIDS];
   __shared__ PlaneBracket<T> sb[PL_LEVELS][PL_Z];
   pdl_trigger();
   const int zb = blockIdx.y * PL_Z;
   {
-    const int* src = reinterpret_cast<const int*>(grids);
+    const int* src = reinterpret_cast<const int*>(arrays);
     int* dst = reinterpret_cast<int*>(sp);
-    for (int i = threadIdx.x; i < ngrids * (int)(sizeof(PlaneGrid) / 4); i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < narrays * (int)(sizeof(PlaneArray) / 4); i += blockDim.x) dst[i] = src[i];
     if (threadIdx.x < (n + 1) * PL_Z) {
       const int l = threadIdx.x / PL_Z, z = threadIdx.x % PL_Z;
       PlaneBracket<T> t;
@@ -312,23 +312,36 @@ __global__ void __launch_bounds__(256) k_combine_planes(const PlaneGrid* __restr
   pdl_wait(E);  // the solve's fields
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= S2) return;
-  int lo = 0, hi = ngrids;  // the last grid with off <= e
+  int lo = 0, hi = narrays;  // the last array with off <= e
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (sp[mid].off <= e) lo = mid;
     else hi = mid;
   }
-  const PlaneGrid P = sp[lo];
-  const int le = e - P.off, g = P.goff + le;
-  const T c = (T)P.coeff;
+  const PlaneArray P = sp[lo];
+  const int le = e - P.off;
   const int x = le & ((1 << P.lx) - 1);
   const int at = e - x + line_pos(x, P.lx, n);
 #pragma unroll
   for (int z = 0; z < PL_Z; ++z) {
     if (zb + z >= nz) break;
-    const PlaneBracket<T> t = sb[P.lz][z];
-    const Term<T, W> v = Term<T, W>::lerp(c * t.w0, load_node<T, W, DP>(E, g + (t.k0 << P.logs)), c * t.w1,
-                                          load_node<T, W, DP>(E, g + (t.k1 << P.logs)));
+    auto term = [&](int q) {
+      const PlaneBracket<T> t = sb[P.lz[q]][z];
+      const T c = (T)P.coeff[q];
+      const int g = P.goff[q] + le;
+      return Term<T, W>::lerp(c * t.w0, load_node<T, W, DP>(E, g + (t.k0 << P.logs)), c * t.w1,
+                              load_node<T, W, DP>(E, g + (t.k1 << P.logs)));
+    };
+    Term<T, W> v = term(0);
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+      for (int q = 1; q < 3; ++q)
+        if (q < P.ng) {
+          const Term<T, W> t = term(q);
+#pragma unroll
+          for (int w = 0; w < W; ++w) v.v[w] += t.v[w];
+        }
+    }
     T* d = out + ((size_t)(zb + z) * S2 + at) * DP;
     if constexpr (sizeof(T) == 4 && W == 4) {
       *reinterpret_cast<ulonglong2*>(d) = make_ulonglong2(v.v[0], v.v[1]);

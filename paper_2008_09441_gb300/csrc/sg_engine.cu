@@ -1282,10 +1282,11 @@ class Engine final : public EngineBase {
   }
 
   // The combination's arrays grouped by x level: the component grids, in 3D
-  // their planes after the z prolongation.
+  // those of a plane after the z prolongation.
   int build_combine_tables() {
     std::vector<LineGrid> lines;
-    std::vector<PlaneGrid> planes;
+    std::vector<PlaneArray> planes;
+    const bool collapse = sizeof(real) == 8 || cfg_.combine_fp64;  // sums in double lose nothing between the kernels
     comb_ = CombineTables();
     comb_.lmin = n_;
     int S2 = 0;
@@ -1299,9 +1300,26 @@ class Engine final : public EngineBase {
           lines.push_back({d.l[0], d.l[1], d.offset, d.coeff});
           continue;
         }
-        lines.push_back({d.l[0], d.l[1], S2, 1});  // the coefficient goes into the planes
-        planes.push_back({S2, d.l[0] + d.l[1], l, d.l[D - 1], d.offset, d.coeff});
-        S2 += 1 << (d.l[0] + d.l[1]);
+        size_t p = collapse ? (size_t)comb_.ls.start[l] : lines.size();
+        while (p < lines.size() && lines[p].ly != d.l[1]) ++p;
+        if (p == lines.size()) {
+          lines.push_back({d.l[0], d.l[1], S2, 1});  // the coefficient goes into the planes
+          PlaneArray q;
+          std::memset(&q, 0, sizeof(q));
+          q.off = S2;
+          q.logs = d.l[0] + d.l[1];
+          q.lx = l;
+          planes.push_back(q);
+          S2 += 1 << q.logs;
+        }
+        PlaneArray& q = planes[p];
+        if (q.ng == 3) {
+          set_error("combination: more than three grids share two levels");
+          return SG_ERR_UNSUPPORTED;
+        }
+        q.goff[q.ng] = d.offset;
+        q.lz[q.ng] = d.l[D - 1];
+        q.coeff[q.ng++] = d.coeff;
       }
     }
     for (int l = n_ + 1; l < 18; ++l) comb_.ls.start[l] = (int)lines.size();
@@ -1313,7 +1331,7 @@ class Engine final : public EngineBase {
     SG_TRY(gtable(&ld, lines.data(), lines.size()));
     comb_.lines = ld;
     if (D == 3) {
-      PlaneGrid* pd = nullptr;
+      PlaneArray* pd = nullptr;
       SG_TRY(gtable(&pd, planes.data(), planes.size()));
       comb_.planes = pd;
       comb_.S2 = S2;

@@ -257,8 +257,8 @@ constexpr int CB_RUN = 4;
 __host__ __device__ __forceinline__ int line_pos(int x, int l, int n) {
   return l == n ? ((x & 3) << (l - 2)) + (x >> 2) : l == n - 1 ? ((x & 1) << (l - 1)) + (x >> 1) : x;
 }
-// The arrays the line kernel combines: the component grids, in 3D with the z
-// axis already prolonged.  Grouped by x level: start[l] .. start[l+1] have
+// The arrays the line kernel combines: the component grids, in 3D those of a
+// plane (PlaneArray), the z axis already prolonged.  Grouped by x level: start[l] .. start[l+1] have
 // l_1 = l; start[l] for l > n holds the count.
 constexpr int CB_MAX_GRIDS = 128;
 struct LineGrid {
@@ -267,17 +267,19 @@ struct LineGrid {
 struct LevelStarts {
   int start[18];
 };
-// 3D: a grid and its place in a plane.
-struct PlaneGrid {
-  int off, logs, lx, lz;  // offset in the plane, l_1 + l_2, l_1, l_3
-  int goff, coeff;        // offset in the arena, coefficient
+// 3D: the grids that make one array of a plane, and its place there.  FP32:
+// one grid; double sums: the up to three that share l_1 and l_2.
+struct PlaneArray {
+  int off, logs, lx, ng;  // offset in the plane, l_1 + l_2, l_1, number of grids
+  int goff[3], lz[3], coeff[3];
+  int pad[3];
 };
 struct CombineTables {
   const LineGrid* lines = nullptr;
   LevelStarts ls{};
   int lmin = 0;  // smallest x level
   // 3D only
-  const PlaneGrid* planes = nullptr;
+  const PlaneArray* planes = nullptr;
   int S2 = 0;  // values of one plane and component
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
