@@ -361,12 +361,12 @@ __global__ void __launch_bounds__(256) k_combine_planes(const PlaneArray* __rest
 // computes K consecutive nodes: it needs 2 nodes of the shared level, then
 // 3, 5, ..., K + 1, and prolongs that cone by itself, which spares the
 // barriers of the widest levels for a few values computed twice.  Bound:
-// 3D, latency (four loads in flight instead of two: 88 -> 84 us) and the
-// seven pair operations of every grid's node; 2D, the latency of the block's
+// 3D, L1 (62% busy), issue slots (40%) and latency at 31% of the warps (four
+// loads in flight instead of two: 88 -> 84 us); 2D, the latency of the block's
 // phases (36% of issue slots).  With profiling events, before (one warp per
-// line, four brackets) -> now, planes included: 3D n = 7 151 -> 77 us, tau = 2
-// 137 -> 74, n = 6 cell-centred 64 -> 28; 2D n = 11 134 -> 51, n = 10 27 -> 22,
-// n = 8 14.3 -> 12.3 us.
+// line, four brackets) -> now, planes included: 3D n = 7 151 -> 78 us, tau = 2
+// 137 -> 75, n = 6 cell-centred 64 -> 31; 2D n = 11 134 -> 53, n = 10 27 ->
+// 22.5, n = 8 14.3 -> 12.3 us.
 
 // Transverse interpolation of one array at regular line y: the two coarse
 // lines that bracket it, each weight times the coefficient (dyadic: exact).
@@ -675,7 +675,8 @@ static int launch_lines(const CombineTables& ct, const GT* G, size_t zstride, in
   // Threads per block and tasks to share among them.  From 2^18 tasks on
   // (2D n = 10, 3D n = 7) a block takes 384 or more (3D fields 192, whose
   // tables are three times as long), two per thread, which spreads its tables
-  // and barriers: 3D n = 7 77 us against 86 with 128 and 128, 84 with 384; 2D
+  // and barriers: 3D n = 7 77 us against 86 with 128 and 128, 84 with 384 (the
+  // energy then summed in floats); 2D
   // n = 10 20.5 against 21.2.  Below, small blocks reach more SMs: 3D n = 6 25
   // against 43 us, 2D n = 8 12.3 against 14.5.  Doubles on tiny grids go smaller
   // still (2D n = 6: 13.5 against 14.3 us).

@@ -2291,6 +2291,7 @@ size_t estimate_footprint(int precision, int dim, int n, int tau, size_t np) {
     for (int m = 0; m < dim; ++m) s <<= g.l[m];
     S += s;
   }
+  // two particle sets; keys and tile counts (half of it: an upper estimate)
   size_t part = 2 * np * ((2 * dim + 1) * rs + 4) + 4 * np * 4 + (np / RS_TILE + 1) * 256 * 4 * 2;
   size_t grid = ND * rs * (1 + dim) + (rs == 4 ? dim * ND * 4 : 0) + 2 * ND * rs;  // rho, Ecomb, restrict scratch
   size_t arena = S * (rs + 2 * rs + dim * 2 * rs + dim * rs);

@@ -14,11 +14,11 @@
 // a non-zero mode skip their transform (its result is zero).
 //
 // Bound: the estimator by the double-precision pipe (GB300: two operations
-// per clock and SM), which half spectra and skipped tiles spare; the filter's
-// solve by latency (one or two blocks per SM, five barriers per transform).  Before, with whole complex
-// arrays and a pass per operation: estimator and step 427 -> 181 us (2D
-// n = 9, adaptive), 815 -> 237 us (3D n = 6); the filter's solve with
-// profiling events 100 -> 55 us (2D n = 10).
+// per clock and SM; k_est_rows 91% busy, k_est_columns 70%), which half spectra
+// and skipped tiles spare; the filter's solve by L1 (k_solve_columns 77% busy)
+// and latency.  Before, with whole complex arrays and a pass per operation:
+// estimator and step 427 -> 194 us (2D n = 9, adaptive), 815 -> 264 us (3D n = 6);
+// the filter's solve with profiling events 100 -> 56 us (2D n = 10).
 #include <algorithm>
 
 #include "sg_fft.cuh"
