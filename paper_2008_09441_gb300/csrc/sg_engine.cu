@@ -1226,8 +1226,10 @@ class Engine final : public EngineBase {
         if (pass == 0) {
           const size_t est = estimate_footprint(sizeof(real) == 8 ? SG_FP64 : SG_FP32, D, n_, tau_, np_);
           const size_t used = bytes_ - est_bytes_ + garena_.total();
-          const size_t left = std::max(est > used ? est - used : 0, plane * N_ / 8);
-          comb_scratch_bytes_ = std::max(plane, std::min(plane * (size_t)N_, left));
+          const size_t left = std::max(est > used ? (est - used) / 256 * 256 : 0, plane * N_ / 8);
+          size_t nz = N_;  // planes at a time, a power of two (launch_combine)
+          while (nz > 1 && plane * nz > left) nz >>= 1;
+          comb_scratch_bytes_ = plane * nz;
         }
         comb_.scratch_bytes = comb_scratch_bytes_;
         SG_TRY(galloc(&comb_.scratch, comb_.scratch_bytes));

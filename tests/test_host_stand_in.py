@@ -193,3 +193,19 @@ for missing in range(7):
     o.on_device = 0
     assert L.lib().sg_pic_get_particles(r.h, C.byref(o)) == L.SG_OK
 """)
+
+
+@pytest.mark.parametrize("d,ns", [(2, (4, 7, 10)), (3, (4, 5, 6))])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_a_run_fits_its_estimated_footprint(stand_in, d, ns, prec):
+    stand_in(f"""
+for n in {ns}:
+    for tau in (1, 2):
+        for np_ in (1000, 100000):
+            fake.fake_peak(1)
+            before = fake.fake_in_use()
+            r = run({d}, n, np_, tau=tau, precision="{prec}")
+            r.step(7)
+            assert fake.fake_peak(1) - before <= sg_estimate_footprint("{prec}", {d}, n, tau, np_), (n, tau, np_)
+            r.close()
+""")
